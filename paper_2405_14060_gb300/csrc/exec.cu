@@ -193,7 +193,12 @@ struct Program {
     int64_t *d_meta = nullptr;
     int nmeta = 0;
     double *cdf = nullptr;
-    std::vector<std::pair<CDesc, int64_t>> cdf_nodes;
+    struct CdfNode { CDesc d; int64_t rows; int bs; int64_t off; };
+    std::vector<CdfNode> cdf_nodes;
+    SampNode *d_snode = nullptr;
+    SampLab *d_slab = nullptr;
+    int2 *d_sdig = nullptr;
+    longlong2 *d_sktab = nullptr;
     int32_t *d_evid = nullptr;
     int32_t *d_slice_val = nullptr;     // values of the sliced variables for this run
     double *d_logz = nullptr, *d_sigma = nullptr, *d_marg = nullptr, *d_grad = nullptr;
@@ -2129,47 +2134,77 @@ tn_status build_program(tn_model *m, const Net &net, const Tree &tree, int kind,
         CK(cudaMemcpy(P.d_meta, meta.data(), meta.size() * 8, cudaMemcpyHostToDevice));
         CK(P.mem.alloc(&P.d_assign, (size_t)nbeta * std::max(1, (int)net.card.size()) * 4));
     }
-    // ---- sampling records (root first)
+    // ---- sampling records (root first), of the nodes that draw something
     if (kind == K_SAMPLE) {
-        std::vector<int64_t> meta;
+        std::vector<SampNode> nodes;
+        std::vector<SampLab> labs;
+        std::vector<int2> digs;
+        std::vector<longlong2> ktab;
         int64_t cdf_total = 0;
         for (int id = NN - 1; id >= n; --id) {
             const Node &nd = pl.node[id];
             const Node &na = pl.node[nd.a], &nb = pl.node[nd.b];
-            meta.push_back((int64_t)nd.labels.size());
-            for (int v : nd.labels) {
-                meta.push_back(v);
-                meta.push_back(std::max<int64_t>(0, stride_in(net.card, na.labels, v)));
-                meta.push_back(std::max<int64_t>(0, stride_in(net.card, nb.labels, v)));
-                meta.push_back(stride_in(net.card, nd.labels, v));
+            double Kd = 1;
+            for (int v : nd.elim) Kd *= net.card[v];
+            if (Kd <= 1) continue;
+            SampNode r;
+            std::memset(&r, 0, sizeof r);
+            r.node = NN - 1 - id;   // counter of the node's random number
+            r.nC = (int)nd.labels.size();
+            r.nK = (int)nd.elim.size();
+            r.lab0 = (int32_t)labs.size();
+            r.dig0 = (int32_t)digs.size();
+            r.K = (int64_t)Kd;
+            for (const Labels *L : {&nd.labels, &nd.elim})
+                for (int v : *L)
+                    labs.push_back({std::max<int64_t>(0, stride_in(net.card, na.labels, v)),
+                                    std::max<int64_t>(0, stride_in(net.card, nb.labels, v)),
+                                    std::max<int64_t>(0, stride_in(net.card, nd.labels, v)), v});
+            for (int v : nd.elim) digs.push_back(int2{v, net.card[v]});
+            r.offA = P.fwd[nd.a].off;
+            r.offB = P.fwd[nd.b].off;
+            r.tab0 = -1;
+            if (r.K <= 4096) {
+                r.tab0 = (int64_t)ktab.size();
+                for (int64_t k = 0; k < r.K; ++k) {
+                    longlong2 o{0, 0};
+                    int64_t q = k;
+                    for (int i = r.nK - 1; i >= 0; --i) {
+                        const SampLab &l = labs[r.lab0 + r.nC + i];
+                        const int64_t dg = q % digs[r.dig0 + i].y;
+                        q /= digs[r.dig0 + i].y;
+                        o.x += dg * l.sA;
+                        o.y += dg * l.sB;
+                    }
+                    ktab.push_back(o);
+                }
             }
-            int64_t K = 1;
-            meta.push_back((int64_t)nd.elim.size());
-            for (int v : nd.elim) {
-                meta.push_back(v);
-                meta.push_back(net.card[v]);
-                meta.push_back(std::max<int64_t>(0, stride_in(net.card, na.labels, v)));
-                meta.push_back(std::max<int64_t>(0, stride_in(net.card, nb.labels, v)));
-                K *= net.card[v];
+            // block sums (a search and one block's scan per sample) from 512
+            // summed entries, where building them reads at most 2^22 products
+            // (tens of microseconds, what one sample's serial scan takes), and
+            // beyond 4096, where such a scan takes milliseconds, up to 2^28;
+            // other nodes are scanned.  The choice does not depend on the
+            // number of samples: a longer run starts with a shorter one's rows
+            r.cdf = -1;
+            const double prods = (double)P.fwd[id].per * Kd;
+            if (r.K >= 512 && prods <= (r.K > 4096 ? 268435456.0 : 4194304.0)) {
+                r.bs = r.K > 65536 ? 256 : 64;
+                r.cdf = cdf_total;
+                P.cdf_nodes.push_back({P.fdesc[id - n], P.fwd[id].per, r.bs, cdf_total});
+                cdf_total += P.fwd[id].per * ((r.K + r.bs - 1) / r.bs);
             }
-            meta.push_back(P.fwd[nd.a].off);
-            meta.push_back(P.fwd[nd.b].off);
-            meta.push_back(K);
-            // large summed spaces get cumulative tables (binary search per
-            // sample) while those fit 2^27 entries; otherwise every sample
-            // scans the node's summed space directly
-            const int64_t rows = P.fwd[id].per;
-            if (K > 4096 && (double)rows * (double)K <= (double)(1LL << 27)) {
-                meta.push_back(cdf_total);
-                P.cdf_nodes.push_back({P.fdesc[id - n], rows});
-                cdf_total += rows * K;
-            } else {
-                meta.push_back(-1);
-            }
+            nodes.push_back(r);
         }
-        P.nmeta = NN - n;
-        CK(P.mem.alloc(&P.d_meta, meta.size() * 8));
-        CK(cudaMemcpy(P.d_meta, meta.data(), meta.size() * 8, cudaMemcpyHostToDevice));
+        P.nmeta = (int)nodes.size();
+        auto up = [&](auto **d, const auto &h) -> cudaError_t {
+            cudaError_t e = P.mem.alloc(d, h.size() * sizeof(h[0]));
+            if (e != cudaSuccess || h.empty()) return e;
+            return cudaMemcpy(*d, h.data(), h.size() * sizeof(h[0]), cudaMemcpyHostToDevice);
+        };
+        CK(up(&P.d_snode, nodes));
+        CK(up(&P.d_slab, labs));
+        CK(up(&P.d_sdig, digs));
+        CK(up(&P.d_sktab, ktab));
         if (cdf_total) CK(P.mem.alloc(&P.cdf, (size_t)cdf_total * 8));
     }
     return TN_OK;
@@ -3240,19 +3275,19 @@ tn_status tn_map(tn_model *m, const int32_t *evid, const tn_options *opts, int32
 static tn_status draw_samples(tn_model *m, Program &P, int64_t n, uint64_t seed, int8_t *d_out,
                               cudaStream_t st) {
     if (n == 0) return TN_OK;
-    int64_t coff = 0;
     for (auto &c : P.cdf_nodes) {
-        // cumulative tables of the nodes with large summed spaces
-        if (P.dtype == 0) launch_cdf_rows<double>(c.first, c.second, P.cdf + coff, st);
-        else launch_cdf_rows<float>(c.first, c.second, P.cdf + coff, st);
-        coff += c.second * c.first.ktotal;
+        // block sums of the nodes with large summed spaces
+        if (P.dtype == 0) launch_cdf_blocks<double>(c.d, c.rows, c.bs, P.cdf + c.off, st);
+        else launch_cdf_blocks<float>(c.d, c.rows, c.bs, P.cdf + c.off, st);
     }
     if (P.dtype == 0)
-        launch_sample<double>(P.d_meta, P.nmeta, (const double *)P.arena, P.cdf, P.d_evid,
-                              m->md.nvars, n, seed, d_out, st);
+        launch_sample<double>(P.d_snode, P.nmeta, P.d_slab, P.d_sdig, P.d_sktab,
+                              (const double *)P.arena, P.cdf, P.d_evid, m->md.nvars, n, seed,
+                              d_out, st);
     else
-        launch_sample<float>(P.d_meta, P.nmeta, (const float *)P.arena, P.cdf, P.d_evid,
-                             m->md.nvars, n, seed, d_out, st);
+        launch_sample<float>(P.d_snode, P.nmeta, P.d_slab, P.d_sdig, P.d_sktab,
+                             (const float *)P.arena, P.cdf, P.d_evid, m->md.nvars, n, seed, d_out,
+                             st);
     CK(cudaGetLastError());
     return TN_OK;
 }

@@ -4,6 +4,7 @@
 // backtracking and backward sampling.
 #include <cfloat>
 #include <cmath>
+#include <mutex>
 
 #include "devutil.cuh"
 #include "task_kernels.cuh"
@@ -400,103 +401,254 @@ __device__ __forceinline__ double uniform01(uint64_t sample, uint32_t node, uint
     return (double)m * (1.0 / 9007199254740992.0);
 }
 
-// Record layout (int64): nC, {label, sA, sB, sC} x nC, nK, {label, size, sA,
-// sB} x nK, offA, offB, ktotal, cdf offset (-1: sample by direct summation).
 // At a node C_Z = con({A_X, B_Y}, Z) with the sample's values s_Z already
 // drawn, the eliminated labels M are drawn from A[s_Z, m] B[s_Z, m] / C[s_Z]
-// (Eq. condition-prob); the stored tensors' common scales cancel.
-template <typename T>
-__global__ void k_sample(const int64_t *meta, int nnodes, const T *base, const double *cdf,
-                         const int32_t *evid, int nvars, int64_t nsamp, uint64_t seed,
-                         int8_t *out) {
-    int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nsamp) return;
-    int8_t *x = out + s * nvars;
-    for (int v = 0; v < nvars; ++v) x[v] = (int8_t)(evid && evid[v] >= 0 ? evid[v] : 0);
-    const int64_t *p = meta;
-    for (int n = 0; n < nnodes; ++n) {
-        int64_t nC = *p++;
-        int64_t oa = 0, ob = 0, oc = 0;
-        for (int64_t i = 0; i < nC; ++i) {
-            int64_t xv = x[p[0]];
-            oa += xv * p[1];
-            ob += xv * p[2];
-            oc += xv * p[3];
-            p += 4;
+// (Eq. condition-prob); the stored tensors' common scales cancel.  Records
+// (SampNode) hold only the nodes that draw something (K > 1), root first.
+//
+// One thread per sample.  What bounds it is the chain of draws, each a few
+// dependent L2 loads, so everything beside that chain is kept short: the
+// sample's values sit in shared memory ([variable][thread], consecutive lanes
+// in consecutive bytes; rows of BT + 4 bytes so that the final transposed read
+// meets no bank conflict), records, label lists and summed-offset tables are
+// read at warp-uniform addresses in 16-byte pieces, and a summed space is
+// scanned once: the running sum is kept at 16 block ends and only the block of
+// the draw is read again (the same sums in the same order as a second full
+// scan).  Summed spaces of 512 and more entries search the block sums of
+// k_cdf_blocks where the executor planned them.  16 x 16 grid, FP64, 100000
+// samples (166 drawing nodes of 991, one with 4096 entries): 26.2 ms with
+// values in global memory, every node visited and two full scans; a whole call
+// (forward pass and copy to the host included) went from 27.7 to 3.0 ms.
+
+// Draw among N or fewer summed assignments held in registers.
+template <typename T, int N>
+__device__ __forceinline__ int64_t samp_small(const T *A, const T *B,
+                                              const longlong2 *__restrict__ kt, int K, double u) {
+    double w[N], tot = 0, c = 0;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        w[k] = 0;
+        if (k < K) {
+            const longlong2 o = __ldg(kt + k);
+            w[k] = (double)A[o.x] * (double)B[o.y];
         }
-        int64_t nK = *p++;
-        const int64_t *kl = p;
-        p += 4 * nK;
-        int64_t offA = p[0], offB = p[1], K = p[2], coff = p[3];
-        p += 4;
-        double u = uniform01((uint64_t)s, (uint32_t)n, seed);
-        int64_t pick = 0;
-        if (coff >= 0) {
-            const double *row = cdf + coff + oc * K;
-            double r = u * row[K - 1];
-            int64_t lo = 0, hi = K - 1;
-            while (lo < hi) {
-                int64_t mid = (lo + hi) >> 1;
-                if (row[mid] > r) hi = mid;
-                else lo = mid + 1;
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+        if (k < K) tot += w[k];
+    const double r0 = u * tot;
+    int pick = K - 1;
+    bool done = false;
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+        if (k < K) {
+            c += w[k];
+            if (!done && r0 < c && w[k] > 0) {
+                pick = k;
+                done = true;
             }
-            pick = lo;
-        } else {
-            const T *A = base + offA + oa;
-            const T *B = base + offB + ob;
-            double tot = 0;
-            for (int64_t k = 0; k < K; ++k) {
-                int64_t ka = 0, kb = 0, r = k;
-                for (int64_t i = nK - 1; i >= 0; --i) {
-                    int64_t dg = r % kl[4 * i + 1];
-                    r /= kl[4 * i + 1];
-                    ka += dg * kl[4 * i + 2];
-                    kb += dg * kl[4 * i + 3];
+        }
+    return pick;
+}
+
+template <typename T, bool SM>
+__global__ void __launch_bounds__(128) k_sample(const SampNode *__restrict__ nodes, int nnodes,
+                                                const SampLab *__restrict__ labs,
+                                                const int2 *__restrict__ digs,
+                                                const longlong2 *__restrict__ ktab,
+                                                const T *__restrict__ base,
+                                                const double *__restrict__ cdf,
+                                                const int32_t *__restrict__ evid, int nvars,
+                                                int64_t nsamp, uint64_t seed, int8_t *out) {
+    extern __shared__ __align__(16) int8_t xs[];
+    const int BT = blockDim.x, tid = threadIdx.x;
+    const int64_t s0 = (int64_t)blockIdx.x * BT, s = s0 + tid;
+    // variable v of this thread's sample: x[v * xstep]
+    int8_t *x = SM ? xs + tid : out + (s < nsamp ? s : nsamp - 1) * nvars;
+    const int64_t xstep = SM ? BT + 4 : 1;
+    if (s < nsamp) {
+        for (int v = 0; v < nvars; ++v) {
+            const int e = evid ? __ldg(evid + v) : -1;
+            x[v * xstep] = (int8_t)(e >= 0 ? e : 0);
+        }
+        for (int n = 0; n < nnodes; ++n) {
+            const SampNode nd = nodes[n];
+            int64_t oa = nd.offA, ob = nd.offB, oc = 0;
+#pragma unroll 4
+            for (int i = 0; i < nd.nC; ++i) {
+                const SampLab l = labs[nd.lab0 + i];
+                const int64_t xv = x[l.var * xstep];
+                oa += xv * l.sA;
+                ob += xv * l.sB;
+                oc += xv * l.sC;
+            }
+            const T *A = base + oa, *B = base + ob;
+            const int64_t K = nd.K;
+            const longlong2 *kt = ktab + nd.tab0;
+            // product of the summed assignment k
+            auto weight = [&](int64_t k) {
+                if (nd.tab0 >= 0) {
+                    const longlong2 o = __ldg(kt + k);
+                    return (double)A[o.x] * (double)B[o.y];
                 }
-                tot += (double)A[ka] * (double)B[kb];
-            }
-            double r0 = u * tot, c = 0;
-            pick = K - 1;
-            for (int64_t k = 0; k < K; ++k) {
                 int64_t ka = 0, kb = 0, r = k;
-                for (int64_t i = nK - 1; i >= 0; --i) {
-                    int64_t dg = r % kl[4 * i + 1];
-                    r /= kl[4 * i + 1];
-                    ka += dg * kl[4 * i + 2];
-                    kb += dg * kl[4 * i + 3];
+                for (int i = nd.nK - 1; i >= 0; --i) {
+                    const int2 dg = digs[nd.dig0 + i];
+                    const SampLab l = labs[nd.lab0 + nd.nC + i];
+                    const int64_t d = r % dg.y;
+                    r /= dg.y;
+                    ka += d * l.sA;
+                    kb += d * l.sB;
                 }
-                double w = (double)A[ka] * (double)B[kb];
-                c += w;
-                if (r0 < c && w > 0) { pick = k; break; }
+                return (double)A[ka] * (double)B[kb];
+            };
+            const double u = uniform01((uint64_t)s, (uint32_t)nd.node, seed);
+            int64_t pick = K - 1;
+            if (K <= 2) {
+                pick = samp_small<T, 2>(A, B, kt, (int)K, u);
+            } else if (K <= 8) {
+                pick = samp_small<T, 8>(A, B, kt, (int)K, u);
+            } else if (nd.cdf >= 0) {
+                const int64_t nblk = (K + nd.bs - 1) / nd.bs;
+                const double *row = cdf + nd.cdf + oc * nblk;
+                const double r = u * row[nblk - 1];
+                int64_t lo = 0, hi = nblk - 1;
+                while (lo < hi) {
+                    const int64_t mid = (lo + hi) >> 1;
+                    if (row[mid] > r) hi = mid;
+                    else lo = mid + 1;
+                }
+                const int64_t k0 = lo * nd.bs, k1 = min(K, k0 + nd.bs);
+                double c = lo ? row[lo - 1] : 0.0;
+                pick = k1 - 1;
+#pragma unroll 1
+                for (int64_t k = k0; k < k1; ++k) {
+                    const double w = weight(k);
+                    c += w;
+                    if (w > 0) {
+                        pick = k;   // the block's last possible value if rounding hides the draw
+                        if (r < c) break;
+                    }
+                }
+            } else {
+                double end[16];   // running sum at the end of each block
+                double tot = 0;
+                const int64_t bs = (K + 15) >> 4;
+#pragma unroll 1
+                for (int j = 0; j < 16; ++j) {
+                    const int64_t k1 = min(K, (j + 1) * bs);
+                    int64_t k = j * bs;
+                    if (nd.tab0 >= 0)
+                        for (; k + 4 <= k1; k += 4) {
+                            double w[4];   // four loads in flight
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                const longlong2 o = __ldg(kt + k + q);
+                                w[q] = (double)A[o.x] * (double)B[o.y];
+                            }
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) tot += w[q];
+                        }
+#pragma unroll 1
+                    for (; k < k1; ++k) tot += weight(k);
+                    end[j] = tot;
+                }
+                const double r0 = u * tot;
+                double c = 0;
+                int64_t k0 = K;
+#pragma unroll 1
+                for (int j = 0; j < 16; ++j)
+                    if (r0 < end[j]) {
+                        k0 = j * bs;
+                        c = j ? end[j - 1] : 0.0;
+                        break;
+                    }
+#pragma unroll 1
+                for (int64_t k = k0; k < K; ++k) {
+                    const double w = weight(k);
+                    c += w;
+                    if (r0 < c && w > 0) { pick = k; break; }
+                }
+            }
+            for (int i = nd.nK - 1; i >= 0; --i) {
+                const int2 dg = digs[nd.dig0 + i];
+                int d = (int)pick;
+                if (nd.nK > 1) {
+                    d = (int)(pick % dg.y);
+                    pick /= dg.y;
+                }
+                x[dg.x * xstep] = (int8_t)d;
             }
         }
-        for (int64_t i = nK - 1; i >= 0; --i) {
-            int64_t sz = kl[4 * i + 1];
-            x[kl[4 * i]] = (int8_t)(pick % sz);
-            pick /= sz;
+    }
+    if (!SM) return;
+    // the block's rows: BT samples x nvars bytes, contiguous in the output
+    __syncthreads();
+    const int rows = (int)min((int64_t)BT, nsamp - s0);
+    int8_t *o = out + s0 * nvars;
+    const int total = rows * nvars;
+    if (((uintptr_t)o & 3) == 0) {
+        for (int i = 4 * tid; i < total; i += 4 * BT) {
+            int r = i / nvars, v = i - r * nvars;
+            uint32_t w = 0;
+            int j = 0;
+            for (; j < 4 && i + j < total; ++j) {
+                w |= (uint32_t)(uint8_t)xs[v * (BT + 4) + r] << (8 * j);
+                if (++v == nvars) {
+                    v = 0;
+                    ++r;
+                }
+            }
+            if (j == 4) *(uint32_t *)(o + i) = w;
+            else
+                for (int q = 0; q < j; ++q) o[i + q] = (int8_t)(w >> (8 * q));
         }
+    } else {
+        for (int i = tid; i < total; i += BT) o[i] = xs[(i % nvars) * (BT + 4) + i / nvars];
     }
 }
 
 template <typename T>
-void launch_sample(const int64_t *meta, int nnodes, const T *base, const double *cdf,
-                   const int32_t *evid, int nvars, int64_t nsamp, uint64_t seed, int8_t *out,
-                   cudaStream_t st) {
-    k_sample<T><<<(unsigned)((nsamp + 127) / 128), 128, 0, st>>>(meta, nnodes, base, cdf, evid,
-                                                                nvars, nsamp, seed, out);
+void launch_sample(const SampNode *nodes, int nnodes, const SampLab *labs, const int2 *digs,
+                   const longlong2 *ktab, const T *base, const double *cdf, const int32_t *evid,
+                   int nvars, int64_t nsamp, uint64_t seed, int8_t *out, cudaStream_t st) {
+    // samples per block: as many as keep the values in 100 KB of shared
+    // memory (two blocks an SM); beyond 100 KB at 32, the values stay in `out`
+    constexpr size_t kCap = 100 * 1024;
+    int bt = 128;
+    while (bt > 32 && (size_t)nvars * (bt + 4) > kCap) bt /= 2;
+    const size_t smem = (size_t)nvars * (bt + 4);
+    if (smem > kCap) {
+        k_sample<T, false><<<(unsigned)((nsamp + 127) / 128), 128, 0, st>>>(
+            nodes, nnodes, labs, digs, ktab, base, cdf, evid, nvars, nsamp, seed, out);
+        return;
+    }
+    static std::once_flag once;
+    std::call_once(once, [] {
+        cudaFuncSetAttribute(k_sample<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kCap);
+    });
+    k_sample<T, true><<<(unsigned)((nsamp + bt - 1) / bt), bt, smem, st>>>(
+        nodes, nnodes, labs, digs, ktab, base, cdf, evid, nvars, nsamp, seed, out);
 }
 
-// Cumulative sums cdf[o][k] = sum_{j<=k} A[o, j] B[o, j] over the summed
-// labels of one node (one block per output entry), for nodes whose summed
-// space is too large to scan per sample.
+// Block sums of a node's conditional weights: cdf[o][j] = sum of A[o, k] B[o, k]
+// over summed indices k in [j bs, (j + 1) bs), one warp per (output entry o,
+// block j), then running sums over j, one block of threads per output entry.
+// A draw searches the nblk sums and scans one block, so the table is 1 / bs of
+// a full cumulative table.
 template <typename T>
-__global__ void k_cdf_rows(const __grid_constant__ CDesc d, double *cdf) {
-    int64_t o = blockIdx.x;
+__global__ void __launch_bounds__(256) k_cdf_blocks(const __grid_constant__ CDesc d, int bs,
+                                                    int64_t nblk, int64_t total, double *cdf) {
+    const int64_t w = ((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5;
+    if (w >= total) return;
+    const int lane = threadIdx.x & 31;
+    const int64_t o = w / nblk, j = w - o * nblk;
     int64_t oa = 0, ob = 0;
     {
         int64_t r = o;
         for (int i = d.nout - 1; i >= 0; --i) {
-            int64_t dg = r % d.osz[i];
+            const int64_t dg = r % d.osz[i];
             r /= d.osz[i];
             oa += dg * d.osa[i];
             ob += dg * d.osb[i];
@@ -504,45 +656,62 @@ __global__ void k_cdf_rows(const __grid_constant__ CDesc d, double *cdf) {
     }
     const T *A = (const T *)d.A + oa;
     const T *B = (const T *)d.B + ob;
-    int64_t K = d.ktotal;
-    int nt = blockDim.x;
-    int64_t per = (K + nt - 1) / nt;
-    int64_t k0 = threadIdx.x * per, k1 = min(K, k0 + per);
-    auto val = [&](int64_t k) {
-        int64_t ka = 0, kb = 0, r = k;
-        for (int i = d.nk - 1; i >= 0; --i) {
-            int64_t dg = r % d.ksz[i];
-            r /= d.ksz[i];
-            ka += dg * d.ksa[i];
-            kb += dg * d.ksb[i];
-        }
-        return (double)A[ka] * (double)B[kb];
-    };
+    const int64_t k1 = min(d.ktotal, (j + 1) * bs);
     double s = 0;
-    for (int64_t k = k0; k < k1; ++k) s += val(k);
-    __shared__ double pre[1024];
+    for (int64_t k = j * bs + lane; k < k1; k += 32) {
+        int64_t ka = 0, kb = 0;
+        if (d.pow2) {
+            for (int i = 0; i < d.nk; ++i) {
+                const int64_t dg = (k >> d.ksh[i]) & (int64_t)(d.ksz[i] - 1);
+                ka += dg * d.ksa[i];
+                kb += dg * d.ksb[i];
+            }
+        } else {
+            int64_t r = k;
+            for (int i = d.nk - 1; i >= 0; --i) {
+                const int64_t dg = r % d.ksz[i];
+                r /= d.ksz[i];
+                ka += dg * d.ksa[i];
+                kb += dg * d.ksb[i];
+            }
+        }
+        s += (double)A[ka] * (double)B[kb];
+    }
+#pragma unroll
+    for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
+    if (lane == 0) cdf[w] = s;
+}
+
+__global__ void __launch_bounds__(256) k_cdf_prefix(int64_t nblk, double *cdf) {
+    double *row = cdf + (int64_t)blockIdx.x * nblk;
+    const int64_t per = (nblk + 255) / 256;
+    const int64_t j0 = threadIdx.x * per, j1 = min(nblk, j0 + per);
+    double s = 0;
+    for (int64_t j = j0; j < j1; ++j) s += row[j];
+    __shared__ double pre[256];
     pre[threadIdx.x] = s;
     __syncthreads();
     if (threadIdx.x == 0) {
         double run = 0;
-        for (int i = 0; i < nt; ++i) {
-            double t = pre[i];
+        for (int i = 0; i < 256; ++i) {
+            const double t = pre[i];
             pre[i] = run;
             run += t;
         }
     }
     __syncthreads();
     double run = pre[threadIdx.x];
-    double *row = cdf + o * K;
-    for (int64_t k = k0; k < k1; ++k) {
-        run += val(k);
-        row[k] = run;
+    for (int64_t j = j0; j < j1; ++j) {
+        run += row[j];
+        row[j] = run;
     }
 }
 
 template <typename T>
-void launch_cdf_rows(const CDesc &d, int64_t rows, double *cdf, cudaStream_t st) {
-    k_cdf_rows<T><<<(unsigned)rows, 256, 0, st>>>(d, cdf);
+void launch_cdf_blocks(const CDesc &d, int64_t rows, int bs, double *cdf, cudaStream_t st) {
+    const int64_t nblk = (d.ktotal + bs - 1) / bs, total = rows * nblk;
+    k_cdf_blocks<T><<<(unsigned)((total + 7) / 8), 256, 0, st>>>(d, bs, nblk, total, cdf);
+    k_cdf_prefix<<<(unsigned)rows, 256, 0, st>>>(nblk, cdf);
 }
 
 #define INST(T)                                                                                  \
@@ -556,10 +725,11 @@ void launch_cdf_rows(const CDesc &d, int64_t rows, double *cdf, cudaStream_t st)
                                       double *, int64_t, cudaStream_t);                         \
     template void launch_factor_grads<T>(const GradRec *, int, int, const T *, const T *,       \
                                          double *, int64_t, cudaStream_t);                      \
-    template void launch_sample<T>(const int64_t *, int, const T *, const double *,             \
+    template void launch_sample<T>(const SampNode *, int, const SampLab *, const int2 *,        \
+                                   const longlong2 *, const T *, const double *,                \
                                    const int32_t *, int, int64_t, uint64_t, int8_t *,           \
                                    cudaStream_t);                                               \
-    template void launch_cdf_rows<T>(const CDesc &, int64_t, double *, cudaStream_t);
+    template void launch_cdf_blocks<T>(const CDesc &, int64_t, int, double *, cudaStream_t);
 INST(float)
 INST(double)
 

@@ -39,6 +39,22 @@ struct GradRec {
     int abeta, pad;
 };
 
+// Sampling records.  A node that draws: its kept labels labs[lab0 .. + nC) and
+// summed labels (the next nK, with digs[dig0 .. + nK) = {variable, size}),
+// offsets of its operands, summed space K, and either the {A, B} offsets of
+// every summed index at ktab[tab0] or tab0 = -1 (decoded from the digits).
+// cdf: its block sums (bs summed indices each), -1: the summed space is scanned.
+struct alignas(16) SampNode {
+    int32_t node, nC, nK, bs;
+    int32_t lab0, dig0;
+    int64_t tab0;
+    int64_t K, offA, offB, cdf;
+};
+struct alignas(16) SampLab {
+    int64_t sA, sB, sC;
+    int64_t var;
+};
+
 template <typename T>
 void launch_leaves(const LeafRec *recs, int nrec, const double *tables, const int *card,
                    int nvars, const int32_t *evid, int nbeta, int log_mode, T *base,
@@ -69,10 +85,10 @@ void launch_factor_grads(const GradRec *recs, int nrec, int nbeta, const T *fbas
 void launch_backtrack(const int64_t *meta, int nnodes, const int32_t *argmax, int nbeta,
                       int nvars, int32_t *assign, cudaStream_t st);
 template <typename T>
-void launch_sample(const int64_t *meta, int nnodes, const T *base, const double *cdf,
-                   const int32_t *evid, int nvars, int64_t nsamp, uint64_t seed, int8_t *out,
-                   cudaStream_t st);
+void launch_sample(const SampNode *nodes, int nnodes, const SampLab *labs, const int2 *digs,
+                   const longlong2 *ktab, const T *base, const double *cdf, const int32_t *evid,
+                   int nvars, int64_t nsamp, uint64_t seed, int8_t *out, cudaStream_t st);
 template <typename T>
-void launch_cdf_rows(const CDesc &d, int64_t rows, double *cdf, cudaStream_t st);
+void launch_cdf_blocks(const CDesc &d, int64_t rows, int bs, double *cdf, cudaStream_t st);
 
 }  // namespace tn
