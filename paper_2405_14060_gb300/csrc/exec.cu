@@ -190,11 +190,12 @@ struct Program {
     MargRec *d_margrec = nullptr;
     GradRec *d_gradrec = nullptr;
     int ngrad = 0;
-    int64_t *d_meta = nullptr;
-    int nmeta = 0;
+    BackHead back{};            // backtrack records
+    uint4 *d_back = nullptr;
     double *cdf = nullptr;
     struct CdfNode { CDesc d; int64_t rows; int bs; int64_t off; };
     std::vector<CdfNode> cdf_nodes;
+    int nsnode = 0;
     SampNode *d_snode = nullptr;
     SampLab *d_slab = nullptr;
     int2 *d_sdig = nullptr;
@@ -2110,28 +2111,56 @@ tn_status build_program(tn_model *m, const Net &net, const Tree &tree, int kind,
             CK(P.mem.alloc(&P.d_grad, (size_t)nbeta * std::max<int64_t>(1, P.grad_stride) * 8));
         }
     }
-    // ---- backtrack records (root first)
+    // ---- backtrack records: the nodes that maximise over something, by the
+    // number of such ancestors
     if (maxplus) {
-        std::vector<int64_t> meta;
+        std::vector<int> level(NN, 0);
+        std::vector<std::vector<int>> by;
         for (int id = NN - 1; id >= n; --id) {
             const Node &nd = pl.node[id];
-            meta.push_back((int64_t)nd.labels.size());
-            for (int v : nd.labels) {
-                meta.push_back(v);
-                meta.push_back(stride_in(net.card, nd.labels, v));
-            }
-            meta.push_back((int64_t)nd.elim.size());
-            for (int v : nd.elim) {
-                meta.push_back(v);
-                meta.push_back(net.card[v]);
-            }
-            meta.push_back(P.am_off[id]);
-            meta.push_back(P.fwd[id].per);
-            meta.push_back(P.fwd[id].beta ? 1 : 0);
+            double K = 1;
+            for (int v : nd.elim) K *= net.card[v];
+            level[nd.a] = level[nd.b] = level[id] + (K > 1 ? 1 : 0);
+            if (K <= 1) continue;
+            if ((int)by.size() <= level[id]) by.resize(level[id] + 1);
+            by[level[id]].push_back(id);
         }
-        P.nmeta = NN - n;
-        CK(P.mem.alloc(&P.d_meta, meta.size() * 8));
-        CK(cudaMemcpy(P.d_meta, meta.data(), meta.size() * 8, cudaMemcpyHostToDevice));
+        std::vector<BackNode> nodes;
+        std::vector<BackLab> labs;
+        std::vector<int2> digs;
+        std::vector<int32_t> lev{0};
+        for (auto &ids : by) {
+            for (int id : ids) {
+                const Node &nd = pl.node[id];
+                BackNode r;
+                r.aoff = P.am_off[id];
+                r.per = P.fwd[id].beta ? P.fwd[id].per : 0;
+                r.lab0 = (int32_t)labs.size();
+                r.nC = (int32_t)nd.labels.size();
+                r.dig0 = (int32_t)digs.size();
+                r.nK = (int32_t)nd.elim.size();
+                for (int v : nd.labels) labs.push_back({stride_in(net.card, nd.labels, v), v, 0});
+                for (int v : nd.elim) digs.push_back(int2{v, net.card[v]});
+                nodes.push_back(r);
+            }
+            lev.push_back((int32_t)nodes.size());
+        }
+        BackHead &h = P.back;
+        h.nlevels = (int32_t)by.size();
+        h.labs = (int32_t)(nodes.size() * sizeof(BackNode));
+        h.digs = h.labs + (int32_t)(labs.size() * sizeof(BackLab));
+        h.levels = h.digs + (int32_t)(digs.size() * sizeof(int2));
+        h.bytes = (h.levels + (int32_t)(lev.size() * 4) + 15) & ~15;
+        std::vector<unsigned char> blob((size_t)h.bytes, 0);
+        auto put = [&](int at, const void *p, size_t len) {
+            if (len) std::memcpy(blob.data() + at, p, len);
+        };
+        put(0, nodes.data(), nodes.size() * sizeof(BackNode));
+        put(h.labs, labs.data(), labs.size() * sizeof(BackLab));
+        put(h.digs, digs.data(), digs.size() * sizeof(int2));
+        put(h.levels, lev.data(), lev.size() * 4);
+        CK(P.mem.alloc(&P.d_back, blob.size()));
+        CK(cudaMemcpy(P.d_back, blob.data(), blob.size(), cudaMemcpyHostToDevice));
         CK(P.mem.alloc(&P.d_assign, (size_t)nbeta * std::max(1, (int)net.card.size()) * 4));
     }
     // ---- sampling records (root first), of the nodes that draw something
@@ -2195,7 +2224,7 @@ tn_status build_program(tn_model *m, const Net &net, const Tree &tree, int kind,
             }
             nodes.push_back(r);
         }
-        P.nmeta = (int)nodes.size();
+        P.nsnode = (int)nodes.size();
         auto up = [&](auto **d, const auto &h) -> cudaError_t {
             cudaError_t e = P.mem.alloc(d, h.size() * sizeof(h[0]));
             if (e != cudaSuccess || h.empty()) return e;
@@ -2389,7 +2418,7 @@ void enqueue_program(tn_model *m, Program &P, cudaStream_t st, Prof *pr = nullpt
     if (maxplus && P.kind == K_MAP) {
         cudaMemcpyAsync(P.d_assign, P.d_evid, (size_t)P.nbeta * m->md.nvars * 4,
                         cudaMemcpyDeviceToDevice, st);
-        launch_backtrack(P.d_meta, P.nmeta, P.am, P.nbeta, m->md.nvars, P.d_assign, st);
+        launch_backtrack(P.back, P.d_back, P.am, P.nbeta, m->md.nvars, P.d_assign, st);
         ++nl;
     }
     (void)NN;
@@ -3281,11 +3310,11 @@ static tn_status draw_samples(tn_model *m, Program &P, int64_t n, uint64_t seed,
         else launch_cdf_blocks<float>(c.d, c.rows, c.bs, P.cdf + c.off, st);
     }
     if (P.dtype == 0)
-        launch_sample<double>(P.d_snode, P.nmeta, P.d_slab, P.d_sdig, P.d_sktab,
+        launch_sample<double>(P.d_snode, P.nsnode, P.d_slab, P.d_sdig, P.d_sktab,
                               (const double *)P.arena, P.cdf, P.d_evid, m->md.nvars, n, seed,
                               d_out, st);
     else
-        launch_sample<float>(P.d_snode, P.nmeta, P.d_slab, P.d_sdig, P.d_sktab,
+        launch_sample<float>(P.d_snode, P.nsnode, P.d_slab, P.d_sdig, P.d_sktab,
                              (const float *)P.arena, P.cdf, P.d_evid, m->md.nvars, n, seed, d_out,
                              st);
     CK(cudaGetLastError());

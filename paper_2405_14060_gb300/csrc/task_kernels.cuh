@@ -39,6 +39,21 @@ struct GradRec {
     int abeta, pad;
 };
 
+// Backtrack records, one buffer: the maximising nodes level by level, their kept
+// labels, their maximised labels {variable, size}, and the first node of each
+// level (BackHead: byte offsets of the parts).
+struct BackNode {
+    int64_t aoff, per;   // argmax offset, entries per item (0: shared by all items)
+    int32_t lab0, nC, dig0, nK;
+};
+struct BackLab {
+    int64_t stride;
+    int32_t var, pad;
+};
+struct BackHead {
+    int32_t bytes, labs, digs, levels, nlevels;
+};
+
 // Sampling records.  A node that draws: its kept labels labs[lab0 .. + nC) and
 // summed labels (the next nK, with digs[dig0 .. + nK) = {variable, size}),
 // offsets of its operands, summed space K, and either the {A, B} offsets of
@@ -82,7 +97,7 @@ void launch_marginals(const MargRec *recs, int nvars, int nbeta, const T *fbase,
 template <typename T>
 void launch_factor_grads(const GradRec *recs, int nrec, int nbeta, const T *fbase,
                          const T *abase, double *grad, int64_t gstride, cudaStream_t st);
-void launch_backtrack(const int64_t *meta, int nnodes, const int32_t *argmax, int nbeta,
+void launch_backtrack(const BackHead &h, const uint4 *blob, const int32_t *argmax, int nbeta,
                       int nvars, int32_t *assign, cudaStream_t st);
 template <typename T>
 void launch_sample(const SampNode *nodes, int nnodes, const SampLab *labs, const int2 *digs,
