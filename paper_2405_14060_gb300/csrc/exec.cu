@@ -19,6 +19,7 @@
 #include <set>
 #include <string>
 #include <tuple>
+#include <unordered_map>
 #include <vector>
 
 #include "bgemm.cuh"
@@ -208,10 +209,9 @@ struct Program {
     std::vector<CDesc> fdesc;      // generic descriptor of every forward node
     std::vector<Step> fsteps, bsteps;
     std::vector<char> micro;                       // node runs inside a micro subtree
-    std::vector<MicroDesc> mf, mb;                 // forward / backward micro lists
-    std::vector<int32_t> mf_beg, mb_beg;           // per subtree start index
-    MicroDesc *d_mf = nullptr, *d_mb = nullptr;
-    int32_t *d_mf_beg = nullptr, *d_mb_beg = nullptr;
+    int mf_smem = 0, mb_smem = 0, mf_width = 1, mb_width = 1;   // micro passes
+    unsigned char *d_mf = nullptr, *d_mb = nullptr;
+    MicroSub *d_mf_sub = nullptr, *d_mb_sub = nullptr;
     char *wsX = nullptr, *wsY = nullptr, *wsD = nullptr;
     int gemm_type = 1;
     std::vector<LeafRec> leafrec;   // host copy (external sources patched per call)
@@ -1018,42 +1018,212 @@ static bool make_bgemm(const std::vector<int> &card, const Labels &lx, bool bx, 
     return d.tile >= 0;
 }
 
-static bool to_micro(const CDesc &d, const char *arena, int esz, const unsigned long long *mxb,
-                     const int32_t *amb, MicroDesc &m) {
-    std::memset(&m, 0, sizeof m);
-    if (d.nout > MICRO_D || d.nk > MICRO_D || d.nbeta > MICRO_BETA) return false;
-    if (d.nout_total * d.nbeta > MICRO_MAX || d.ktotal > (1LL << 30)) return false;
-    m.nout = d.nout;
-    m.nk = d.nk;
-    m.pow2 = d.pow2;
-    m.nbeta = d.nbeta;
-    m.nout_total = (int32_t)d.nout_total;
-    m.ktotal = (int32_t)d.ktotal;
-    m.offA = ((const char *)d.A - arena) / esz;
-    m.offB = ((const char *)d.B - arena) / esz;
-    m.offC = ((const char *)d.C - arena) / esz;
-    m.bsa = (int32_t)d.bsa;
-    m.bsb = (int32_t)d.bsb;
-    for (int i = 0; i < d.nout; ++i) {
-        m.osz[i] = d.osz[i];
-        m.osh[i] = d.osh[i];
-        m.osa[i] = (int32_t)d.osa[i];
-        m.osb[i] = (int32_t)d.osb[i];
+// Records of one pass over the micro subtrees (micro.cuh), built subtree by
+// subtree: nodes are added with their level, then the subtree is closed.
+struct MicroList {
+    std::vector<unsigned char> blob;
+    std::vector<MicroSub> subs;
+    int smem = 0;      // largest subtree (bytes)
+    int width = 1;     // largest level (tasks)
+    struct Item {
+        int level;
+        MicroHead h;
+        std::vector<int4> dims;
+        int64_t nA, nB;   // entries of the operands
+    };
+    std::vector<Item> open;
+
+    bool add(const CDesc &d, int level, int64_t na, int64_t nb, const char *arena, int esz,
+             const unsigned long long *mxb, const int32_t *amb) {
+        if (d.nbeta > MICRO_BETA || d.nout_total * d.nbeta > MICRO_MAX || d.ktotal > (1LL << 30))
+            return false;
+        Item it;
+        it.level = level;
+        it.nA = na;
+        it.nB = nb;
+        MicroHead &m = it.h;
+        std::memset(&m, 0, sizeof m);
+        m.nout = d.nout;
+        m.nk = d.nk;
+        m.flags = d.pow2 ? 1 : 0;
+        m.nout_total = (int32_t)d.nout_total;
+        m.ktotal = (int32_t)d.ktotal;
+        m.nbeta = d.nbeta;
+        m.elems = (int32_t)(d.nout_total * d.nbeta);
+        const int kl = micro_lanes(m.elems, (double)d.ktotal);
+        while ((1 << m.klog) < kl) ++m.klog;
+        m.offA = ((const char *)d.A - arena) / esz;
+        m.offB = ((const char *)d.B - arena) / esz;
+        m.offC = ((const char *)d.C - arena) / esz;
+        m.bsa = (int16_t)d.bsa;   // at most MICRO_MAX, as every tensor
+        m.bsb = (int16_t)d.bsb;
+        for (int i = 0; i < d.nout; ++i)
+            it.dims.push_back(int4{d.osz[i], d.osh[i], (int)d.osa[i], (int)d.osb[i]});
+        for (int i = 0; i < d.nk; ++i)
+            it.dims.push_back(int4{d.ksz[i], d.ksh[i], (int)d.ksa[i], (int)d.ksb[i]});
+        m.mxa = d.mxa ? d.mxa - mxb : -1;
+        m.mxb = d.mxb ? d.mxb - mxb : -1;
+        m.mxc = d.mxc ? d.mxc - mxb : -1;
+        m.mxa_bs = d.mxa_bs;
+        m.mxb_bs = d.mxb_bs;
+        m.amoff = d.argmax ? d.argmax - amb : -1;
+        m.sA = m.sB = m.sC = m.smxa = m.smxb = m.smxc = -1;
+        open.push_back(std::move(it));
+        return true;
     }
-    for (int i = 0; i < d.nk; ++i) {
-        m.ksz[i] = d.ksz[i];
-        m.ksh[i] = d.ksh[i];
-        m.ksa[i] = (int32_t)d.ksa[i];
-        m.ksb[i] = (int32_t)d.ksb[i];
+    // false when the records exceed MICRO_BLOB bytes
+    bool close(int esz) {
+        std::stable_sort(open.begin(), open.end(),
+                         [](const Item &x, const Item &y) { return x.level < y.level; });
+        std::vector<int32_t> lev;
+        std::vector<uint32_t> at, tasks;   // head positions relative to the first head
+        // offset tables of the outputs of an item and of the summed indices
+        // (equal ones stored once); dimensions only where there is no table
+        std::vector<uint32_t> tabs;
+        std::unordered_map<std::string, int32_t> seen;   // by sizes and strides
+        auto table = [&](const int4 *dim, int nd, int total) {
+            auto r = seen.emplace(std::string((const char *)dim, (size_t)nd * sizeof(int4)),
+                                  (int32_t)(tabs.size() * 4));
+            if (!r.second) return r.first->second;
+            int dig[MAXD] = {0};
+            uint32_t a = 0, b = 0;
+            for (int i = 0; i < total; ++i) {
+                tabs.push_back(a | (b << 16));
+                for (int q = nd - 1; q >= 0; --q) {
+                    a += (uint32_t)dim[q].z;
+                    b += (uint32_t)dim[q].w;
+                    if (++dig[q] < dim[q].x) break;
+                    a -= (uint32_t)(dim[q].z * dim[q].x);
+                    b -= (uint32_t)(dim[q].w * dim[q].x);
+                    dig[q] = 0;
+                }
+            }
+            return r.first->second;
+        };
+        uint32_t units = 0;
+        for (auto &it : open) {
+            MicroHead &m = it.h;
+            m.otab = m.nout_total <= MICRO_OTAB ? table(it.dims.data(), m.nout, m.nout_total) : -1;
+            m.ktab = m.ktotal <= MICRO_KTAB
+                         ? table(it.dims.data() + m.nout, m.nk, m.ktotal) : -1;
+            if (m.otab >= 0 && m.ktab >= 0) it.dims.clear();
+            at.push_back(units);
+            units += (uint32_t)(sizeof(MicroHead) / 16 + it.dims.size());
+        }
+        int last = -1;
+        for (size_t i = 0; i < open.size(); ++i) {
+            if (open[i].level != last) lev.push_back((int32_t)tasks.size());
+            last = open[i].level;
+            const int per = 32 >> open[i].h.klog, nt = (open[i].h.elems + per - 1) / per;
+            if (nt == 1 && open[i].h.nbeta == 1) open[i].h.flags |= 2;
+            for (int q = 0; q < nt; ++q) tasks.push_back((at[i] << 16) | (uint32_t)q);
+        }
+        lev.push_back((int32_t)tasks.size());
+        for (size_t i = 0; i + 1 < lev.size(); ++i) width = std::max(width, lev[i + 1] - lev[i]);
+        auto r16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
+        const size_t t0 = r16(lev.size() * 4), h0 = r16(t0 + tasks.size() * 4);
+        const size_t tab0 = h0 + (size_t)units * 16;
+        const size_t bytes = r16(tab0 + tabs.size() * 4);
+        for (auto &it : open) {
+            if (it.h.otab >= 0) it.h.otab += (int32_t)tab0;
+            if (it.h.ktab >= 0) it.h.ktab += (int32_t)tab0;
+        }
+        if (bytes > (size_t)MICRO_BLOB) return false;
+        for (auto &t : tasks) t += (uint32_t)(h0 / 16) << 16;
+        // maxima: staged together, or all left in global memory
+        std::vector<uint32_t> mslot;
+        {
+            std::map<int64_t, int32_t> pos;
+            bool ok = true;
+            auto want = [&](int64_t slot, int n, bool own) {
+                if (slot < 0 || !ok) return;
+                auto r = pos.emplace(slot, (int32_t)mslot.size());
+                if (slot + n > 0x7fffffffLL) ok = false;
+                else if (r.second)
+                    for (int j = 0; j < n; ++j)
+                        mslot.push_back((uint32_t)(slot + j) | (own ? 0x80000000u : 0u));
+                if ((int)mslot.size() > MICRO_MAXIMA) ok = false;
+            };
+            for (auto &it : open) want(it.h.mxc, it.h.nbeta, true);
+            for (auto &it : open) {
+                want(it.h.mxa, it.h.mxa_bs ? it.h.nbeta : 1, false);
+                want(it.h.mxb, it.h.mxb_bs ? it.h.nbeta : 1, false);
+            }
+            if (!ok) mslot.clear();
+            else
+                for (auto &it : open) {
+                    if (it.h.mxa >= 0) it.h.smxa = pos[it.h.mxa];
+                    if (it.h.mxb >= 0) it.h.smxb = pos[it.h.mxb];
+                    if (it.h.mxc >= 0) it.h.smxc = pos[it.h.mxc];
+                }
+        }
+        // values: the smallest tensors first, while they fit
+        std::vector<uint32_t> src;
+        size_t vals = 0;
+        {
+            struct Tn { int64_t n; bool own; int32_t pos; };
+            std::map<int64_t, Tn> ten;   // by arena offset
+            for (auto &it : open) ten[it.h.offC] = {it.h.elems, true, -1};
+            for (auto &it : open) {
+                ten.insert({it.h.offA, {it.nA, false, -1}});
+                ten.insert({it.h.offB, {it.nB, false, -1}});
+            }
+            std::vector<std::pair<int64_t, int64_t>> order;   // entries, offset
+            for (auto &t : ten) order.push_back({t.second.n, t.first});
+            std::sort(order.begin(), order.end());
+            const size_t room =
+                ((size_t)MICRO_SMEM - bytes - ((mslot.size() + 1) & ~(size_t)1) * 8) / esz;
+            for (auto &o : order) {
+                Tn &t = ten[o.second];
+                if (vals + (size_t)t.n > room) break;
+                if (!t.own && o.second + t.n > 0xffffffffLL) continue;
+                vals += (size_t)t.n;
+                t.pos = 0;   // taken
+            }
+            int32_t next = 0;
+            for (bool own : {false, true})   // inputs first: one gather fills them
+                for (auto &kv : ten) {
+                    Tn &t = kv.second;
+                    if (t.pos < 0 || t.own != own) continue;
+                    t.pos = next;
+                    next += (int32_t)t.n;
+                    if (!own)
+                        for (int64_t j = 0; j < t.n; ++j) src.push_back((uint32_t)(kv.first + j));
+                }
+            for (auto &it : open) {
+                it.h.sA = ten[it.h.offA].pos;
+                it.h.sB = ten[it.h.offB].pos;
+                it.h.sC = ten[it.h.offC].pos;
+            }
+        }
+        const size_t off = blob.size();
+        blob.resize(off + r16(bytes + (src.size() + mslot.size()) * 4), 0);
+        std::memcpy(&blob[off], lev.data(), lev.size() * 4);
+        if (!tasks.empty()) std::memcpy(&blob[off + t0], tasks.data(), tasks.size() * 4);
+        for (size_t i = 0; i < open.size(); ++i) {
+            unsigned char *p = &blob[off + h0 + (size_t)at[i] * 16];
+            std::memcpy(p, &open[i].h, sizeof(MicroHead));
+            if (!open[i].dims.empty())
+                std::memcpy(p + sizeof(MicroHead), open[i].dims.data(), open[i].dims.size() * 16);
+        }
+        if (!tabs.empty()) std::memcpy(&blob[off + tab0], tabs.data(), tabs.size() * 4);
+        if (!src.empty()) std::memcpy(&blob[off + bytes], src.data(), src.size() * 4);
+        if (!mslot.empty())
+            std::memcpy(&blob[off + bytes + src.size() * 4], mslot.data(), mslot.size() * 4);
+        MicroSub sub;
+        std::memset(&sub, 0, sizeof sub);
+        sub.off = (int64_t)off;
+        sub.bytes = (int32_t)bytes;
+        sub.nlevels = (int32_t)lev.size() - 1;
+        sub.tasks = (int32_t)t0;
+        sub.nin = (int32_t)src.size();
+        sub.nmx = (int32_t)mslot.size();
+        subs.push_back(sub);
+        smem = std::max(smem, (int)(bytes + ((mslot.size() + 1) & ~(size_t)1) * 8 + vals * esz));
+        open.clear();
+        return true;
     }
-    m.mxa = d.mxa ? d.mxa - mxb : -1;
-    m.mxb = d.mxb ? d.mxb - mxb : -1;
-    m.mxc = d.mxc ? d.mxc - mxb : -1;
-    m.mxa_bs = d.mxa_bs;
-    m.mxb_bs = d.mxb_bs;
-    m.amoff = d.argmax ? d.argmax - amb : -1;
-    return true;
-}
+};
 
 // Inner offset tables of the streaming kernels (computed once per node).
 // Chunk table of one operand tile of a dense kernel (dense_impl.cuh): tiles
@@ -1330,14 +1500,24 @@ tn_status build_program(tn_model *m, const Net &net, const Tree &tree, int kind,
         }
     }
     P.nmx = nmx;
-    // ---- micro subtrees: maximal subtrees of at most MICRO_NODES nodes whose
-    // tensors (and adjoints) all hold at most MICRO_MAX entries
+    // ---- micro subtrees: maximal subtrees of cheap nodes whose tensors (and
+    // adjoints) all hold at most MICRO_MAX entries.  A node is cheap up to the
+    // warp steps that one CTA does in about the 4 us that a launch of its own
+    // takes in a chain of dependent launches (FP64: two multiply-adds a clock
+    // and SM, so fewer); a subtree stops where one CTA's serial work outgrows
+    // running its parts on several SMs and launching the rest.  Measured (us a
+    // call, limits 512 / 1536 / 4096): 24 x 24 grid TF32 3202 / 3108 / 3060;
+    // 10 x 10 grid FP64 581 / 515 / 513, and a batch of 12 x 12 grids FP64
+    // 1529 / 1504 / 1509; MAP of 300 variables 164 / 182 / 181 (the first
+    // levels hold half the nodes, and no other lane runs beside them)
     P.micro.assign(NN, 0);
     std::vector<int> micro_root(NN, -1);
     if (nbeta <= MICRO_BETA) {
+        const double node_max = dtype == 0 ? 256 : 512;
+        const double tree_max = maxplus ? 512 : dtype == 0 ? 1536 : 4096;
         std::vector<char> small(NN, 0);
-        std::vector<int> cnt(NN, 0);
-        const int INF = 1 << 29;
+        std::vector<double> cost(NN, 0);
+        std::vector<int64_t> bytes(NN, 0);   // records of the subtree
         auto emax = [&](int id) {
             int64_t e = P.fwd[id].elems;
             if (backward) e = std::max(e, P.adj[id].elems);
@@ -1348,14 +1528,43 @@ tn_status build_program(tn_model *m, const Net &net, const Tree &tree, int kind,
             bool ok = !nd.gemm && emax(id) <= MICRO_MAX && emax(nd.a) <= MICRO_MAX &&
                       emax(nd.b) <= MICRO_MAX && (nd.a < n || small[nd.a]) &&
                       (nd.b < n || small[nd.b]);
-            small[id] = ok;
-            cnt[id] = ok ? 1 + (nd.a < n ? 0 : cnt[nd.a]) + (nd.b < n ? 0 : cnt[nd.b]) : INF;
+            if (!ok) continue;
+            // steps and record bytes of each pass, the larger pass counts
+            int64_t dims = 0;
+            for (int c : {nd.a, nd.b}) dims += (int64_t)pl.node[c].labels.size();
+            auto rec = [&](int64_t per, int64_t elems, double K) {
+                return (int64_t)sizeof(MicroHead) + 4 * ((elems * micro_lanes(elems, K) + 31) / 32) +
+                       (per <= MICRO_OTAB && K <= MICRO_KTAB ? 0 : 16 * dims) +
+                       (per <= MICRO_OTAB ? 4 * per : 0) + (K <= MICRO_KTAB ? 4 * (int64_t)K : 0);
+            };
+            auto kof = [&](int64_t size) { return nd.muladds / (double)size; };
+            const double kf = kof(nd.size);
+            double c = micro_cost(P.fwd[id].elems, kf), worst = c;
+            int64_t by = rec(nd.size, P.fwd[id].elems, kf);
+            if (backward) {
+                double cb = 0;
+                int64_t bb = 0;
+                for (int ch : {nd.a, nd.b})
+                    if (P.need_adj[ch]) {
+                        const double k = kof(pl.node[ch].size);
+                        cb += micro_cost(P.adj[ch].elems, k);
+                        worst = std::max(worst, micro_cost(P.adj[ch].elems, k));
+                        bb += rec(pl.node[ch].size, P.adj[ch].elems, k);
+                    }
+                c = std::max(c, cb);
+                by = std::max(by, bb);
+            }
+            if (worst > node_max) continue;
+            small[id] = 1;
+            cost[id] = c + cost[nd.a] + cost[nd.b];
+            bytes[id] = by + bytes[nd.a] + bytes[nd.b];
         }
         for (int id = NN - 1; id >= n; --id) {
             int par = pl.node[id].parent;
             if (par >= 0 && micro_root[par] >= 0) {
                 micro_root[id] = micro_root[par];
-            } else if (small[id] && cnt[id] <= MICRO_NODES) {
+            } else if (small[id] && cost[id] <= tree_max &&
+                       bytes[id] + 8192 <= (int64_t)MICRO_BLOB) {
                 micro_root[id] = id;
             }
             if (micro_root[id] >= 0) P.micro[id] = 1;
@@ -1838,58 +2047,65 @@ tn_status build_program(tn_model *m, const Net &net, const Tree &tree, int kind,
     P.mlane_beg.assign(P.nlanes + 1, 0);
     for (auto &lo : morder) P.mlane_beg[lo.first + 1]++;
     for (int l = 0; l < P.nlanes; ++l) P.mlane_beg[l + 1] += P.mlane_beg[l];
+    MicroList mf, mb;
+    std::vector<int> mlev(NN, 0);   // height inside the subtree (forward level)
     for (auto &lo : morder) {
         auto &kv = *msub.find(lo.second);
-        P.mf_beg.push_back((int32_t)P.mf.size());
         for (int id : kv.second) {
-            MicroDesc md;
-            if (!to_micro(P.fdesc[id - n], P.arena, P.esz, P.mx, P.am, md))
+            const Node &nd = pl.node[id];
+            mlev[id] = 1 + std::max(mlev[nd.a], mlev[nd.b]);
+            if (!mf.add(P.fdesc[id - n], mlev[id], P.fwd[nd.a].elems, P.fwd[nd.b].elems, P.arena,
+                        P.esz, P.mx, P.am))
                 return fail(TN_E_UNSUPPORTED, "micro node conversion");
-            P.mf.push_back(md);
         }
+        if (!mf.close(P.esz)) return fail(TN_E_UNSUPPORTED, "micro subtree records");
         if (!backward) continue;
-        P.mb_beg.push_back((int32_t)P.mb.size());
+        std::vector<int> depth(NN, 0);   // backward level: distance from the subtree's root
         for (auto it = kv.second.rbegin(); it != kv.second.rend(); ++it) {
             int id = *it;
             const Node &nd = pl.node[id];
             const Node &na = pl.node[nd.a], &nb = pl.node[nd.b];
             char *cbar = aptr(id);
+            depth[nd.a] = depth[nd.b] = depth[id] + 1;
             CDesc d;
-            MicroDesc md;
             if (P.need_adj[nd.a]) {
                 err = make_desc(net.card, alab(id), P.adj_beta[id], P.adj[id].per, cbar,
                                 P.mx + P.adj[id].mx, nb.labels, nb.beta, P.fwd[nd.b].per,
                                 fptr(nd.b), P.mx + P.fwd[nd.b].mx, alab(nd.a), P.adj_beta[nd.a],
                                 aptr(nd.a), P.mx + P.adj[nd.a].mx, nullptr, nbeta, nullptr, d);
-                if (!err.empty() || !to_micro(d, P.arena, P.esz, P.mx, P.am, md))
+                if (!err.empty() || !mb.add(d, depth[id], P.adj[id].elems, P.fwd[nd.b].elems,
+                                            P.arena, P.esz, P.mx, P.am))
                     return fail(TN_E_UNSUPPORTED, "micro adjoint conversion");
-                P.mb.push_back(md);
             }
             if (P.need_adj[nd.b]) {
                 err = make_desc(net.card, na.labels, na.beta, P.fwd[nd.a].per, fptr(nd.a),
                                 P.mx + P.fwd[nd.a].mx, alab(id), P.adj_beta[id], P.adj[id].per,
                                 cbar, P.mx + P.adj[id].mx, alab(nd.b), P.adj_beta[nd.b],
                                 aptr(nd.b), P.mx + P.adj[nd.b].mx, nullptr, nbeta, nullptr, d);
-                if (!err.empty() || !to_micro(d, P.arena, P.esz, P.mx, P.am, md))
+                if (!err.empty() || !mb.add(d, depth[id], P.fwd[nd.a].elems, P.adj[id].elems,
+                                            P.arena, P.esz, P.mx, P.am))
                     return fail(TN_E_UNSUPPORTED, "micro adjoint conversion");
-                P.mb.push_back(md);
             }
         }
+        if (!mb.close(P.esz)) return fail(TN_E_UNSUPPORTED, "micro subtree records");
     }
-    P.mf_beg.push_back((int32_t)P.mf.size());
-    P.mb_beg.push_back((int32_t)P.mb.size());
-    if (!P.mf.empty()) {
-        CK(P.mem.alloc(&P.d_mf, sizeof(MicroDesc) * P.mf.size()));
-        CK(cudaMemcpy(P.d_mf, P.mf.data(), sizeof(MicroDesc) * P.mf.size(), cudaMemcpyHostToDevice));
-        CK(P.mem.alloc(&P.d_mf_beg, 4 * P.mf_beg.size()));
-        CK(cudaMemcpy(P.d_mf_beg, P.mf_beg.data(), 4 * P.mf_beg.size(), cudaMemcpyHostToDevice));
-    }
-    if (!P.mb.empty()) {
-        CK(P.mem.alloc(&P.d_mb, sizeof(MicroDesc) * P.mb.size()));
-        CK(cudaMemcpy(P.d_mb, P.mb.data(), sizeof(MicroDesc) * P.mb.size(), cudaMemcpyHostToDevice));
-        CK(P.mem.alloc(&P.d_mb_beg, 4 * P.mb_beg.size()));
-        CK(cudaMemcpy(P.d_mb_beg, P.mb_beg.data(), 4 * P.mb_beg.size(), cudaMemcpyHostToDevice));
-    }
+    auto upload_micro = [&](const MicroList &l, unsigned char **blob, MicroSub **subs) -> cudaError_t {
+        if (l.subs.empty()) return cudaSuccess;
+        cudaError_t e = P.mem.alloc(blob, l.blob.size());
+        if (e == cudaSuccess) e = P.mem.alloc(subs, l.subs.size() * sizeof(MicroSub));
+        if (e == cudaSuccess)
+            e = cudaMemcpy(*blob, l.blob.data(), l.blob.size(), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess)
+            e = cudaMemcpy(*subs, l.subs.data(), l.subs.size() * sizeof(MicroSub),
+                           cudaMemcpyHostToDevice);
+        return e;
+    };
+    P.mf_smem = mf.smem;
+    P.mb_smem = mb.smem;
+    P.mf_width = mf.width;
+    P.mb_width = mb.width;
+    CK(upload_micro(mf, &P.d_mf, &P.d_mf_sub));
+    CK(upload_micro(mb, &P.d_mb, &P.d_mb_sub));
     // ---- step lanes and the events that order them across lanes: event id
     // for fwd[v] = v, for adj[v] = NN + v (the root adjoint's is recorded
     // after it is set to one), 2 NN = start, 2 NN + 1 + l = end of lane l
@@ -2353,12 +2569,14 @@ void enqueue_program(tn_model *m, Program &P, cudaStream_t st, Prof *pr = nullpt
         for (int l = 1; l < P.nlanes; ++l) cudaStreamWaitEvent(lane_stream(l), P.ev[2 * NN], 0);
     }
     // micro subtrees: one launch, or one per lane when the lanes run apart
-    auto micro = [&](const MicroDesc *d, const int32_t *beg, int sem) {
+    auto micro = [&](const unsigned char *d, const MicroSub *subs, int smem, int width, int sem) {
+        // a warp per task of the widest level, 4 to 32
+        const int thr = std::min(MICRO_THREADS, std::max(128, 32 * width));
         if (!par) {
             int ns = (int)P.mlane_beg.back();
             if (ns > 0) {
                 timed(pr, st, C_SMALL, 0, 0,
-                      [&] { launch_micro<T>(d, beg, ns, sem, (T *)P.arena, P.mx, P.am, st); });
+                      [&] { launch_micro<T>(d, subs, ns, smem, sem, thr, (T *)P.arena, P.mx, P.am, st); });
                 ++nl;
             }
             return;
@@ -2366,11 +2584,12 @@ void enqueue_program(tn_model *m, Program &P, cudaStream_t st, Prof *pr = nullpt
         for (int l = 0; l < P.nlanes; ++l) {
             int s0 = P.mlane_beg[l], s1 = P.mlane_beg[l + 1];
             if (s1 <= s0) continue;
-            launch_micro<T>(d, beg + s0, s1 - s0, sem, (T *)P.arena, P.mx, P.am, lane_stream(l));
+            launch_micro<T>(d, subs + s0, s1 - s0, smem, sem, thr, (T *)P.arena, P.mx, P.am,
+                            lane_stream(l));
             ++nl;
         }
     };
-    if (!P.mf.empty()) micro(P.d_mf, P.d_mf_beg, maxplus ? MAXPLUS : SUM);
+    if (P.d_mf) micro(P.d_mf, P.d_mf_sub, P.mf_smem, P.mf_width, maxplus ? MAXPLUS : SUM);
     auto run_steps = [&](std::vector<Step> &steps) {
         for (auto &s : steps) {
             cudaStream_t ls = lane_stream(s.lane);
@@ -2404,7 +2623,7 @@ void enqueue_program(tn_model *m, Program &P, cudaStream_t st, Prof *pr = nullpt
         ++nl;
         if (par) cudaEventRecord(P.ev[NN + pl.root], st);
         run_steps(P.bsteps);
-        if (!P.mb.empty()) micro(P.d_mb, P.d_mb_beg, SUM);
+        if (P.d_mb) micro(P.d_mb, P.d_mb_sub, P.mb_smem, P.mb_width, SUM);
         join_lanes();
         launch_marginals<T>(P.d_margrec, m->md.nvars, P.nbeta, (const T *)P.arena,
                             (const T *)P.arena, P.d_marg, P.marg_stride, st);

@@ -1,0 +1,97 @@
+"""GPU kernels at the sizes where their variants change (edges of tiles,
+remainders, smallest and largest of a rule's range), against the oracle."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2405_14060_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+if torch.cuda.is_available():
+    from paper_2405_14060_gb300 import tn
+
+
+def _two_tables(nvars, card, seed):
+    """Two factors over the same variables: the last contraction sums them all."""
+    rng = np.random.default_rng(seed)
+    scope = np.arange(nvars, dtype=np.int32)
+    t = [rng.random(card ** nvars) + 1e-3 for _ in range(2)]
+    return synth.Model(np.full(nvars, card, np.int32), [scope, scope], t)
+
+
+# summed spaces: two and eight entries (registers), scanned (27, 511 and one
+# label of 100), block sums (512 and 2187 entries, a ragged last block)
+@pytest.mark.parametrize("nvars,card", [(1, 2), (3, 2), (3, 3), (1, 100), (9, 2), (7, 3)])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_sampling_summed_spaces(nvars, card, prec):
+    m = _two_tables(nvars, card, nvars)
+    M = tn.Model.from_synth(m)
+    n = 100000
+    s = M.sample(n, seed=11, prec=prec)
+    idx = np.zeros(n, np.int64)
+    for v in range(nvars):
+        idx = idx * card + s[:, v]
+    joint = m.tables[0] * m.tables[1]
+    expc = joint / joint.sum() * n
+    emp = np.bincount(idx, minlength=len(joint))
+    keep = expc >= 5
+    chi2 = np.sum((emp[keep] - expc[keep]) ** 2 / expc[keep])
+    dof = int(keep.sum()) - 1
+    assert chi2 < dof + 6 * np.sqrt(2 * dof)
+    for k in (1, 33, 129):      # counter-based: a longer run starts with a shorter one's rows
+        np.testing.assert_array_equal(M.sample(k, seed=11, prec=prec), s[:k])
+
+
+# values of a sample in shared memory with 128, 64 and 32 threads a block, and
+# beyond its size in the output rows
+@pytest.mark.parametrize("nvars", [7, 900, 2000, 3300])
+def test_sampling_many_variables(nvars):
+    m = synth.tree_ising(nvars, 5, 0.7)
+    M = tn.Model.from_synth(m)
+    n = 4001
+    s = M.sample(n, seed=3)
+    # closed form: the spins of an edge agree with probability e^J / (e^J + e^-J)
+    spin = 2 * s.astype(np.int64) - 1
+    for (i, j), t in list(zip(m.scopes, m.tables))[:50]:
+        want = (t[0] - t[1]) / (t[0] + t[1])
+        assert abs(np.mean(spin[:, i] * spin[:, j]) - want) < 6 / np.sqrt(n)
+    np.testing.assert_array_equal(M.sample(130, seed=3), s[:130])
+
+
+@pytest.mark.parametrize("mk", [lambda: synth.chain_model(40, [5, 2, 3, 4] * 10, 3),
+                                lambda: synth.bayes_net(60, 4),
+                                lambda: synth.grid_ising(5, 6),
+                                lambda: _two_tables(4, 5, 9)])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_backtrack_levels(mk, prec):
+    m = mk()
+    M = tn.Model.from_synth(m)
+    for method in (0, 1):
+        M.set_order(*M.optimize_order(method, 2, 1))
+        x, lp = M.map(prec=prec)
+        xo, lpo = oracle.ve_map(m)
+        np.testing.assert_array_equal(x, xo)
+        assert abs(lp - lpo) < (1e-9 if prec == "fp64" else 1e-4)
+
+
+# micro subtrees: batches whose items share a warp or not (2 to 48 entries an
+# item, powers of two and not), summed spaces shared by lanes, cards that give
+# tables with and without power-of-two sizes, tensors too large to be staged
+@pytest.mark.parametrize("batch", [1, 3, 32, 100])
+@pytest.mark.parametrize("mk", [lambda: synth.random_markov(12, 14, 3, 2, cards=(2, 3)),
+                                lambda: synth.bayes_net(30, 8, cards=(2, 4)),
+                                lambda: synth.chain_model(12, [37] * 12, 4),
+                                lambda: synth.grid_ising(6, 9)])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_micro_subtrees(mk, batch, prec):
+    m = mk()
+    ev = synth.evidence_batch(m, batch, 0.2, 17)
+    M = tn.Model.from_synth(m)
+    lz, mg = M.mar(ev, prec=prec)
+    tol = 1e-10 if prec == "fp64" else 1e-4
+    for b in sorted({0, batch // 2, batch - 1}):
+        lo, mo = oracle.ve_mar(m, ev[b])
+        # the stated log Z (relative) and marginal tolerances of each precision
+        assert abs(lz[b] - lo) <= tol * max(1.0, abs(lo))
+        assert np.max(np.abs(mg[b] - np.concatenate(mo))) <= tol
