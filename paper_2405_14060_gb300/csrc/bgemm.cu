@@ -12,6 +12,9 @@
 //                Each thread holds a TM x TN register tile whose rows and
 //                columns are strided by the thread grid, so that consecutive
 //                lanes store consecutive entries along C's fastest group.
+//   k_bgemm_direct  FP64: a warp computes a strip of
+//                rows times 1, 2 or 4 columns straight from the operands (L1),
+//                without tiles in shared memory.
 //   k_bgemm_fin  when K is split: sums the split partials in split order
 //                (deterministic), applies the operands' power-of-two scales,
 //                stores C and records its per-item maximum.
@@ -23,6 +26,7 @@
 #include <algorithm>
 #include <cmath>
 #include <mutex>
+#include <utility>
 
 #include "bgemm.cuh"
 #include "devutil.cuh"
@@ -57,6 +61,22 @@ __device__ __forceinline__ TilePos tile_pos(const BDesc &d, int64_t t, int BM, i
         p.g = r;
     }
     q = div_tile(q, d.nbeta, log2_if_pow2(d.nbeta), r);
+    p.beta = r;
+    p.split = (int)q;
+    return p;
+}
+
+// Task t of the direct kernel: columns fastest, then rows, G, items, splits.
+__device__ __forceinline__ TilePos direct_pos(const BDesc &d, int64_t t, int MW, int TN) {
+    const int64_t tm = (d.M + MW - 1) / MW, tn = (d.N + TN - 1) / TN;
+    TilePos p;
+    int64_t r, q = div_tile(t, tn, -1, r);
+    p.n0 = r * TN;
+    q = div_tile(q, tm, -1, r);
+    p.m0 = r * MW;
+    q = div_tile(q, d.G, -1, r);
+    p.g = r;
+    q = div_tile(q, d.nbeta, -1, r);
     p.beta = r;
     p.split = (int)q;
     return p;
@@ -241,6 +261,100 @@ __global__ void __launch_bounds__(kThreads, 2)
     cp_async_wait<0>();
 }
 
+// One warp per task: 32 / KL rows (lanes) times TN columns of one (item, g),
+// over one split of the summed space, KL = 1 << klog lanes sharing an output's
+// summed indices.  Tasks run columns fastest, so the warps of a block read the
+// same rows of A.
+//
+// FP64: an SM does two multiply-adds a clock, a warp's multiply-add takes 16,
+// its two or three loads (L1 hits) 2 to 32, so nothing but the count of
+// multiply-adds matters: no padding (a 64 x 64 x 16 tile costs 16 us whatever
+// part of it is used) and an even spread over the SMs.  The small nodes of a
+// 12 x 12 grid with 16 evidence sets took 29 us each on tiles and take 7.4 us;
+// 10 x 10 grid PR + MAR 520 -> 253 us, the batched 12 x 12 step 1112 -> 381 us.
+template <typename T, int TN>
+__global__ void __launch_bounds__(kThreads) k_bgemm_direct(const __grid_constant__ BDesc d, T *part,
+                                                           int64_t ntask) {
+    __shared__ double smax[kThreads / 32];
+    __shared__ int64_t sbeta[kThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int KL = 1 << d.klog, ks = lane & (KL - 1), MW = 32 >> d.klog;
+    const int64_t t = (int64_t)blockIdx.x * (kThreads / 32) + warp;
+    int64_t beta = -1;
+    T mx = 0;
+    if (t < ntask) {
+        const TilePos tp = direct_pos(d, t, MW, TN);
+        beta = tp.beta;
+        const int64_t m = tp.m0 + (lane >> d.klog);
+        const bool om = m < d.M;
+        const T *A = (const T *)d.A + tp.beta * d.bsa + __ldg(d.tag + tp.g) +
+                     __ldg(d.tam + (om ? m : d.M - 1));
+        const T *B = (const T *)d.B + tp.beta * d.bsb + __ldg(d.tbg + tp.g);
+        int32_t bo[TN];
+#pragma unroll
+        for (int j = 0; j < TN; ++j)
+            bo[j] = __ldg(d.tbn + (tp.n0 + j < d.N ? tp.n0 + j : d.N - 1));
+        T acc[TN];
+#pragma unroll
+        for (int j = 0; j < TN; ++j) acc[j] = T(0);
+        const int k0 = (int)(tp.split * d.kchunk);
+        const int k1 = (int)min(d.K, (int64_t)k0 + d.kchunk);
+#pragma unroll 4
+        for (int k = k0 + ks; k < k1; k += KL) {
+            const int32_t ka = __ldg(d.tak + k), kb = __ldg(d.tbk + k);
+            const T a = __ldg(A + ka);
+#pragma unroll
+            for (int j = 0; j < TN; ++j) acc[j] += a * __ldg(B + (bo[j] + kb));
+        }
+        for (int s = KL >> 1; s > 0; s >>= 1)
+#pragma unroll
+            for (int j = 0; j < TN; ++j) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], s);
+        const bool st = om && ks == 0;
+        if (d.nsplit > 1) {
+            // unscaled partials, dense [split][item][g][n][m]
+            T *P = part + (((int64_t)tp.split * d.nbeta + tp.beta) * d.G + tp.g) * d.M * d.N;
+#pragma unroll
+            for (int j = 0; j < TN; ++j)
+                if (st && tp.n0 + j < d.N) P[(tp.n0 + j) * d.M + m] = acc[j];
+        } else {
+            const T sca = d.mxa ? pow2neg<T>(exp_of_bits(d.mxa[tp.beta * d.mxa_bs])) : T(1);
+            const T scb = d.mxb ? pow2neg<T>(exp_of_bits(d.mxb[tp.beta * d.mxb_bs])) : T(1);
+            const T sc = sca * scb;
+            T *Cb = (T *)d.C + tp.beta * d.bsc + __ldg(d.tcg + tp.g) + __ldg(d.tcm + (om ? m : 0));
+#pragma unroll
+            for (int j = 0; j < TN; ++j)
+                if (st && tp.n0 + j < d.N) {
+                    const T v = acc[j] * sc;
+                    Cb[__ldg(d.tcn + tp.n0 + j)] = v;
+                    mx = mx > v ? mx : v;
+                }
+        }
+    }
+    if (!d.mxc || d.nsplit > 1) return;   // uniform
+    // one recorded maximum per run of equal items in the block
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) {
+        const T o = __shfl_xor_sync(0xffffffffu, mx, s);
+        mx = mx > o ? mx : o;
+    }
+    if (lane == 0) {
+        smax[warp] = (double)mx;
+        sbeta[warp] = beta;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 0; w < kThreads / 32;) {
+            const int64_t b = sbeta[w];
+            unsigned long long m = 0ull;
+            for (; w < kThreads / 32 && sbeta[w] == b; ++w) {
+                const unsigned long long o = dbits(smax[w]);
+                m = o > m ? o : m;
+            }
+            if (b >= 0 && m) atomicMax(d.mxc + b, m);
+        }
+    }
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_bgemm_fin(const __grid_constant__ BDesc d,
                                                         const T *part) {
@@ -276,18 +390,6 @@ struct Tiles<float> {
     static constexpr int BM[4] = {128, 256, 256, 128}, BN[4] = {64, 32, 16, 8};
     static constexpr int TM[4] = {8, 8, 8, 4}, TN[4] = {4, 4, 2, 1};
 };
-template <>
-struct Tiles<double> {
-    static constexpr int BM[4] = {64, 64, 128, 128}, BN[4] = {64, 32, 16, 8};
-    static constexpr int TM[4] = {4, 2, 4, 4}, TN[4] = {4, 4, 2, 1};
-};
-
-template <typename T>
-void tile_dims(const BDesc &d, int &bm, int &bn) {
-    bm = Tiles<T>::BM[d.tile];
-    bn = Tiles<T>::BN[d.tile];
-}
-
 template <typename T, int TILE>
 constexpr size_t smem_bytes() {
     return (size_t)kStages * kBK *
@@ -324,12 +426,69 @@ void go(const BDesc &d, T *part, int64_t ntiles, cudaStream_t st) {
 
 }  // namespace
 
+// Direct form: warps wanted (eight an SM keep the FP64 pipe and the load
+// latency covered), then the most columns per thread (loads of A shared), lanes
+// per output and splits of the summed space that give them.
+static int64_t direct_tasks(const BDesc &d) {
+    const int64_t mw = 32 >> d.klog;
+    return ((d.M + mw - 1) / mw) * ((d.N + d.direct - 1) / d.direct) * d.G * d.nbeta;
+}
+static void configure_direct(BDesc &d) {
+    const int64_t want = 152LL * 8;
+    // lanes run along rows: C's fastest group goes there when the columns fill
+    // a warp's store
+    if (d.c_nfast && d.N >= 16) {
+        std::swap(d.M, d.N);
+        std::swap(d.A, d.B);
+        std::swap(d.bsa, d.bsb);
+        std::swap(d.mxa, d.mxb);
+        std::swap(d.mxa_bs, d.mxb_bs);
+        std::swap(d.tag, d.tbg);
+        std::swap(d.tam, d.tbn);
+        std::swap(d.tcm, d.tcn);
+        std::swap(d.tak, d.tbk);
+        std::swap(d.a_kfast, d.b_kfast);
+        d.c_nfast = 0;
+    }
+    d.klog = 0;
+    while (d.klog < 5 && (16 >> d.klog) >= d.M && d.K >= (8LL << d.klog)) ++d.klog;
+    d.direct = d.N >= 4 ? 4 : d.N >= 2 ? 2 : 1;
+    // a long summed space is split over blocks (their loads of A still serve
+    // four columns), a shorter one over the columns and lanes of a warp, which
+    // needs no second kernel
+    if (d.K < 4096) {
+        while (d.direct > 1 && direct_tasks(d) < want) d.direct /= 2;
+        while (d.klog < 5 && direct_tasks(d) < want && d.K >= (8LL << d.klog)) ++d.klog;
+    }
+    int64_t ns = 1;
+    const int64_t tasks = direct_tasks(d);
+    if (tasks < want && d.K >= 1024)
+        ns = std::max<int64_t>(1, std::min<int64_t>((want + tasks - 1) / tasks, d.K / 512));
+    d.kchunk = (d.K + ns - 1) / ns;
+    d.kchunk = std::max<int64_t>((d.kchunk + 31) / 32 * 32, 32);
+    d.nsplit = (int)std::max<int64_t>(1, (d.K + d.kchunk - 1) / d.kchunk);
+}
+
 // Tile shape and K split; d.tile = -1 when the contraction does not fit the
 // kernels' 31-bit tile and group indices.
 void bgemm_configure(BDesc &d, int elem_bytes) {
+    d.direct = 0;
+    d.klog = 0;
+    d.tc = 0;
     d.tile = d.N > 48 ? 0 : d.N > 16 ? 1 : d.N > 8 ? 2 : 3;
-    const int bm = elem_bytes == 8 ? Tiles<double>::BM[d.tile] : Tiles<float>::BM[d.tile];
-    const int bn = elem_bytes == 8 ? Tiles<double>::BN[d.tile] : Tiles<float>::BN[d.tile];
+    if (d.M >= (1LL << 31) || d.N >= (1LL << 31) || d.K >= (1LL << 31)) {
+        d.tile = -1;
+        return;
+    }
+    // FP64 always direct (the pipe's two multiply-adds a clock and SM leave
+    // nothing for tiles to save); FP32 never: tiles and direct form measured the
+    // same on the 24 x 24 grid's small nodes (3026 us a call against 3046)
+    if (elem_bytes == 8) {
+        configure_direct(d);
+        if ((double)direct_tasks(d) * d.nsplit >= 1e10) d.tile = -1;
+        return;
+    }
+    const int bm = Tiles<float>::BM[d.tile], bn = Tiles<float>::BN[d.tile];
     const int64_t tiles = ((d.M + bm - 1) / bm) * ((d.N + bn - 1) / bn) * d.G * d.nbeta;
     // split the summed space when the output tiles alone leave most SMs idle
     // and every split still runs several K steps; partials stay under 1 GiB
@@ -349,13 +508,11 @@ void bgemm_configure(BDesc &d, int elem_bytes) {
     d.nsplit = (int)((d.K + d.kchunk - 1) / d.kchunk);
     if (d.nsplit < 1) d.nsplit = 1;
     // the kernels count tiles and index groups in 31 bits
-    if ((double)tiles * d.nsplit >= 2147483647.0 || d.M >= (1LL << 31) || d.N >= (1LL << 31) ||
-        d.K >= (1LL << 31))
-        d.tile = -1;
+    if ((double)tiles * d.nsplit >= 2147483647.0) d.tile = -1;
     // float data with whole K per tile and wide tiles: the tensor-core gather
     // kernel (with 32-column tiles its per-tile handoffs cost more than the
     // CUDA-core multiply-adds; measured on the 3-regular batched workload)
-    d.tc = elem_bytes == 4 && d.tile >= 0 && d.nsplit == 1 && d.N > 64 && d.M >= 128 &&
+    d.tc = d.tile >= 0 && d.nsplit == 1 && d.N > 64 && d.M >= 128 &&
            (double)tc_gather_tiles(d) < 2147483647.0;
 }
 
@@ -366,34 +523,46 @@ size_t bgemm_scratch_bytes(const BDesc &d, int elem_bytes) {
 
 int bgemm_launches(const BDesc &d) { return d.nsplit > 1 && !d.tc ? 2 : 1; }
 
-template <typename T>
-void launch_bgemm(const BDesc &d, void *scratch, cudaStream_t st) {
+template <>
+void launch_bgemm<double>(const BDesc &d, void *scratch, cudaStream_t st) {
     const int64_t outs = d.G * d.M * d.N * d.nbeta;
     if (outs == 0) return;
-    if (sizeof(T) == 4 && d.tc) {
+    const int64_t ntask = direct_tasks(d) * d.nsplit;
+    const unsigned grid = (unsigned)((ntask + kThreads / 32 - 1) / (kThreads / 32));
+    double *p = (double *)scratch;
+    if (d.direct == 1) k_bgemm_direct<double, 1><<<grid, kThreads, 0, st>>>(d, p, ntask);
+    else if (d.direct == 2) k_bgemm_direct<double, 2><<<grid, kThreads, 0, st>>>(d, p, ntask);
+    else k_bgemm_direct<double, 4><<<grid, kThreads, 0, st>>>(d, p, ntask);
+    if (d.nsplit > 1)
+        k_bgemm_fin<double>
+            <<<(unsigned)((outs + kThreads - 1) / kThreads), kThreads, 0, st>>>(d, p);
+}
+
+template <>
+void launch_bgemm<float>(const BDesc &d, void *scratch, cudaStream_t st) {
+    const int64_t outs = d.G * d.M * d.N * d.nbeta;
+    if (outs == 0) return;
+    if (d.tc) {
         launch_tc_gather(d, st);
         return;
     }
-    int bm, bn;
-    tile_dims<T>(d, bm, bn);
+    const int bm = Tiles<float>::BM[d.tile], bn = Tiles<float>::BN[d.tile];
     const int64_t ntiles =
         ((d.M + bm - 1) / bm) * ((d.N + bn - 1) / bn) * d.G * d.nbeta * d.nsplit;
-    T *part = (T *)scratch;
+    float *part = (float *)scratch;
     switch (d.tile * 2 + (d.c_nfast ? 1 : 0)) {
-        case 0: go<T, 0, false>(d, part, ntiles, st); break;
-        case 1: go<T, 0, true>(d, part, ntiles, st); break;
-        case 2: go<T, 1, false>(d, part, ntiles, st); break;
-        case 3: go<T, 1, true>(d, part, ntiles, st); break;
-        case 4: go<T, 2, false>(d, part, ntiles, st); break;
-        case 5: go<T, 2, true>(d, part, ntiles, st); break;
-        case 6: go<T, 3, false>(d, part, ntiles, st); break;
-        default: go<T, 3, true>(d, part, ntiles, st); break;
+        case 0: go<float, 0, false>(d, part, ntiles, st); break;
+        case 1: go<float, 0, true>(d, part, ntiles, st); break;
+        case 2: go<float, 1, false>(d, part, ntiles, st); break;
+        case 3: go<float, 1, true>(d, part, ntiles, st); break;
+        case 4: go<float, 2, false>(d, part, ntiles, st); break;
+        case 5: go<float, 2, true>(d, part, ntiles, st); break;
+        case 6: go<float, 3, false>(d, part, ntiles, st); break;
+        default: go<float, 3, true>(d, part, ntiles, st); break;
     }
     if (d.nsplit > 1)
-        k_bgemm_fin<T><<<(unsigned)((outs + kThreads - 1) / kThreads), kThreads, 0, st>>>(d, part);
+        k_bgemm_fin<float>
+            <<<(unsigned)((outs + kThreads - 1) / kThreads), kThreads, 0, st>>>(d, part);
 }
-
-template void launch_bgemm<float>(const BDesc &, void *, cudaStream_t);
-template void launch_bgemm<double>(const BDesc &, void *, cudaStream_t);
 
 }  // namespace tn

@@ -39,6 +39,8 @@ struct BDesc {
     int nsplit;                    // K split over this many blocks (partials in scratch)
     int64_t kchunk;                // summed indices per split (a multiple of the K tile)
     int tile;                      // tile shape id (see bgemm.cu); -1: does not fit
+    int direct;                    // columns per thread of the direct kernel (0: tiles)
+    int klog;                      // direct kernel: log2 of the lanes that share an output
     int tc;                        // 1: tensor-core gather kernel (float data, no K split)
     int *err;                      // set by a bounded device wait that gave up (tc kernel)
 };
@@ -49,7 +51,7 @@ size_t bgemm_scratch_bytes(const BDesc &d, int elem_bytes);
 // -1 when the contraction exceeds the kernels' index ranges.
 void bgemm_configure(BDesc &d, int elem_bytes);
 template <typename T>
-void launch_bgemm(const BDesc &d, void *scratch, cudaStream_t st);
+void launch_bgemm(const BDesc &d, void *scratch, cudaStream_t st);   // double: direct form
 int bgemm_launches(const BDesc &d);
 // The tensor-core form (tcgather.cu): tiles of 128 rows, and its launch.
 int64_t tc_gather_tiles(const BDesc &d);

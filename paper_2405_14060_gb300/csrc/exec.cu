@@ -1811,6 +1811,24 @@ tn_status build_program(tn_model *m, const Net &net, const Tree &tree, int kind,
         return "";
     };
     auto per_items = [&](bool b) { return b ? (double)nbeta : 1.0; };
+    // FP64 sum-product steps are bound by the multiply-adds (two a clock and SM),
+    // so a step with too few positions to give every SM a block of a streaming
+    // kernel runs on the direct form of the batched GEMM, which spreads outputs
+    // and summed indices evenly (32 x 32 combinations over 128 positions: one
+    // block, 43 us, against 5 us)
+    auto try_bgemm = [&](Step &st, const Opnd &A, const Opnd &B, const Labels &lo, bool bo,
+                         int64_t pero, void *out, unsigned long long *omx) {
+        if (!make_bgemm(net.card, *A.lab, A.beta, A.per, A.ptr, A.mx, *B.lab, B.beta, B.per, B.ptr,
+                        B.mx, lo, bo, pero, out, omx, nbeta, P.esz, st.bd, st.btab))
+            return false;
+        st.kind = 4;
+        scratch = std::max(scratch, bgemm_scratch_bytes(st.bd, P.esz));
+        return true;
+    };
+    auto few_positions = [&](const Step &st) {
+        return dtype == 0 && !maxplus && st.ad.ns * st.ad.nt >= 8 &&
+               st.ad.nr * st.ad.nbeta < 152 * 512;
+    };
     // the forward step of node id writing its result at `outp` (the arena
     // slot, or the recompute slot of a dropped tensor); the operands are
     // always read from their forward slots
@@ -1829,7 +1847,22 @@ tn_status build_program(tn_model *m, const Net &net, const Tree &tree, int kind,
         double items = per_items(nd.beta);
         double flops = 2.0 * nd.muladds * items;
         double bytes = (double)P.esz * (P.fwd[nd.a].elems + P.fwd[nd.b].elems + P.fwd[id].elems);
-        if (nd.gemm) {
+        Step fp64_gemm;   // FP64 has no tensor-core form worth a permutation of the operands
+        const bool direct =
+            nd.gemm && dtype == 0 &&
+            try_bgemm(fp64_gemm,
+                      Opnd{&pl.node[nd.a].labels, pl.node[nd.a].beta, P.fwd[nd.a].per, fptr(nd.a),
+                           mxp(P.fwd[nd.a].mx)},
+                      Opnd{&pl.node[nd.b].labels, pl.node[nd.b].beta, P.fwd[nd.b].per, fptr(nd.b),
+                           mxp(P.fwd[nd.b].mx)},
+                      nd.labels, nd.beta, P.fwd[id].per, outp, mxp(P.fwd[id].mx));
+        if (direct) {
+            fp64_gemm.flops = flops;
+            fp64_gemm.bytes = bytes;
+            fp64_gemm.node = id;
+            fp64_gemm.recompute = recomp;
+            steps.push_back(fp64_gemm);
+        } else if (nd.gemm) {
             Opnd X{&pl.node[nd.ga].labels, pl.node[nd.ga].beta, P.fwd[nd.ga].per, fptr(nd.ga),
                    P.mx + P.fwd[nd.ga].mx};
             Opnd Y{&pl.node[nd.gb].labels, pl.node[nd.gb].beta, P.fwd[nd.gb].per, fptr(nd.gb),
@@ -1858,6 +1891,12 @@ tn_status build_program(tn_model *m, const Net &net, const Tree &tree, int kind,
                             mxp(P.fwd[id].mx), &nd.elim, nbeta,
                             maxplus ? P.am + P.am_off[id] : nullptr, st.ad, !maxplus)) {
                 st.kind = 2;
+                if (few_positions(st))
+                    try_bgemm(st, Opnd{&na.labels, na.beta, P.fwd[nd.a].per, fptr(nd.a),
+                                       mxp(P.fwd[nd.a].mx)},
+                              Opnd{&nb.labels, nb.beta, P.fwd[nd.b].per, fptr(nd.b),
+                                   mxp(P.fwd[nd.b].mx)},
+                              nd.labels, nd.beta, P.fwd[id].per, outp, mxp(P.fwd[id].mx));
             } else if (!maxplus &&
                        make_reduce(net.card, na.labels, na.beta, P.fwd[nd.a].per, fptr(nd.a),
                                    mxp(P.fwd[nd.a].mx), nb.labels, nb.beta, P.fwd[nd.b].per,
@@ -1919,6 +1958,35 @@ tn_status build_program(tn_model *m, const Net &net, const Tree &tree, int kind,
                 }
             double items = per_items(P.adj_beta[id]);
             double flops = 2.0 * nd.muladds * items;
+            // operands of the adjoint steps, in place
+            const Opnd oC{&alab(id), (bool)P.adj_beta[id], P.adj[id].per, cbar,
+                          P.mx + P.adj[id].mx};
+            const Opnd oA{&na.labels, na.beta, P.fwd[nd.a].per, bfptr(nd.a),
+                          P.mx + P.fwd[nd.a].mx};
+            const Opnd oB{&nb.labels, nb.beta, P.fwd[nd.b].per, bfptr(nd.b),
+                          P.mx + P.fwd[nd.b].mx};
+            auto adj_bgemm = [&](Step &st, const Opnd &X, const Opnd &Y, int c) {
+                return try_bgemm(st, X, Y, alab(c), P.adj_beta[c], P.adj[c].per, aptr(c),
+                                 P.mx + P.adj[c].mx);
+            };
+            bool fp64_direct = nd.gemm && dtype == 0;
+            if (fp64_direct) {
+                Step s0, s1;
+                const bool na_ok = !P.need_adj[nd.a] || adj_bgemm(s0, oC, oB, nd.a);
+                const bool nb_ok = !P.need_adj[nd.b] || adj_bgemm(s1, oA, oC, nd.b);
+                fp64_direct = na_ok && nb_ok;
+                for (int c : {nd.a, nd.b}) {
+                    if (!fp64_direct || !P.need_adj[c]) continue;
+                    Step &st = c == nd.a ? s0 : s1;
+                    st.flops = flops;
+                    st.bytes = (double)P.esz * (P.adj[id].elems + P.adj[c].elems +
+                                                P.fwd[c == nd.a ? nd.b : nd.a].elems);
+                    st.node = c;
+                    st.adjoint = true;
+                    P.bsteps.push_back(st);
+                }
+            }
+            if (fp64_direct) continue;
             if (nd.gemm) {
                 const Node &xa = pl.node[nd.ga], &xb = pl.node[nd.gb];
                 Opnd Cb{&alab(id), (bool)P.adj_beta[id], P.adj[id].per, cbar, P.mx + P.adj[id].mx};
@@ -1966,6 +2034,7 @@ tn_status build_program(tn_model *m, const Net &net, const Tree &tree, int kind,
                                 P.adj[nd.a].per, aptr(nd.a), P.mx + P.adj[nd.a].mx, nullptr, nbeta,
                                 nullptr, st.ad, true)) {
                     st.kind = 2;
+                    if (few_positions(st)) adj_bgemm(st, oC, oB, nd.a);
                 } else if (make_bgemm(net.card, alab(id), P.adj_beta[id], P.adj[id].per, cbar,
                                       P.mx + P.adj[id].mx, nb.labels, nb.beta, P.fwd[nd.b].per,
                                       bfptr(nd.b), P.mx + P.fwd[nd.b].mx, alab(nd.a),
@@ -2005,6 +2074,7 @@ tn_status build_program(tn_model *m, const Net &net, const Tree &tree, int kind,
                                  P.adj[nd.b].per, aptr(nd.b), P.mx + P.adj[nd.b].mx, nullptr,
                                  nbeta, nullptr, st.ad, true))) {
                     st.kind = 2;
+                    if (few_positions(st)) adj_bgemm(st, oA, oC, nd.b);
                 } else if (make_reduce(net.card, na.labels, na.beta, P.fwd[nd.a].per, bfptr(nd.a),
                                 P.mx + P.fwd[nd.a].mx, alab(id), P.adj_beta[id], P.adj[id].per,
                                 cbar, P.mx + P.adj[id].mx, alab(nd.b), P.adj_beta[nd.b],
@@ -3949,7 +4019,11 @@ tn_status tn_contract_dev(int nlabels, const int *sizes, int na, const int *labe
             for (int v : l) q *= card[v];
             return q;
         };
-        if (!onesided && prod(gm) >= 64 && prod(gn) >= 64 && prod(gk) >= 64) {
+        // FP64 within the batched GEMM's index ranges runs on its direct form
+        // below, in place
+        const bool direct = dtype == 0 && prod(la) < (1LL << 31) && prod(lb) < (1LL << 31) &&
+                            prod(lc) < (1LL << 31);
+        if (!direct && !onesided && prod(gm) >= 64 && prod(gn) >= 64 && prod(gk) >= 64) {
             int store_t = dtype == 0 ? E_F64 : E_F32;
             int gemm_t = dtype == 0 ? E_F64 : prec == TN_BF16 ? E_BF16 : E_F32;
             Opnd X{&la, false, 0, A, nullptr}, Y{&lb, false, 0, B, nullptr};

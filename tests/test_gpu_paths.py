@@ -95,3 +95,26 @@ def test_micro_subtrees(mk, batch, prec):
         # the stated log Z (relative) and marginal tolerances of each precision
         assert abs(lz[b] - lo) <= tol * max(1.0, abs(lo))
         assert np.max(np.abs(mg[b] - np.concatenate(mo))) <= tol
+
+
+# direct form of the FP64 batched GEMM: one row or column, rows and columns
+# around the strip sizes (32 rows, 1 / 2 / 4 columns), lanes sharing a summed
+# space, splits over blocks with a ragged last one, either side fastest in the
+# output, a group label, GEMM-sized groups
+@pytest.mark.parametrize("m,n,k", [(1, 1, 1), (1, 5, 9), (3, 2, 4097), (20, 30, 9000), (31, 4, 8),
+                                   (33, 7, 17), (64, 65, 66), (130, 3, 700), (257, 129, 64)])
+@pytest.mark.parametrize("spec", ["mk,kn->mn", "km,nk->nm", "gmk,kgn->mgn"])
+def test_direct_fp64(m, n, k, spec):
+    (a, b), c = spec.split("->")[0].split(","), spec.split("->")[1]
+    letters = "gkmn"
+    size = dict(g=3, k=k, m=m, n=n)
+    rng = np.random.default_rng(m * n + k)
+    A = rng.random([size[l] for l in a])
+    B = rng.random([size[l] for l in b])
+    ref = np.einsum(spec, A, B)
+    C = torch.full([size[l] for l in c], float("nan"), dtype=torch.float64, device="cuda")
+    tn.contract_dev([size[l] for l in letters], [letters.index(l) for l in a], torch.tensor(A).cuda(),
+                    [letters.index(l) for l in b], torch.tensor(B).cuda(),
+                    [letters.index(l) for l in c], C)
+    # positive terms: every order of summation is within k ulp
+    np.testing.assert_allclose(C.cpu().numpy(), ref, rtol=k * 2.3e-16 + 1e-15, atol=0)
