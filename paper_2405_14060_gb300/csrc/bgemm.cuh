@@ -45,6 +45,17 @@ struct BDesc {
     int *err;                      // set by a bounded device wait that gave up (tc kernel)
 };
 
+// The group offset tables as dimensions (neighbours fused), for tables built on
+// the device: table i holds n[i] offsets from position start[i].
+constexpr int GT_MAXD = 16;
+struct GroupTabs {
+    int64_t start[9], n[9], total;
+    int32_t nd[9];
+    int32_t sz[9][GT_MAXD];
+    int64_t st[9][GT_MAXD];
+};
+void launch_group_tables(const GroupTabs &g, int32_t *out, cudaStream_t st);
+
 // Scratch bytes of the split-K partials (0 when the K space is not split).
 size_t bgemm_scratch_bytes(const BDesc &d, int elem_bytes);
 // Choose the tile shape and the K split of a descriptor (host); sets tile to

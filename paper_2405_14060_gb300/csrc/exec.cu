@@ -53,6 +53,62 @@ static tn_status fail(tn_status s, const std::string &msg) {
 
 namespace {
 
+constexpr uint64_t kPoolKeep = 512ull << 20;
+std::mutex g_pool_mu;
+std::map<int, cudaMemPool_t> g_pools;
+
+cudaError_t scratch_pool(cudaMemPool_t *out) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    cudaMemPool_t &p = g_pools[dev];
+    if (!p) {
+        cudaMemPoolProps pr;
+        std::memset(&pr, 0, sizeof pr);
+        pr.allocType = cudaMemAllocationTypePinned;
+        pr.handleTypes = cudaMemHandleTypeNone;
+        pr.location.type = cudaMemLocationTypeDevice;
+        pr.location.id = dev;
+        e = cudaMemPoolCreate(&p, &pr);
+        if (e != cudaSuccess) {
+            p = nullptr;
+            return e;
+        }
+        uint64_t keep = kPoolKeep;
+        e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (e != cudaSuccess) return e;
+    }
+    *out = p;
+    return cudaSuccess;
+}
+// Give back what the current device's pool holds unused.
+void trim_scratch_pool() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    auto it = g_pools.find(dev);
+    if (it != g_pools.end() && it->second) cudaMemPoolTrimTo(it->second, 0);
+}
+
+// Stream-ordered scratch of one call; freed on its stream with the object.
+struct CallMem {
+    cudaStream_t st;
+    void *p = nullptr;
+    explicit CallMem(cudaStream_t s) : st(s) {}
+    CallMem(const CallMem &) = delete;
+    ~CallMem() {
+        if (p) cudaFreeAsync(p, st);
+    }
+    cudaError_t alloc(size_t bytes) {
+        cudaMemPool_t pool;
+        cudaError_t e = scratch_pool(&pool);
+        if (e == cudaSuccess) e = cudaMallocFromPoolAsync(&p, std::max<size_t>(bytes, 16), pool, st);
+        if (e != cudaSuccess) p = nullptr;
+        return e;
+    }
+};
+
 struct Slot {
     int64_t off = -1;     // element offset in the arena
     int64_t per = 0;      // entries per item
@@ -103,6 +159,11 @@ struct DevMem {
     cudaError_t alloc(T **p, size_t bytes) {
         void *q = nullptr;
         cudaError_t e = cudaMalloc(&q, std::max<size_t>(bytes, 256));
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            trim_scratch_pool();
+            e = cudaMalloc(&q, std::max<size_t>(bytes, 256));
+        }
         if (e == cudaSuccess) {
             ptrs.push_back(q);
             *p = (T *)q;
@@ -898,7 +959,7 @@ static bool make_bgemm(const std::vector<int> &card, const Labels &lx, bool bx, 
                        const Labels &lo, bool bo, int64_t pero, void *O,
                        unsigned long long *mxo, int nbeta, int esz, BDesc &d,
                        std::vector<int32_t> &tab, bool tc_orient = false,
-                       bool swapped = false) {
+                       GroupTabs *dims = nullptr, bool swapped = false) {
     std::memset(&d, 0, sizeof d);
     if (bo != (bx || by)) return false;
     std::set<int> sx(lx.begin(), lx.end()), sy(ly.begin(), ly.end()), so(lo.begin(), lo.end());
@@ -940,14 +1001,46 @@ static bool make_bgemm(const std::vector<int> &card, const Labels &lx, bool bx, 
     const bool o_in_m = std::find(M.begin(), M.end(), fo) != M.end();
     if (!swapped && (tc_orient && esz == 4 ? (o_in_n || (!o_in_m && d.N > d.M)) : d.N > d.M))
         return make_bgemm(card, ly, by, pery, Y, mxy, lx, bx, perx, X, mxx, lo, bo, pero, O, mxo,
-                          nbeta, esz, d, tab, tc_orient, true);
+                          nbeta, esz, d, tab, tc_orient, dims, true);
     if (perx >= (1LL << 31) || pery >= (1LL << 31) || pero >= (1LL << 31)) return false;
     const int64_t ntab = 3 * d.G + 2 * d.M + 2 * d.N + 2 * d.K;
     if (ntab > (1LL << 26)) return false;
-    tab.assign((size_t)ntab, 0);
+    // tables as dimensions for the device to fill, where they fit its records
+    if (dims) {
+        GroupTabs &g = *dims;
+        std::memset(&g, 0, sizeof g);
+        struct { const Labels *grp, *lt; const std::set<int> *st; } src[9] = {
+            {&G, &lx, &sx}, {&G, &ly, &sy}, {&G, &lo, &so}, {&M, &lx, &sx}, {&M, &lo, &so},
+            {&N, &ly, &sy}, {&N, &lo, &so}, {&K, &lx, &sx}, {&K, &ly, &sy}};
+        bool ok = true;
+        for (int i = 0; i < 9 && ok; ++i) {
+            g.start[i] = g.total;
+            g.n[i] = prod(*src[i].grp);
+            g.total += g.n[i];
+            int &nd = g.nd[i];
+            for (int v : *src[i].grp) {
+                if (card[v] == 1) continue;
+                const int64_t sd = stride_in(card, *src[i].lt, v);
+                if (nd && g.st[i][nd - 1] == sd * card[v] &&
+                    (int64_t)g.sz[i][nd - 1] * card[v] < (1LL << 31)) {
+                    g.sz[i][nd - 1] *= card[v];
+                    g.st[i][nd - 1] = sd;
+                } else if (nd < GT_MAXD) {
+                    g.sz[i][nd] = card[v];
+                    g.st[i][nd++] = sd;
+                } else {
+                    ok = false;
+                }
+            }
+        }
+        if (!ok) g.total = 0;   // filled here instead
+    }
+    const bool host = !dims || dims->total == 0;
+    tab.assign(host ? (size_t)ntab : 0, 0);
     // offsets of every index of a group (labels in the given order, last
     // fastest) in one tensor
     auto fill = [&](const Labels &grp, const Labels &lt, const std::set<int> &st, int32_t *out) {
+        if (!host) return;
         int64_t tot = prod(grp);
         std::vector<int64_t> sz, sd;
         for (int v : grp) {
@@ -966,7 +1059,7 @@ static bool make_bgemm(const std::vector<int> &card, const Labels &lx, bool bx, 
             }
         }
     };
-    int32_t *t = tab.data();
+    int32_t *t = host ? tab.data() : nullptr;
     int64_t p = 0;
     int64_t o_ag = p; fill(G, lx, sx, t + p); p += d.G;
     int64_t o_bg = p; fill(G, ly, sy, t + p); p += d.G;
@@ -1668,6 +1761,7 @@ tn_status build_program(tn_model *m, const Net &net, const Tree &tree, int kind,
     P.keep_all_elems = arena_top;
     int64_t budget = opts ? opts->hbm_budget_bytes : 0;
     size_t freeb = 0, totb = 0;
+    trim_scratch_pool();
     CK(cudaMemGetInfo(&freeb, &totb));
     // the memory the program may take: the budget, else what is free
     const double limit = budget > 0 ? (double)budget : (double)freeb - (double)(256u << 20);
@@ -3639,14 +3733,14 @@ tn_status tn_sample(tn_model *m, const int32_t *evid, uint64_t seed, int64_t n,
         CK(cudaMemcpy(&lz, P->d_logz, 8, cudaMemcpyDeviceToHost));
         if (!(lz > -INFINITY)) return fail(TN_E_ARG, "p(e) = 0");
         if (n == 0) return TN_OK;
-        int8_t *d_out = nullptr;
-        CK(cudaMallocAsync(&d_out, (size_t)n * nv, st));
+        CallMem out(st);
+        CK(out.alloc((size_t)n * nv));
+        int8_t *d_out = (int8_t *)out.p;
         CK(cudaEventRecord(m->ev0, st));
         s = draw_samples(m, *P, n, seed, d_out, st);
         if (s) return s;
         CK(cudaEventRecord(m->ev1, st));
         CK(cudaMemcpyAsync(samples, d_out, (size_t)n * nv, cudaMemcpyDeviceToHost, st));
-        CK(cudaFreeAsync(d_out, st));
         CK(cudaStreamSynchronize(st));
         float ms = 0;
         CK(cudaEventElapsedTime(&ms, m->ev0, m->ev1));
@@ -3712,8 +3806,9 @@ tn_status tn_sample(tn_model *m, const int32_t *evid, uint64_t seed, int64_t n,
         int64_t a = std::upper_bound(cum.begin(), cum.end(), u) - cum.begin();
         cnt[std::min(a, nass - 1)]++;
     }
-    int8_t *d_out = nullptr;
-    CK(cudaMallocAsync(&d_out, (size_t)n * nv, st));
+    CallMem out(st);
+    CK(out.alloc((size_t)n * nv));
+    int8_t *d_out = (int8_t *)out.p;
     int64_t off = 0;
     for (int64_t a = 0; a < nass; ++a) {
         if (!cnt[a]) continue;
@@ -3732,7 +3827,6 @@ tn_status tn_sample(tn_model *m, const int32_t *evid, uint64_t seed, int64_t n,
     }
     std::vector<int8_t> h((size_t)n * nv);
     CK(cudaMemcpyAsync(h.data(), d_out, h.size(), cudaMemcpyDeviceToHost, st));
-    CK(cudaFreeAsync(d_out, st));
     CK(cudaStreamSynchronize(st));
     // rows grouped by assignment -> a uniformly random order (Fisher-Yates)
     std::vector<int64_t> perm(n);
@@ -3952,7 +4046,13 @@ tn_status tn_mmap(tn_model *m, const int32_t *evid, int nq, const int32_t *query
     return finish(*m->mmap->top, lconst, build_ms, launches);
 }
 
-// One pairwise contraction on caller-provided device buffers.
+// Scratch memory of the calls that keep no program (single contractions, the
+// samples of tn_sample) comes from a pool of the library's own on each device:
+// stream-ordered as before, safe from any thread and stream, but up to
+// kPoolKeep bytes stay with it between calls (the default pool hands every
+// byte back at each synchronisation: 100 to 250 us a call to map it again).
+// What it holds is given back before a program measures the free memory, and
+// whenever an allocation of the library fails.
 // One wait-timeout flag per device for the single-contraction entry points,
 // created on first use.
 static tn_status device_err_flag(int **out) {
@@ -3967,6 +4067,19 @@ static tn_status device_err_flag(int **out) {
         CK(cudaMemset(f, 0, 16));
     }
     *out = f;
+    return TN_OK;
+}
+
+// End of a single contraction: wait for its stream; `err` (tensor-core
+// kernels): the flag of a wait that gave up, read behind the kernels.
+static tn_status finish_call(cudaStream_t st, int *err) {
+    int herr = 0;
+    if (err) CK(cudaMemcpyAsync(&herr, err, 4, cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    if (herr) {
+        CK(cudaMemset(err, 0, 4));
+        return fail(TN_E_TIMEOUT, "a device-side wait exceeded its time limit");
+    }
     return TN_OK;
 }
 
@@ -4032,10 +4145,6 @@ tn_status tn_contract_dev(int nlabels, const int *sizes, int na, const int *labe
             std::string e = make_gemm_op(card, 1, store_t, gemm_t, X, Y, bt, gm, gn, gk, lc, false,
                                          C, nullptr, op, nx, ny, nd);
             if (!e.empty()) return fail(TN_E_UNSUPPORTED, e);
-            void *wx = nullptr, *wy = nullptr, *wd = nullptr;
-            CK(cudaMallocAsync(&wx, nx, st));
-            CK(cudaMallocAsync(&wy, ny, st));
-            if (nd) CK(cudaMallocAsync(&wd, nd, st));
             // tiled-permutation tables: one device copy for the call
             std::vector<int32_t> tall;
             for (auto pr : {std::make_pair(&op.px, &op.tpx), std::make_pair(&op.py, &op.tpy),
@@ -4045,9 +4154,13 @@ tn_status tn_contract_dev(int nlabels, const int *sizes, int na, const int *labe
                 pr.first->tl.ttab = (const int32_t *)(uintptr_t)tall.size();   // offset for now
                 tall.insert(tall.end(), pr.second->begin(), pr.second->end());
             }
-            int32_t *dtab = nullptr;
+            // one allocation: X, Y and D workspaces and the tables
+            auto r256 = [](size_t v) { return (v + 255) & ~(size_t)255; };
+            CallMem ws(st);
+            CK(ws.alloc(r256(nx) + r256(ny) + r256(nd) + tall.size() * 4));
+            char *wx = (char *)ws.p, *wy = wx + r256(nx), *wd = wy + r256(ny);
+            int32_t *dtab = (int32_t *)(wd + r256(nd));
             if (!tall.empty()) {
-                CK(cudaMallocAsync(&dtab, tall.size() * 4, st));
                 CK(cudaMemcpyAsync(dtab, tall.data(), tall.size() * 4, cudaMemcpyHostToDevice, st));
                 for (PDesc *q : {&op.px, &op.py, &op.post})
                     if (q->tl.tn > 0) q->tl.ttab = dtab + (uintptr_t)q->tl.ttab;
@@ -4073,25 +4186,12 @@ tn_status tn_contract_dev(int nlabels, const int *sizes, int na, const int *labe
             else launch_simt_gemm(op.g, st);
             if (op.has_post) launch_permute(op.post, st);
             cudaError_t e2 = cudaGetLastError();
-            cudaFreeAsync(wx, st);
-            cudaFreeAsync(wy, st);
-            if (wd) cudaFreeAsync(wd, st);
-            if (dtab) {
-                // the pageable source of the table copy must outlive it
-                cudaStreamSynchronize(st);
-                cudaFreeAsync(dtab, st);
-            }
-            if (le != cudaSuccess || e2 != cudaSuccess)
+            if (le != cudaSuccess || e2 != cudaSuccess) {
+                cudaStreamSynchronize(st);   // the table copy reads host memory of this call
                 return fail(TN_E_CUDA, std::string("GEMM launch: ") +
                                            cudaGetErrorString(le != cudaSuccess ? le : e2));
-            CK(cudaStreamSynchronize(st));
-            int herr = 0;
-            CK(cudaMemcpy(&herr, d_err, 4, cudaMemcpyDeviceToHost));
-            if (herr) {
-                CK(cudaMemset(d_err, 0, 4));
-                return fail(TN_E_TIMEOUT, "a device-side wait exceeded its time limit");
             }
-            return TN_OK;
+            return finish_call(st, tc ? d_err : nullptr);
         }
     }
     int es = dtype == 0 ? 8 : 4;
@@ -4099,40 +4199,34 @@ tn_status tn_contract_dev(int nlabels, const int *sizes, int na, const int *labe
     // operand: the batched strided GEMM
     if (semiring == 0) {
         BDesc bd;
+        GroupTabs gt;
         std::vector<int32_t> tab;
         const bool tc_in = prec == TN_TF32 || prec == TN_BF16;
         if (make_bgemm(card, la, false, 0, A, nullptr, lb, false, 0, B, nullptr, lc, false, 0, C,
-                       nullptr, 1, es, bd, tab, tc_in)) {
-            int32_t *dtab = nullptr;
-            void *part = nullptr;
-            size_t pb = bgemm_scratch_bytes(bd, es);
-            CK(cudaMallocAsync(&dtab, tab.size() * 4, st));
-            CK(cudaMemcpyAsync(dtab, tab.data(), tab.size() * 4, cudaMemcpyHostToDevice, st));
+                       nullptr, 1, es, bd, tab, tc_in, &gt)) {
+            if (!tc_in) bd.tc = 0;   // TF32 inputs only when asked
+            const size_t ntab = gt.total ? (size_t)gt.total : tab.size();
+            const size_t tb = (ntab * 4 + 255) & ~(size_t)255;
+            CallMem ws(st);
+            CK(ws.alloc(tb + bgemm_scratch_bytes(bd, es)));
+            int32_t *dtab = (int32_t *)ws.p;
+            void *part = (char *)ws.p + tb;
+            if (gt.total) launch_group_tables(gt, dtab, st);
+            else CK(cudaMemcpyAsync(dtab, tab.data(), ntab * 4, cudaMemcpyHostToDevice, st));
             for (const int32_t **q : {&bd.tag, &bd.tbg, &bd.tcg, &bd.tam, &bd.tcm, &bd.tbn,
                                       &bd.tcn, &bd.tak, &bd.tbk})
                 *q = dtab + (intptr_t)*q;
-            if (pb) CK(cudaMallocAsync(&part, pb, st));
             tn_status fs = device_err_flag(&bd.err);
             if (fs) return fs;
-            if (!tc_in) bd.tc = 0;   // TF32 inputs only when asked
             if (dtype == 0) launch_bgemm<double>(bd, part, st);
             else launch_bgemm<float>(bd, part, st);
             cudaError_t e = cudaGetLastError();
-            // the pageable source of the table copy must outlive it
-            cudaError_t e2 = cudaStreamSynchronize(st);
-            cudaFreeAsync(dtab, st);
-            if (part) cudaFreeAsync(part, st);
-            if (e != cudaSuccess || e2 != cudaSuccess)
-                return fail(TN_E_CUDA, std::string("batched GEMM launch: ") +
-                                           cudaGetErrorString(e != cudaSuccess ? e : e2));
-            CK(cudaStreamSynchronize(st));
-            int herr = 0;
-            CK(cudaMemcpy(&herr, bd.err, 4, cudaMemcpyDeviceToHost));
-            if (herr) {
-                CK(cudaMemset(bd.err, 0, 4));
-                return fail(TN_E_TIMEOUT, "a device-side wait exceeded its time limit");
+            if (e != cudaSuccess) {
+                cudaStreamSynchronize(st);   // a table copy may read host memory of this call
+                return fail(TN_E_CUDA,
+                            std::string("batched GEMM launch: ") + cudaGetErrorString(e));
             }
-            return TN_OK;
+            return finish_call(st, bd.tc ? bd.err : nullptr);
         }
     }
     CDesc d;
@@ -4141,12 +4235,11 @@ tn_status tn_contract_dev(int nlabels, const int *sizes, int na, const int *labe
                                 semiring == 1 ? argmax : nullptr, d);
     if (!err.empty()) return fail(TN_E_UNSUPPORTED, err);
     size_t sb = contract_scratch_bytes(d, es);
-    void *scratch = nullptr;
-    if (sb) CK(cudaMallocAsync(&scratch, sb, st));
-    if (dtype == 0) launch_contract<double>(d, semiring, scratch, sb, st, nullptr);
-    else launch_contract<float>(d, semiring, scratch, sb, st, nullptr);
+    CallMem ws(st);
+    if (sb) CK(ws.alloc(sb));
+    if (dtype == 0) launch_contract<double>(d, semiring, ws.p, sb, st, nullptr);
+    else launch_contract<float>(d, semiring, ws.p, sb, st, nullptr);
     cudaError_t e = cudaGetLastError();
-    if (scratch) cudaFreeAsync(scratch, st);
     if (e != cudaSuccess) return fail(TN_E_CUDA, std::string("contract launch: ") + cudaGetErrorString(e));
     CK(cudaStreamSynchronize(st));
     return TN_OK;

@@ -326,34 +326,28 @@ void plan_permute_tiles(PDesc &p, std::vector<int32_t> &tab) {
     }
     // input offsets [n], output offsets [n], then the 16-bit slots [n]
     tab.assign((size_t)(2 * n + (n + 1) / 2), 0);
-    for (int64_t e = 0; e < n; ++e) {
-        int64_t r = e, off = 0;
-        for (int i : oi) {
-            int64_t dg = r % d[i].sz;
-            r /= d[i].sz;
-            off += dg * d[i].sin;
-        }
-        if (off >= (1LL << 31)) {
-            tab.clear();
-            return;
-        }
-        tab[e] = (int32_t)off;
-    }
     std::vector<int> ein_of((size_t)n);
-    for (int64_t e = 0; e < n; ++e) {
-        int64_t r = e, off = 0, ein = 0;
-        for (int i : oo) {
-            int64_t dg = r % d[i].sz;
-            r /= d[i].sz;
-            off += dg * d[i].sout;
-            ein += dg * wi[i];
+    for (bool by_in : {true, false}) {
+        const std::vector<int> &o = by_in ? oi : oo;
+        std::vector<int64_t> dig(o.size(), 0);
+        int64_t off = 0, ein = 0;
+        for (int64_t e = 0; e < n; ++e) {
+            if (off >= (1LL << 31)) {
+                tab.clear();
+                return;
+            }
+            tab[(by_in ? 0 : n) + e] = (int32_t)off;
+            if (!by_in) ein_of[e] = (int)ein;
+            for (size_t q = 0; q < o.size(); ++q) {
+                const D &x = d[o[q]];
+                off += by_in ? x.sin : x.sout;
+                ein += wi[o[q]];
+                if (++dig[q] < x.sz) break;
+                off -= (by_in ? x.sin : x.sout) * x.sz;
+                ein -= wi[o[q]] * x.sz;
+                dig[q] = 0;
+            }
         }
-        if (off >= (1LL << 31)) {
-            tab.clear();
-            return;
-        }
-        tab[n + e] = (int32_t)off;
-        ein_of[e] = (int)ein;
     }
     PTile &t = p.tl;
     t.nrest = 0;
@@ -416,27 +410,28 @@ void plan_permute_tiles(PDesc &p, std::vector<int32_t> &tab) {
             return esz == 8 ? pt_slot<8>(e, swz) : pt_slot<4>(e, swz);
         };
         int64_t best = -1;
+        const int64_t ideal = (n + 31) / 32 * (esz / 4);   // no conflict anywhere
         std::vector<int> sl((size_t)n);
-        for (int swz = 0; swz < PT_NSWZ; ++swz) {
+        for (int swz = 0; swz < PT_NSWZ && best != ideal; ++swz) {
             for (int64_t e = 0; e < n; ++e) sl[e] = slot_of(ein_of[e], swz);
             int64_t waves = 0;
-            for (int64_t b = 0; b < n; b += 256 * G)
+            for (int64_t b = 0; b < n && (best < 0 || waves < best); b += 256 * G)
                 for (int w = 0; w < 8; ++w)
                     for (int j = 0; j < G; ++j) {
                         // one warp-wide shared load: per bank, the distinct words
-                        int cnt[32] = {0};
-                        int64_t seen[32][32];
+                        int8_t cnt[32] = {0};
+                        int32_t seen[32][32];
+                        int mx = 0;
                         for (int l = 0; l < 32; ++l) {
                             const int64_t e = b + (int64_t)(w * 32 + l) * G + j;
-                            if (e >= n) continue;
-                            const int64_t word = (int64_t)sl[e] * (esz / 4);
-                            const int bank = (int)(word & 31);
+                            if (e >= n) break;
+                            const int32_t word = sl[e] * (esz / 4);
+                            const int bank = word & 31;
                             bool dup = false;
                             for (int k = 0; k < cnt[bank]; ++k) dup = dup || seen[bank][k] == word;
                             if (!dup) seen[bank][cnt[bank]++] = word;
+                            mx = std::max(mx, (int)cnt[bank]);
                         }
-                        int mx = 0;
-                        for (int k = 0; k < 32; ++k) mx = std::max(mx, cnt[k]);
                         waves += mx;
                     }
             if (best < 0 || waves < best) {

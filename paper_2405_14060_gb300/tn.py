@@ -415,10 +415,14 @@ def _contract_args(sizes, la, A, lb, B, lc, C, argmax):
             raise TNError(1, f"{name} has dtype {t.dtype}, A has {A.dtype}")
         if t.device != dev or not t.is_contiguous():
             raise TNError(1, f"{name} must be a contiguous tensor on {dev}")
+    # plain integers: a call's labels are few, and array operations cost microseconds each
+    size = sz.tolist()
     for name, t, l in (("A", A, a), ("B", B, b), ("C", C, c)):
-        if np.any(l < 0) or np.any(l >= len(sz)):
-            raise TNError(1, f"label of {name} out of range")
-        want = int(np.prod([int(sz[v]) for v in l])) if len(l) else 1
+        want = 1
+        for v in l.tolist():
+            if v < 0 or v >= len(size):
+                raise TNError(1, f"label of {name} out of range")
+            want *= size[v]
         if t.numel() != want:
             raise TNError(1, f"{name} has {t.numel()} entries, its labels give {want}")
     if argmax is not None:
