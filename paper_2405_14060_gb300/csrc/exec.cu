@@ -183,7 +183,7 @@ enum Cls { C_SMALL = 0, C_STREAM = 1, C_SPLITK = 2, C_TCGEMM = 3, C_SIMTGEMM = 4
 
 struct GemmOp {
     PDesc px, py, post;
-    std::vector<int32_t> tpx, tpy, tpost;   // tiled-permutation tables (host copies)
+    PTabs tpx{}, tpy{}, tpost{};   // tiled-permutation tables
     bool has_post = false;
     bool direct = false;
     bool x_in_place = false;   // X already in GEMM form: read in place, its scale in the epilogue
@@ -2331,7 +2331,8 @@ tn_status build_program(tn_model *m, const Net &net, const Tree &tree, int kind,
                         if (pr.first->tl.tn <= 0) continue;
                         all.resize((all.size() + 3) & ~(size_t)3);   // 16-byte aligned
                         pwhere.push_back({pr.first, all.size()});
-                        all.insert(all.end(), pr.second->begin(), pr.second->end());
+                        all.resize(all.size() + pr.second->words());
+                        fill_permute_table(*pr.second, &all[pwhere.back().second]);
                     }
                     continue;
                 }
@@ -4145,30 +4146,34 @@ tn_status tn_contract_dev(int nlabels, const int *sizes, int na, const int *labe
             std::string e = make_gemm_op(card, 1, store_t, gemm_t, X, Y, bt, gm, gn, gk, lc, false,
                                          C, nullptr, op, nx, ny, nd);
             if (!e.empty()) return fail(TN_E_UNSUPPORTED, e);
-            // tiled-permutation tables: one device copy for the call
-            std::vector<int32_t> tall;
-            for (auto pr : {std::make_pair(&op.px, &op.tpx), std::make_pair(&op.py, &op.tpy),
-                            std::make_pair(&op.post, &op.tpost)}) {
-                if (pr.first->tl.tn <= 0) continue;
-                tall.resize((tall.size() + 3) & ~(size_t)3);   // 16-byte aligned
-                pr.first->tl.ttab = (const int32_t *)(uintptr_t)tall.size();   // offset for now
-                tall.insert(tall.end(), pr.second->begin(), pr.second->end());
-            }
-            // one allocation: X, Y and D workspaces and the tables
+            // an operand already in GEMM form ([batch][rows][K] in the GEMM's
+            // type) is read in place
+            const bool xin = op.x_in_place;
+            const bool yin = op.py.nd == 1 && op.py.sin[0] == 1 && op.py.sout[0] == 1 &&
+                             op.g.K == op.g.ldy && store_t == gemm_t && ((uintptr_t)B & 15) == 0;
+            if (xin) op.tpx.n = 0;
+            if (yin) op.tpy.n = 0;
+            // one allocation: X, Y and D workspaces and the permutation tables
             auto r256 = [](size_t v) { return (v + 255) & ~(size_t)255; };
+            const size_t bx = xin ? 0 : r256(nx), by = yin ? 0 : r256(ny), bd = r256(nd);
+            PTabs3 pt{{op.tpx, op.tpy, op.tpost}, {nullptr, nullptr, nullptr}};
             CallMem ws(st);
-            CK(ws.alloc(r256(nx) + r256(ny) + r256(nd) + tall.size() * 4));
-            char *wx = (char *)ws.p, *wy = wx + r256(nx), *wd = wy + r256(ny);
-            int32_t *dtab = (int32_t *)(wd + r256(nd));
-            if (!tall.empty()) {
-                CK(cudaMemcpyAsync(dtab, tall.data(), tall.size() * 4, cudaMemcpyHostToDevice, st));
-                for (PDesc *q : {&op.px, &op.py, &op.post})
-                    if (q->tl.tn > 0) q->tl.ttab = dtab + (uintptr_t)q->tl.ttab;
+            size_t total = bx + by + bd;
+            for (auto &t : pt.t) total += r256(t.words() * 4);
+            CK(ws.alloc(total));
+            char *wx = (char *)ws.p, *wy = wx + bx, *wd = wy + by, *at = wd + bd;
+            PDesc *pd[3] = {&op.px, &op.py, &op.post};
+            for (int i = 0; i < 3; ++i) {
+                if (pt.t[i].n == 0) continue;
+                pt.out[i] = (int32_t *)at;
+                pd[i]->tl.ttab = pt.out[i];
+                at += r256(pt.t[i].words() * 4);
             }
+            launch_permute_tables(pt, st);
             op.px.out = wx;
             op.py.out = wy;
-            op.g.X = wx;
-            op.g.Y = wy;
+            op.g.X = xin ? A : wx;
+            op.g.Y = yin ? B : wy;
             if (op.has_post) {
                 op.g.D = wd;
                 op.post.in = wd;
@@ -4179,18 +4184,16 @@ tn_status tn_contract_dev(int nlabels, const int *sizes, int na, const int *labe
                 tn_status fs = device_err_flag(&d_err);
                 if (fs) return fs;
             }
-            launch_permute(op.px, st);
-            launch_permute(op.py, st);
+            if (!xin) launch_permute(op.px, st);
+            if (!yin) launch_permute(op.py, st);
             cudaError_t le = cudaSuccess;
             if (tc) le = launch_tc_gemm(op.g, d_err, st);
             else launch_simt_gemm(op.g, st);
             if (op.has_post) launch_permute(op.post, st);
             cudaError_t e2 = cudaGetLastError();
-            if (le != cudaSuccess || e2 != cudaSuccess) {
-                cudaStreamSynchronize(st);   // the table copy reads host memory of this call
+            if (le != cudaSuccess || e2 != cudaSuccess)
                 return fail(TN_E_CUDA, std::string("GEMM launch: ") +
                                            cudaGetErrorString(le != cudaSuccess ? le : e2));
-            }
             return finish_call(st, tc ? d_err : nullptr);
         }
     }

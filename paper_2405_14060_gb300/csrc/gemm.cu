@@ -253,9 +253,9 @@ __global__ void __launch_bounds__(256, 4) k_permute_tiled(const __grid_constant_
     if (p.mxo) block_max_atomic(p.mxo + item, (double)mxv);
 }
 
-void plan_permute_tiles(PDesc &p, std::vector<int32_t> &tab) {
+void plan_permute_tiles(PDesc &p, PTabs &pt) {
     p.tl.tn = 0;
-    tab.clear();
+    pt.n = 0;
     if (p.nd < 2 || p.total < 8192 || p.total / 64 >= (1LL << 31)) return;
     struct D { int64_t sz, sin, sout; bool beta; };
     std::vector<D> d;
@@ -324,30 +324,13 @@ void plan_permute_tiles(PDesc &p, std::vector<int32_t> &tab) {
             w *= d[i].sz;
         }
     }
-    // input offsets [n], output offsets [n], then the 16-bit slots [n]
-    tab.assign((size_t)(2 * n + (n + 1) / 2), 0);
-    std::vector<int> ein_of((size_t)n);
-    for (bool by_in : {true, false}) {
-        const std::vector<int> &o = by_in ? oi : oo;
-        std::vector<int64_t> dig(o.size(), 0);
-        int64_t off = 0, ein = 0;
-        for (int64_t e = 0; e < n; ++e) {
-            if (off >= (1LL << 31)) {
-                tab.clear();
-                return;
-            }
-            tab[(by_in ? 0 : n) + e] = (int32_t)off;
-            if (!by_in) ein_of[e] = (int)ein;
-            for (size_t q = 0; q < o.size(); ++q) {
-                const D &x = d[o[q]];
-                off += by_in ? x.sin : x.sout;
-                ein += wi[o[q]];
-                if (++dig[q] < x.sz) break;
-                off -= (by_in ? x.sin : x.sout) * x.sz;
-                ein -= wi[o[q]] * x.sz;
-                dig[q] = 0;
-            }
+    {
+        int64_t mi = 0, mo = 0;
+        for (int i : U) {
+            mi += (d[i].sz - 1) * d[i].sin;
+            mo += (d[i].sz - 1) * d[i].sout;
         }
+        if (mi >= (1LL << 31) || mo >= (1LL << 31) || U.size() > (size_t)MAXD) return;
     }
     PTile &t = p.tl;
     t.nrest = 0;
@@ -355,10 +338,7 @@ void plan_permute_tiles(PDesc &p, std::vector<int32_t> &tab) {
     t.ntiles = 1;
     for (int i = 0; i < (int)d.size(); ++i) {
         if (in_u[i]) continue;
-        if (t.nrest >= MAXD) {
-            tab.clear();
-            return;
-        }
+        if (t.nrest >= MAXD) return;
         if (d[i].beta) t.rest_beta = t.nrest;
         t.rsz[t.nrest] = (int32_t)d[i].sz;
         t.rsh[t.nrest] = (d[i].sz & (d[i].sz - 1)) ? -1 : __builtin_ctzll((unsigned long long)d[i].sz);
@@ -368,81 +348,131 @@ void plan_permute_tiles(PDesc &p, std::vector<int32_t> &tab) {
         ++t.nrest;
     }
     // per-item maxima need the batch dim outermost (one item per grid row)
-    if ((p.mxo && t.rest_beta > 0) || t.ntiles >= (1LL << 31)) {
-        tab.clear();
-        return;
-    }
+    if ((p.mxo && t.rest_beta > 0) || t.ntiles >= (1LL << 31)) return;
     t.tn = (int)n;
-    t.ttab = nullptr;   // device copy of `tab`, set by the caller
-    // 16-byte stores: every aligned group of G output-ordered entries is
-    // contiguous and starts on a multiple of G elements in every tile
-    t.vec = 0;
-    {
-        const int G = p.out_type == E_F64 ? 2 : p.out_type == E_F32 ? 4 : 8;
-        bool ok = n % G == 0;
-        for (int64_t e0 = 0; ok && e0 < n; e0 += G) {
-            const int32_t o = tab[n + e0];
-            ok = o % G == 0;
-            for (int j = 1; ok && j < G; ++j) ok = tab[n + e0 + j] == o + j;
-        }
-        for (int k = 0; ok && k < t.nrest; ++k) ok = t.rout[k] % G == 0;
-        if (ok) t.vec = G;
+    t.ttab = nullptr;   // device table, set by the caller
+    pt.n = (int)n;
+    pt.esz = p.in_type == E_F64 ? 8 : 4;
+    pt.ni = pt.no = (int)U.size();
+    for (int q = 0; q < pt.ni; ++q) {
+        pt.isz[q] = (int32_t)d[oi[q]].sz;
+        pt.ioff[q] = (int32_t)d[oi[q]].sin;
+        pt.osz[q] = (int32_t)d[oo[q]].sz;
+        pt.ooff[q] = (int32_t)d[oo[q]].sout;
+        pt.oin[q] = (int32_t)wi[oo[q]];
     }
-    // 16-byte input copies: the same condition on the input-ordered entries
-    t.vin = 0;
+    // 16-byte stores / input copies of G entries: every aligned group of G
+    // entries (in output / input order) is contiguous and starts on a multiple
+    // of G elements in every tile, that is, the contiguous run of the fastest
+    // digits holds a multiple of G entries and every other stride is one
+    auto groups = [&](int G, const int32_t *sz, const int32_t *off, int nd, const int64_t *rest) {
+        if (n % G) return 0;
+        int64_t run = 1;
+        int q = 0;
+        while (q < nd && off[q] == run) run *= sz[q++];
+        if (run % G) return 0;
+        for (; q < nd; ++q)
+            if (off[q] % G) return 0;
+        for (int k = 0; k < t.nrest; ++k)
+            if (rest[k] % G) return 0;
+        return G;
+    };
+    t.vec = groups(p.out_type == E_F64 ? 2 : p.out_type == E_F32 ? 4 : 8, pt.osz, pt.ooff, pt.no,
+                   t.rout);
+    t.vin = groups(p.in_type == E_F64 ? 2 : 4, pt.isz, pt.ioff, pt.ni, t.rin);
+    // shared-memory layout: the one whose reads of a tile (output order, t.vec
+    // entries per thread, or one) take the fewest wavefronts, counted on 16
+    // warp-wide loads spread over the tile (all of a full tile's 128 cost 100 us
+    // a permutation, more than it takes to run)
     {
-        const int G = p.in_type == E_F64 ? 2 : 4;
-        bool ok = n % G == 0;
-        for (int64_t e0 = 0; ok && e0 < n; e0 += G) {
-            const int32_t o = tab[e0];
-            ok = o % G == 0;
-            for (int j = 1; ok && j < G; ++j) ok = tab[e0 + j] == o + j;
-        }
-        for (int k = 0; ok && k < t.nrest; ++k) ok = t.rin[k] % G == 0;
-        if (ok) t.vin = G;
-    }
-    // shared-memory layout: the one whose reads of a tile (output order,
-    // t.vec entries per thread, or one) take the fewest wavefronts
-    {
-        const int esz = p.in_type == E_F64 ? 8 : 4;
         const int G = t.vec > 0 ? t.vec : 1;
-        auto slot_of = [&](int e, int swz) {
-            return esz == 8 ? pt_slot<8>(e, swz) : pt_slot<4>(e, swz);
-        };
-        int64_t best = -1;
-        const int64_t ideal = (n + 31) / 32 * (esz / 4);   // no conflict anywhere
-        std::vector<int> sl((size_t)n);
-        for (int swz = 0; swz < PT_NSWZ && best != ideal; ++swz) {
-            for (int64_t e = 0; e < n; ++e) sl[e] = slot_of(ein_of[e], swz);
-            int64_t waves = 0;
-            for (int64_t b = 0; b < n && (best < 0 || waves < best); b += 256 * G)
-                for (int w = 0; w < 8; ++w)
-                    for (int j = 0; j < G; ++j) {
-                        // one warp-wide shared load: per bank, the distinct words
-                        int8_t cnt[32] = {0};
-                        int32_t seen[32][32];
-                        int mx = 0;
-                        for (int l = 0; l < 32; ++l) {
-                            const int64_t e = b + (int64_t)(w * 32 + l) * G + j;
-                            if (e >= n) break;
-                            const int32_t word = sl[e] * (esz / 4);
-                            const int bank = word & 31;
-                            bool dup = false;
-                            for (int k = 0; k < cnt[bank]; ++k) dup = dup || seen[bank][k] == word;
-                            if (!dup) seen[bank][cnt[bank]++] = word;
-                            mx = std::max(mx, (int)cnt[bank]);
-                        }
-                        waves += mx;
-                    }
+        const int nload = ((int)n + 31) / 32, step = std::max(1, nload / 16);
+        int ein[32][32], lanes[32], ns = 0;   // input index of every sampled lane
+        for (int w = 0; w < nload && ns < 32; w += step, ++ns) {
+            // load w: the 32 lanes of warp w / G, entry w % G of each
+            int l = 0;
+            for (; l < 32; ++l) {
+                int r = ((w / G) * 32 + l) * G + w % G, x = 0;
+                if (r >= (int)n) break;
+                for (int q = 0; q < pt.no; ++q) {
+                    const int y = r / pt.osz[q];
+                    x += (r - y * pt.osz[q]) * pt.oin[q];
+                    r = y;
+                }
+                ein[ns][l] = x;
+            }
+            lanes[ns] = l;
+        }
+        int best = -1;
+        for (int swz = 0; swz < PT_NSWZ; ++swz) {
+            int waves = 0;
+            for (int w = 0; w < ns; ++w) {
+                int8_t cnt[32] = {0};
+                int32_t seen[32][32];
+                int mx = 0;
+                for (int l = 0; l < lanes[w]; ++l) {
+                    const int slot = pt.esz == 8 ? pt_slot<8>(ein[w][l], swz)
+                                                 : pt_slot<4>(ein[w][l], swz);
+                    const int32_t word = slot * (pt.esz / 4);
+                    const int bank = word & 31;
+                    bool dup = false;   // per bank, the distinct words
+                    for (int k = 0; k < cnt[bank]; ++k) dup = dup || seen[bank][k] == word;
+                    if (!dup) seen[bank][cnt[bank]++] = word;
+                    mx = std::max(mx, (int)cnt[bank]);
+                }
+                waves += mx;
+            }
             if (best < 0 || waves < best) {
                 best = waves;
                 t.swz = swz;
             }
+            if (best <= ns * (pt.esz / 4)) break;   // no conflict anywhere
         }
         t.nbuf = pt_nbuf((int)n, t.swz);
-        uint16_t *s16 = (uint16_t *)(tab.data() + 2 * n);
-        for (int64_t e = 0; e < n; ++e) s16[e] = (uint16_t)slot_of(ein_of[e], t.swz);
+        pt.swz = t.swz;
     }
+}
+
+// Table entry e: input offset, output offset, shared-memory slot of the e-th
+// output.
+__host__ __device__ inline void permute_entry(const PTabs &t, int e, int32_t &in, int32_t &out,
+                                              uint16_t &slot) {
+    int r = e;
+    in = 0;
+    for (int q = 0; q < t.ni; ++q) {
+        const int x = r / t.isz[q];
+        in += (r - x * t.isz[q]) * t.ioff[q];
+        r = x;
+    }
+    r = e;
+    out = 0;
+    int ein = 0;
+    for (int q = 0; q < t.no; ++q) {
+        const int x = r / t.osz[q], dg = r - x * t.osz[q];
+        out += dg * t.ooff[q];
+        ein += dg * t.oin[q];
+        r = x;
+    }
+    slot = (uint16_t)(t.esz == 8 ? pt_slot<8>(ein, t.swz) : pt_slot<4>(ein, t.swz));
+}
+
+void fill_permute_table(const PTabs &t, int32_t *out) {
+    uint16_t *slot = (uint16_t *)(out + 2 * t.n);
+    for (int e = 0; e < t.n; ++e) permute_entry(t, e, out[e], out[t.n + e], slot[e]);
+}
+
+__global__ void __launch_bounds__(256) k_permute_tables(const __grid_constant__ PTabs3 a) {
+    const PTabs &t = a.t[blockIdx.y];
+    const int e = blockIdx.x * 256 + threadIdx.x;
+    if (e >= t.n) return;
+    int32_t *out = a.out[blockIdx.y];
+    permute_entry(t, e, out[e], out[t.n + e], ((uint16_t *)(out + 2 * t.n))[e]);
+}
+
+void launch_permute_tables(const PTabs3 &a, cudaStream_t st) {
+    int n = 0;
+    for (auto &t : a.t) n = std::max(n, t.n);
+    if (n > 0) k_permute_tables<<<dim3((unsigned)((n + 255) / 256), 3), 256, 0, st>>>(a);
 }
 
 void launch_permute(const PDesc &p, cudaStream_t st) {

@@ -79,9 +79,27 @@ struct PDesc {
     PTile tl;
 };
 
+// A tile's table as digits (fastest first) in the input's and in the output's
+// order: sizes, offsets, and for the output's the weight in the input order.
+struct PTabs {
+    int n, swz, esz, ni, no;
+    int32_t isz[MAXD], ioff[MAXD];
+    int32_t osz[MAXD], ooff[MAXD], oin[MAXD];
+    size_t words() const { return (size_t)(2 * n + (n + 1) / 2); }
+};
+
 // Choose the tiled form for p when it pays (host): fills p.tl (but for the
-// device table pointer) and the table; leaves p.tl.tn = 0 otherwise.
-void plan_permute_tiles(PDesc &p, std::vector<int32_t> &tab);
+// device table pointer) and the table's digits; leaves p.tl.tn = t.n = 0
+// otherwise.
+void plan_permute_tiles(PDesc &p, PTabs &t);
+// The tables from their digits: on the host (programs, once), or on the device
+// for up to three permutations of a call (out[i] unused where t[i].n = 0).
+void fill_permute_table(const PTabs &t, int32_t *out);
+struct PTabs3 {
+    PTabs t[3];
+    int32_t *out[3];
+};
+void launch_permute_tables(const PTabs3 &t, cudaStream_t st);
 
 // D[b][r][c] = sum_k X[b][r][k] * Y[b][c][k]   (X, Y K-major, D row-major FP32/FP64)
 struct GDesc {
