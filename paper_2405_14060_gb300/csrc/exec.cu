@@ -4071,6 +4071,12 @@ static tn_status device_err_flag(int **out) {
     return TN_OK;
 }
 
+// CUDA-core GEMM tiles that leave half of the SMs idle while each sums at least
+// 256 terms.
+static bool few_gemm_tiles(int64_t batch, int64_t rows, int64_t cols, int64_t k) {
+    return k >= 256 && (double)((rows + 63) / 64) * (double)((cols + 63) / 64) * (double)batch < 76;
+}
+
 // End of a single contraction: wait for its stream; `err` (tensor-core
 // kernels): the flag of a wait that gave up, read behind the kernels.
 static tn_status finish_call(cudaStream_t st, int *err) {
@@ -4134,8 +4140,12 @@ tn_status tn_contract_dev(int nlabels, const int *sizes, int na, const int *labe
             return q;
         };
         // FP64 within the batched GEMM's index ranges runs on its direct form
-        // below, in place
-        const bool direct = dtype == 0 && prod(la) < (1LL << 31) && prod(lb) < (1LL << 31) &&
+        // below, in place; so does FP32 with few tiles and a summed space that
+        // the batched GEMM splits over blocks (100 x 130 x 4000: 6 tiles, 286 us
+        // a call on the tiled GEMM, 73 there)
+        const bool tcp = prec == TN_TF32 || prec == TN_BF16;
+        const bool direct = (dtype == 0 || (!tcp && few_gemm_tiles(prod(bt), prod(gm), prod(gn),
+                                                                   prod(gk)))) && prod(la) < (1LL << 31) && prod(lb) < (1LL << 31) &&
                             prod(lc) < (1LL << 31);
         if (!direct && !onesided && prod(gm) >= 64 && prod(gn) >= 64 && prod(gk) >= 64) {
             int store_t = dtype == 0 ? E_F64 : E_F32;

@@ -948,10 +948,179 @@ __global__ void __launch_bounds__(256) k_simt_gemm(const __grid_constant__ GDesc
     record_max(g.mxd, beta, any, (double)mx);
 }
 
+// FP32 form: BM x BN tiles, eight warps, K steps of 16 through two shared
+// buffers (global loads of the next step in registers while the current one is
+// multiplied), TM x TN outputs a thread as pairs of rows (fma.rn.f32x2: two
+// multiply-adds an instruction, so that shared loads and address work issue
+// beside them).  A warp covers 4 x 8 lanes of quads without bank conflicts.
+// Bound by the shared-memory pipe for small thread tiles (a word per lane and
+// clock: 8 x 4 outputs take 12 clocks of loads for 8 of multiply-adds, 8 x 8 take
+// 16 for 16, 12 x 8 take 20 for 24), else by the FP32 pipe.  2048 x 1536 x 1024:
+// 316 us with 4 x 4 outputs a thread and scalar shared loads, 150 us
+// now (192 x 128 tiles; 163 with 128 x 64, 192 with 128 x 128, 219 with 64 x 64).
+__device__ __forceinline__ void unpack2(uint64_t v, float &lo, float &hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t dup2(float v) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ void fma2(uint64_t &d, uint64_t a, uint64_t b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+
+template <int BM, int BN, int TM, int TN>
+__global__ void __launch_bounds__(256, TM * TN > 64 ? 1 : 2) k_sgemm(const __grid_constant__ GDesc g) {
+    constexpr int BK = 16, LX = BM + 4, LY = BN + 4;
+    constexpr int QM = TM / 4, QN = TN / 4;          // quads a thread holds each way
+    constexpr int WM = BM / 4, WN = BN / 2;          // a warp's rows and columns
+    static_assert(QM * 16 == WM && QN * 32 == WN, "warp tile");
+    constexpr int LXN = BM / 64, LYN = BN / 64;      // 16-byte loads a thread and step
+    __shared__ __align__(16) float sx[2][BK][LX];
+    __shared__ __align__(16) float sy[2][BK][LY];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t ntn = (g.C + BN - 1) / BN, ntm = (g.R + BM - 1) / BM;
+    const int64_t b = (int64_t)blockIdx.x / (ntn * ntm), rem = (int64_t)blockIdx.x - b * ntn * ntm;
+    const int64_t r0 = (rem / ntn) * BM, c0 = (rem % ntn) * BN;
+    const int q = tid & 3, lr = tid >> 2;            // K quad and row of this thread's loads
+    const float *xp[LXN], *yp[LYN];
+#pragma unroll
+    for (int i = 0; i < LXN; ++i)
+        xp[i] = (const float *)g.X + b * g.bsx + min(r0 + lr + 64 * i, g.R - 1) * g.ldx + 4 * q;
+#pragma unroll
+    for (int i = 0; i < LYN; ++i)
+        yp[i] = (const float *)g.Y + b * g.bsy + min(c0 + lr + 64 * i, g.C - 1) * g.ldy + 4 * q;
+    const int K = (int)g.K, nk = (K + BK - 1) / BK;
+    float4 vx[LXN], vy[LYN];
+    // entries past K are zero (the padding of a row is not written); K is
+    // padded to a multiple of 8 in memory, so quads never leave the row
+    auto load = [&](int ks) {
+        const int k = ks * BK + 4 * q;
+#pragma unroll
+        for (int i = 0; i < LXN + LYN; ++i) {
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (k < K) {
+                v = __ldg((const float4 *)((i < LXN ? xp[i < LXN ? i : 0] : yp[i < LXN ? 0 : i - LXN]) +
+                                           ks * BK));
+                if (k + 1 >= K) v.y = 0.f;
+                if (k + 2 >= K) v.z = 0.f;
+                if (k + 3 >= K) v.w = 0.f;
+            }
+            if (i < LXN) vx[i < LXN ? i : 0] = v;
+            else vy[i < LXN ? 0 : i - LXN] = v;
+        }
+    };
+    auto store = [&](int s) {
+#pragma unroll
+        for (int i = 0; i < LXN; ++i) {
+            const float *v = (const float *)&vx[i];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) sx[s][4 * q + j][lr + 64 * i] = v[j];
+        }
+#pragma unroll
+        for (int i = 0; i < LYN; ++i) {
+            const float *v = (const float *)&vy[i];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) sy[s][4 * q + j][lr + 64 * i] = v[j];
+        }
+    };
+    const int tm = (warp >> 1) * WM + (lane >> 3) * 4;   // first row quad; the others 16 rows on
+    const int tn = (warp & 1) * WN + (lane & 7) * 4;     // first column quad; the others 32 on
+    uint64_t acc[TM / 2][TN];   // rows 2i, 2i + 1
+#pragma unroll
+    for (int i = 0; i < TM / 2; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) acc[i][j] = 0ull;
+    load(0);
+    store(0);
+    __syncthreads();
+    for (int ks = 0; ks < nk; ++ks) {
+        const int s = ks & 1;
+        if (ks + 1 < nk) load(ks + 1);
+#pragma unroll
+        for (int k = 0; k < BK; ++k) {
+            uint64_t a[TM / 2];
+            float y[TN];
+#pragma unroll
+            for (int i = 0; i < QM; ++i)
+                *(ulonglong2 *)(a + 2 * i) = *(const ulonglong2 *)&sx[s][k][tm + 16 * i];
+#pragma unroll
+            for (int j = 0; j < QN; ++j)
+                *(float4 *)(y + 4 * j) = *(const float4 *)&sy[s][k][tn + 32 * j];
+#pragma unroll
+            for (int j = 0; j < TN; ++j) {
+                const uint64_t yy = dup2(y[j]);
+#pragma unroll
+                for (int i = 0; i < TM / 2; ++i) fma2(acc[i][j], a[i], yy);
+            }
+        }
+        if (ks + 1 < nk) store(s ^ 1);
+        __syncthreads();
+    }
+    float *D = (float *)g.D + b * g.bsd;
+    const float sxs = g.mxsx ? pow2neg<float>(exp_of_bits(*g.mxsx)) : 1.f;
+    const bool vec = (g.ldd & 3) == 0 && (g.bsd & 3) == 0 && ((uintptr_t)g.D & 15) == 0;
+    float mxall = 0.f;
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+        const int64_t r = r0 + tm + (i >> 2) * 16 + (i & 3);
+        float mx = 0.f;
+#pragma unroll
+        for (int j = 0; j < QN; ++j) {
+            const int64_t c = c0 + tn + 32 * j;
+            float v[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                float lo, hi;
+                unpack2(acc[i >> 1][4 * j + e], lo, hi);
+                v[e] = ((i & 1) ? hi : lo) * sxs;
+            }
+            if (r >= g.R) continue;
+            if (vec && c + 4 <= g.C) {
+                *(float4 *)(D + r * g.ldd + c) = make_float4(v[0], v[1], v[2], v[3]);
+                mx = fmaxf(mx, fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])));
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (c + e < g.C) {
+                        D[r * g.ldd + c + e] = v[e];
+                        mx = fmaxf(mx, v[e]);
+                    }
+            }
+        }
+        // rows of one tile may belong to different items
+        if (g.mxd && g.beta_div_batch <= 0 && g.beta_div_row > 0)
+            record_max(g.mxd, min(r, g.R - 1) / g.beta_div_row, r < g.R, (double)mx);
+        else
+            mxall = fmaxf(mxall, mx);
+    }
+    if (g.mxd && (g.beta_div_batch > 0 || g.beta_div_row <= 0))
+        record_max(g.mxd, g.beta_div_batch > 0 ? b / g.beta_div_batch : 0, true, (double)mxall);
+}
+
+template <int BM, int BN>
+static int64_t sgemm_tiles(const GDesc &g) {
+    return ((g.C + BN - 1) / BN) * ((g.R + BM - 1) / BM) * g.batch;
+}
 void launch_simt_gemm(const GDesc &g, cudaStream_t st) {
-    dim3 grid((unsigned)(((g.C + 63) / 64) * ((g.R + 63) / 64) * g.batch), 1, 1);
-    if (g.xtype == E_F64) k_simt_gemm<double><<<grid, 256, 0, st>>>(g);
-    else k_simt_gemm<float><<<grid, 256, 0, st>>>(g);
+    if (g.xtype == E_F64) {
+        dim3 grid((unsigned)(((g.C + 63) / 64) * ((g.R + 63) / 64) * g.batch), 1, 1);
+        k_simt_gemm<double><<<grid, 256, 0, st>>>(g);
+        return;
+    }
+    // the tile whose busiest SM has the least work: tiles per SM, rounded up,
+    // times a tile's outputs, over the share of the FP32 rate it reaches
+    const int64_t t0 = sgemm_tiles<192, 128>(g), t1 = sgemm_tiles<128, 128>(g),
+                  t2 = sgemm_tiles<128, 64>(g), t3 = sgemm_tiles<64, 64>(g);
+    auto cost = [](int64_t t, int out, double rate) { return (double)((t + 151) / 152) * out / rate; };
+    const double c0 = cost(t0, 192 * 128, 0.73), c1 = cost(t1, 128 * 128, 0.76),
+                 c2 = cost(t2, 128 * 64, 0.67), c3 = cost(t3, 64 * 64, 0.5);
+    const double c = std::min(std::min(c0, c1), std::min(c2, c3));
+    if (c == c0) k_sgemm<192, 128, 12, 8><<<(unsigned)t0, 256, 0, st>>>(g);
+    else if (c == c1) k_sgemm<128, 128, 8, 8><<<(unsigned)t1, 256, 0, st>>>(g);
+    else if (c == c2) k_sgemm<128, 64, 8, 4><<<(unsigned)t2, 256, 0, st>>>(g);
+    else k_sgemm<64, 64, 4, 4><<<(unsigned)t3, 256, 0, st>>>(g);
 }
 
 }  // namespace tn

@@ -118,3 +118,24 @@ def test_direct_fp64(m, n, k, spec):
                     [letters.index(l) for l in c], C)
     # positive terms: every order of summation is within k ulp
     np.testing.assert_allclose(C.cpu().numpy(), ref, rtol=k * 2.3e-16 + 1e-15, atol=0)
+
+
+# FP32 GEMM: one tile of every shape and several, ragged rows, columns and
+# summed space, operands already in GEMM form, split long summed spaces
+@pytest.mark.parametrize("m,n,k", [(64, 64, 64), (65, 70, 77), (193, 129, 96), (1000, 900, 130),
+                                   (2500, 2000, 64), (100, 130, 3000)])
+@pytest.mark.parametrize("spec", ["mk,nk->mn", "km,kn->nm", "gmk,gkn->gmn"])
+def test_gemm_fp32_tiles(m, n, k, spec):
+    (a, b), c = spec.split("->")[0].split(","), spec.split("->")[1]
+    letters = "gkmn"
+    size = dict(g=2, k=k, m=m, n=n)
+    rng = np.random.default_rng(m + n * k)
+    A = rng.random([size[l] for l in a]).astype(np.float32)
+    B = rng.random([size[l] for l in b]).astype(np.float32)
+    ref = torch.einsum(spec, torch.tensor(A).cuda().double(), torch.tensor(B).cuda().double())
+    C = torch.full([size[l] for l in c], float("nan"), dtype=torch.float32, device="cuda")
+    tn.contract_dev([size[l] for l in letters], [letters.index(l) for l in a], torch.tensor(A).cuda(),
+                    [letters.index(l) for l in b], torch.tensor(B).cuda(),
+                    [letters.index(l) for l in c], C, prec="fp32")
+    err = ((C.double() - ref).abs() / ref).max().item()
+    assert err <= (k + 1) * 6e-8
