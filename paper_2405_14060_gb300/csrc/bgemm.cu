@@ -2,16 +2,19 @@
 // or summed group is too small for the tensor-core tiles and whose operands
 // are both too large to stream against a small one (bgemm.cuh).
 //
-//   k_bgemm      persistent blocks (a few per SM), each walking its share of
+//   k_bgemm      FP32: persistent blocks (two per SM), each walking its share of
 //                the output tiles (item, g, m tile, n tile, K split).  The A and
 //                B tiles are gathered through the offset tables straight into
-//                shared memory by asynchronous copies, kStages K steps ahead
-//                of the multiply-adds; the pipeline runs across tile
-//                boundaries, so short summed spaces (K of 8 to 32, common in
-//                evidence-batched trees) still keep the memory system busy.
-//                Each thread holds a TM x TN register tile whose rows and
-//                columns are strided by the thread grid, so that consecutive
-//                lanes store consecutive entries along C's fastest group.
+//                shared memory by asynchronous copies (of 4, 2 or 1 floats, as
+//                the operand's contiguous runs allow), kStages - 1 K steps ahead
+//                of the multiply-adds; the pipeline runs across tile boundaries,
+//                so short summed spaces (K of 8 to 32, common in evidence-batched
+//                trees) still keep the memory system busy.  Shapes of the
+//                batched workload (us before, with scalar shared loads and
+//                copies, and now; entries 2^27 + 2^10): rows 2^20, 128 columns,
+//                8 summed 291 / 171; 2^17, 1024, 32 463 / 297; 2^17, 32, 1024
+//                400 / 290; 2^20, 8, 128 327 / 170; 2^18 x 4 rows, 36, 24 271 /
+//                186.
 //   k_bgemm_direct  FP64: a warp computes a strip of
 //                rows times 1, 2 or 4 columns straight from the operands (L1),
 //                without tiles in shared memory.
@@ -82,89 +85,160 @@ __device__ __forceinline__ TilePos direct_pos(const BDesc &d, int64_t t, int MW,
     return p;
 }
 
-template <typename T, int BM, int BN, int TM, int TN, bool NFAST>
+// Asynchronous copy of V floats (1, 2 or 4); zeros when !ok.
+template <int V>
+__device__ __forceinline__ void cp_vec(uint32_t dst, const float *src, bool ok) {
+    const int n = ok ? 4 * V : 0;
+    if constexpr (V == 4)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n)
+                     : "memory");
+    else if constexpr (V == 2)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(n)
+                     : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(n)
+                     : "memory");
+}
+// Packed pairs of floats: d += a * b in both halves (one instruction).
+__device__ __forceinline__ void fma2(uint64_t &d, uint64_t a, uint64_t b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ uint64_t dup2(float v) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float half_of(uint64_t v, int h) {
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+    return h ? hi : lo;
+}
+
+// One operand tile of ROWS rows (of M or N) x kBK summed indices, gathered into
+// one stage of kBK rows of ROWS + 4 floats.  A thread keeps either its rows or
+// its summed index fixed over a step, whichever its operand's fastest label is
+// in, so that neighbouring threads read neighbouring addresses; copies of V
+// floats where the operand's rows run contiguously.
+template <int ROWS, bool REG = true>
+struct Gather {
+    static constexpr int N = (ROWS * kBK + kThreads - 1) / kThreads;   // floats a thread
+    static constexpr int LD = ROWS + 4, SIZE = kBK * LD;
+    // REG: offsets of this thread's rows (one unless summed fastest; -1: none);
+    // else (64 outputs a thread leave no registers) they are looked up every step
+    int32_t off[REG ? N : 1];
+    const int32_t *trow;
+    int left;
+
+    // rows of this thread's copies for a tile starting at row r0
+    __device__ __forceinline__ void rows(const int32_t *t, int64_t nrow, int r0, bool kfast, int v) {
+        if constexpr (!REG) {
+            trow = t + r0;
+            left = (int)min(nrow - r0, (int64_t)ROWS);
+        } else if (kfast) {
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const int r = (int)threadIdx.x / kBK + i * (kThreads / kBK);
+                off[i] = r < ROWS && r0 + r < nrow ? __ldg(t + r0 + r) : -1;
+            }
+        } else {
+            const int r = r0 + (int)threadIdx.x % (ROWS / v) * v;
+            off[0] = r < nrow ? __ldg(t + r) : -1;
+        }
+    }
+    // offset of row r of the tile, this thread's i-th (-1: past the end)
+    __device__ __forceinline__ int32_t row_off(int r, int i) const {
+        if constexpr (REG) return off[i];
+        return r < left ? __ldg(trow + r) : -1;
+    }
+    __device__ __forceinline__ void issue(uint32_t s, const float *base, const int32_t *tk, int k0,
+                                          int kend, int klen, bool kfast, int v) const {
+        if (kfast) {
+            const int kk = (int)threadIdx.x % kBK, k = k0 + kk;
+            if (kk >= klen) return;
+            const bool kok = k < kend;
+            const int32_t ko = kok ? __ldg(tk + k) : 0;
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const int r = (int)threadIdx.x / kBK + i * (kThreads / kBK);
+                if (r >= ROWS) break;
+                const int32_t ro = row_off(r, i);
+                const bool ok = kok && ro >= 0;
+                cp_vec<1>(s + 4u * (uint32_t)(kk * LD + r), ok ? base + (ro + ko) : base, ok);
+            }
+        } else if (v == 4) {
+            along<4>(s, base, tk, k0, kend, klen);
+        } else if (v == 2) {
+            along<2>(s, base, tk, k0, kend, klen);
+        } else {
+            along<1>(s, base, tk, k0, kend, klen);
+        }
+    }
+    template <int V>
+    __device__ __forceinline__ void along(uint32_t s, const float *base, const int32_t *tk, int k0,
+                                          int kend, int klen) const {
+        constexpr int per = ROWS / V, step = kThreads / per;
+        static_assert(step * per == kThreads, "copy grid");
+        const int r = ((int)threadIdx.x % per) * V;
+        const int32_t ro = row_off(r, 0);
+#pragma unroll
+        for (int i = 0; i < (kBK + step - 1) / step; ++i) {
+            const int kk = (int)threadIdx.x / per + i * step;
+            if (kk >= klen) break;
+            const bool ok = ro >= 0 && k0 + kk < kend;
+            cp_vec<V>(s + 4u * (uint32_t)(kk * LD + r),
+                      ok ? base + (ro + __ldg(tk + k0 + kk)) : base, ok);
+        }
+    }
+};
+
+// FP32 kernel: a thread holds TM x TN outputs as pairs of rows (fma.rn.f32x2),
+// rows RQ side by side (4 where C stores quads of rows, else 2, so that a warp's
+// stores of shorter runs still fill sectors together), columns up to 4.  A
+// word of shared memory per lane costs a clock of its pipe, a multiply-add a
+// quarter: 8 x 8 outputs balance the two, 8 x 4 are bound by the loads at 2/3.
+// NFAST: lanes run along C's columns.
+template <int BM, int BN, int TM, int TN, bool NFAST, int RQ>
 __global__ void __launch_bounds__(kThreads, 2)
-    k_bgemm(const __grid_constant__ BDesc d, T *part, int ntiles) {
-    constexpr int MT = BM / TM, NT = BN / TN;
+    k_bgemm(const __grid_constant__ BDesc d, float *part, int ntiles) {
+    constexpr int MT = BM / TM, NT = BN / TN;   // thread grid
     static_assert(MT * NT == kThreads, "thread grid");
-    // loads per thread and stage (B tiles narrower than the thread count:
-    // the threads past the tile copy nothing)
-    constexpr int LA = BM * kBK / kThreads, LB = (BN * kBK + kThreads - 1) / kThreads;
-    static_assert(LA >= 1 && LA * kThreads == BM * kBK, "tile loads");
-    constexpr int RA = BM + 1, RB = BN + 1;              // padded shared rows
-    constexpr int SA = kBK * RA, SB = kBK * RB;          // per stage
-    extern __shared__ __align__(16) unsigned char smraw[];
-    T *As = (T *)smraw;
-    T *Bs = As + kStages * SA;
+    using GA = Gather<BM, (TM * TN < 64)>;
+    using GB = Gather<BN, (TM * TN < 64)>;
+    constexpr int SA = GA::SIZE, SB = GB::SIZE;
+    extern __shared__ __align__(16) float smf[];
+    float *As = smf, *Bs = smf + kStages * SA;
     const int tid = threadIdx.x;
-    const int nks = (d.kchunk + kBK - 1) / kBK;          // K steps per tile
-    const int mine = ntiles > (int)blockIdx.x ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-    // fixed element mapping of this thread's tile loads: summed index within
-    // the stage and shared-memory slot (bytes from the stage's base)
-    int ak[LA], bk[LB], am[LA], bn[LB];
-    bool bv[LB];
-    uint32_t sdA[LA], sdB[LB];
-#pragma unroll
-    for (int r = 0; r < LA; ++r) {
-        const int e = tid + kThreads * r;
-        am[r] = d.a_kfast ? e / kBK : e % BM;
-        ak[r] = d.a_kfast ? e % kBK : e / BM;
-        sdA[r] = (uint32_t)((ak[r] * RA + am[r]) * sizeof(T));
-    }
-#pragma unroll
-    for (int r = 0; r < LB; ++r) {
-        const int e = tid + kThreads * r;
-        bv[r] = e < BN * kBK;
-        bn[r] = bv[r] ? (d.b_kfast ? e / kBK : e % BN) : 0;
-        bk[r] = bv[r] ? (d.b_kfast ? e % kBK : e / BN) : 0;
-        sdB[r] = (uint32_t)((bk[r] * RB + bn[r]) * sizeof(T));
-    }
+    const int nks = (int)((d.kchunk + kBK - 1) / kBK);   // K steps per tile
+    const int mine =
+        ntiles > (int)blockIdx.x ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+    // a last step with at most half of its summed indices: the other half is
+    // neither copied nor multiplied (64 outputs a thread: only where it is also
+    // the first step, for want of registers)
+    constexpr bool TAIL = TM * TN < 64;
+    const int klast = d.nsplit == 1 && d.K - (TAIL ? (int64_t)(nks - 1) * kBK : 0) <= kBK / 2
+                          ? kBK / 2 : kBK;
     const uint32_t sA0 = (uint32_t)__cvta_generic_to_shared(As);
     const uint32_t sB0 = (uint32_t)__cvta_generic_to_shared(Bs);
     // producer state: the tile (local index) and K step being loaded next
-    int p_li = 0, p_ks = 0, p_stage = 0, p_loaded = -1;
-    int p_kbeg = 0, p_kend = 0;
-    const T *pA = (const T *)d.A, *pB = (const T *)d.B;
-    int32_t aoff[LA], boff[LB];
+    int p_li = 0, p_ks = 0, p_stage = 0, p_kbeg = 0, p_kend = 0;
+    const float *pA = (const float *)d.A, *pB = (const float *)d.B;
+    GA ga;
+    GB gb;
     auto issue = [&]() {
         if (p_li < mine) {
-            if (p_li != p_loaded) {
-                p_loaded = p_li;
-                const TilePos tp = tile_pos(d, (int64_t)blockIdx.x + (int64_t)p_li * gridDim.x, BM, BN);
-                pA = (const T *)d.A + tp.beta * d.bsa + __ldg(d.tag + tp.g);
-                pB = (const T *)d.B + tp.beta * d.bsb + __ldg(d.tbg + tp.g);
-                p_kbeg = tp.split * d.kchunk;
-                p_kend = min(d.K, (int64_t)p_kbeg + d.kchunk);
-                const int m0 = (int)tp.m0, n0 = (int)tp.n0;
-#pragma unroll
-                for (int r = 0; r < LA; ++r)
-                    aoff[r] = m0 + am[r] < d.M ? __ldg(d.tam + m0 + am[r]) : -1;
-#pragma unroll
-                for (int r = 0; r < LB; ++r)
-                    boff[r] = n0 + bn[r] < d.N ? __ldg(d.tbn + n0 + bn[r]) : -1;
+            if (p_ks == 0) {
+                const TilePos tp =
+                    tile_pos(d, (int64_t)blockIdx.x + (int64_t)p_li * gridDim.x, BM, BN);
+                pA = (const float *)d.A + tp.beta * d.bsa + __ldg(d.tag + tp.g);
+                pB = (const float *)d.B + tp.beta * d.bsb + __ldg(d.tbg + tp.g);
+                p_kbeg = (int)(tp.split * d.kchunk);
+                p_kend = (int)min(d.K, (int64_t)p_kbeg + d.kchunk);
+                ga.rows(d.tam, d.M, (int)tp.m0, d.a_kfast, d.va);
+                gb.rows(d.tbn, d.N, (int)tp.n0, d.b_kfast, d.vb);
             }
-            const int k0 = p_kbeg + p_ks * kBK;
-            const uint32_t sa = sA0 + (uint32_t)(p_stage * SA * sizeof(T));
-            const uint32_t sb = sB0 + (uint32_t)(p_stage * SB * sizeof(T));
-#pragma unroll
-            for (int r = 0; r < LA; ++r) {
-                const int k = k0 + ak[r];
-                const bool ok = aoff[r] >= 0 && k < p_kend;
-                const T *src = ok ? pA + (aoff[r] + __ldg(d.tak + k)) : pA;
-                asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(sa + sdA[r]),
-                             "l"(src), "n"(sizeof(T)), "r"(ok ? (int)sizeof(T) : 0)
-                             : "memory");
-            }
-#pragma unroll
-            for (int r = 0; r < LB; ++r) {
-                if (!bv[r]) continue;
-                const int k = k0 + bk[r];
-                const bool ok = boff[r] >= 0 && k < p_kend;
-                const T *src = ok ? pB + (boff[r] + __ldg(d.tbk + k)) : pB;
-                asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(sb + sdB[r]),
-                             "l"(src), "n"(sizeof(T)), "r"(ok ? (int)sizeof(T) : 0)
-                             : "memory");
-            }
+            const int k0 = p_kbeg + p_ks * kBK, klen = !TAIL || p_ks == nks - 1 ? klast : kBK;
+            ga.issue(sA0 + (uint32_t)(p_stage * SA * 4), pA, d.tak, k0, p_kend, klen, d.a_kfast, d.va);
+            gb.issue(sB0 + (uint32_t)(p_stage * SB * 4), pB, d.tbk, k0, p_kend, klen, d.b_kfast, d.vb);
             if (++p_ks == nks) {
                 p_ks = 0;
                 ++p_li;
@@ -173,41 +247,57 @@ __global__ void __launch_bounds__(kThreads, 2)
         }
         cp_async_commit();
     };
-    const int im = NFAST ? tid / NT : tid % MT;
-    const int in = NFAST ? tid % NT : tid / MT;
-    T acc[TM][TN];
+    // thread grid: im of MT, in of NT
+    constexpr int LN = NFAST ? (NT < 8 ? NT : 8) : (NT < 4 ? NT : 4);   // lanes along N
+    constexpr int LM = 32 / LN, WM = MT / LM;                           // warps along M
+    static_assert(WM >= 1 && WM * LM == MT, "warp grid");
+    const int lane = tid & 31, warp = tid >> 5;
+    const int ln = NFAST ? lane % LN : lane / LM, lm = NFAST ? lane / LN : lane % LM;
+    const int im = (warp % WM) * LM + lm, in = (warp / WM) * LN + ln;
+    // rows and columns of this thread (i-th row, j-th column)
+    auto row = [&](int i) { return im * RQ + i % RQ + (i / RQ) * (RQ * MT); };
+    constexpr int CQ = TN < 4 ? TN : 4;   // columns side by side
+    auto col = [&](int j) { return in * CQ + j % CQ + (j / CQ) * (CQ * NT); };
+    uint64_t acc[TM / 2][TN];
 #pragma unroll
-    for (int i = 0; i < TM; ++i)
+    for (int i = 0; i < TM / 2; ++i)
 #pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = T(0);
+        for (int j = 0; j < TN; ++j) acc[i][j] = 0ull;
+    auto value = [&](int i, int j) { return half_of(acc[i >> 1][j], i & 1); };
+    auto kstep = [&](const float *ra, const float *rb) {
+        uint64_t a[TM / 2];
+#pragma unroll
+        for (int i = 0; i < TM / 2; i += RQ / 2) {
+            if (RQ == 4) *(ulonglong2 *)(a + i) = *(const ulonglong2 *)(ra + row(2 * i));
+            else a[i] = *(const uint64_t *)(ra + row(2 * i));
+        }
+        float b[TN];
+#pragma unroll
+        for (int j = 0; j < TN; j += CQ) {
+            if (CQ == 4) *(float4 *)(b + j) = *(const float4 *)(rb + col(j));
+            else if (CQ == 2) *(float2 *)(b + j) = *(const float2 *)(rb + col(j));
+            else b[j] = rb[col(j)];
+        }
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+            const uint64_t bb = dup2(b[j]);
+#pragma unroll
+            for (int i = 0; i < TM / 2; ++i) fma2(acc[i][j], a[i], bb);
+        }
+    };
 #pragma unroll
     for (int s = 0; s < kStages - 1; ++s) issue();
     int c_li = 0, c_ks = 0, c_stage = 0;
-    const bool kshort = d.nsplit == 1 && d.K <= kBK / 2;
     while (c_li < mine) {
         cp_async_wait<kStages - 2>();
         __syncthreads();
         issue();
-        const T *sa = As + c_stage * SA + im;
-        const T *sb = Bs + c_stage * SB + in;
-        auto kstep = [&](int kk) {
-            T a[TM], bv[TN];
-#pragma unroll
-            for (int i = 0; i < TM; ++i) a[i] = sa[kk * RA + i * MT];
-#pragma unroll
-            for (int j = 0; j < TN; ++j) bv[j] = sb[kk * RB + j * NT];
-#pragma unroll
-            for (int i = 0; i < TM; ++i)
-#pragma unroll
-                for (int j = 0; j < TN; ++j) acc[i][j] += a[i] * bv[j];
-        };
-        if (kshort) {
-            // summed space of at most half a stage: the other half is zeros
-#pragma unroll
-            for (int kk = 0; kk < kBK / 2; ++kk) kstep(kk);
-        } else {
-#pragma unroll
-            for (int kk = 0; kk < kBK; ++kk) kstep(kk);
+        const float *sa = As + c_stage * SA, *sb = Bs + c_stage * SB;
+#pragma unroll(TM * TN < 64 ? 8 : 2)
+        for (int kk = 0; kk < kBK / 2; ++kk) kstep(sa + kk * GA::LD, sb + kk * GB::LD);
+        if (klast == kBK || (TAIL && c_ks < nks - 1)) {
+#pragma unroll(TM * TN < 64 ? 8 : 2)
+            for (int kk = kBK / 2; kk < kBK; ++kk) kstep(sa + kk * GA::LD, sb + kk * GB::LD);
         }
         c_stage = c_stage == kStages - 1 ? 0 : c_stage + 1;
         if (++c_ks < nks) continue;
@@ -218,45 +308,96 @@ __global__ void __launch_bounds__(kThreads, 2)
         const int m0 = (int)tp.m0, n0 = (int)tp.n0;
         if (d.nsplit > 1) {
             // unscaled partials, dense [split][item][g][n][m]
-            T *P = part + (((int64_t)tp.split * d.nbeta + tp.beta) * d.G + tp.g) * d.M * d.N;
+            float *P = part + (((int64_t)tp.split * d.nbeta + tp.beta) * d.G + tp.g) * d.M * d.N;
 #pragma unroll
-            for (int i = 0; i < TM; ++i) {
-                const int m = m0 + im + i * MT;
+            for (int i = 0; i < TM; ++i)
 #pragma unroll
                 for (int j = 0; j < TN; ++j) {
-                    const int n = n0 + in + j * NT;
-                    if (m < d.M && n < d.N) P[(int64_t)n * d.M + m] = acc[i][j];
-                    acc[i][j] = T(0);
+                    const int m = m0 + row(i), n = n0 + col(j);
+                    if (m < d.M && n < d.N) P[(int64_t)n * d.M + m] = value(i, j);
+                }
+        } else {
+            const float sca = d.mxa ? pow2neg<float>(exp_of_bits(d.mxa[tp.beta * d.mxa_bs])) : 1.f;
+            const float scb = d.mxb ? pow2neg<float>(exp_of_bits(d.mxb[tp.beta * d.mxb_bs])) : 1.f;
+            const float sc = sca * scb;
+            float *Cb = (float *)d.C + tp.beta * d.bsc + __ldg(d.tcg + tp.g);
+            float mx = 0.f;
+            if (!NFAST && RQ == 4) {
+                // quads of rows are contiguous in C
+#pragma unroll
+                for (int i = 0; i < TM; i += 4) {
+                    const int m = m0 + row(i);
+                    if (m >= d.M) continue;
+                    float *Cm = Cb + __ldg(d.tcm + m);
+#pragma unroll
+                    for (int j = 0; j < TN; ++j) {
+                        const int n = n0 + col(j);
+                        if (n >= d.N) continue;
+                        const float4 v = make_float4(value(i, j) * sc, value(i + 1, j) * sc,
+                                                     value(i + 2, j) * sc, value(i + 3, j) * sc);
+                        *(float4 *)(Cm + __ldg(d.tcn + n)) = v;
+                        mx = fmaxf(mx, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+                    }
+                }
+            } else if (!NFAST && d.vc == 2) {
+                // pairs of rows are contiguous in C
+#pragma unroll
+                for (int i = 0; i < TM; i += 2) {
+                    const int m = m0 + row(i);
+                    if (m >= d.M) continue;
+                    float *Cm = Cb + __ldg(d.tcm + m);
+#pragma unroll
+                    for (int j = 0; j < TN; ++j) {
+                        const int n = n0 + col(j);
+                        if (n >= d.N) continue;
+                        const float2 v = make_float2(value(i, j) * sc, value(i + 1, j) * sc);
+                        *(float2 *)(Cm + __ldg(d.tcn + n)) = v;
+                        mx = fmaxf(mx, fmaxf(v.x, v.y));
+                    }
+                }
+            } else if (NFAST && TN >= 4 && d.vc == 4) {
+                // quads of columns are contiguous in C
+#pragma unroll
+                for (int i = 0; i < TM; ++i) {
+                    const int m = m0 + row(i);
+                    if (m >= d.M) continue;
+                    float *Cm = Cb + __ldg(d.tcm + m);
+#pragma unroll
+                    for (int j = 0; j + 3 < TN; j += 4) {
+                        const int n = n0 + col(j);
+                        if (n >= d.N) continue;
+                        const float4 v = make_float4(value(i, j) * sc, value(i, j + 1) * sc,
+                                                     value(i, j + 2) * sc, value(i, j + 3) * sc);
+                        *(float4 *)(Cm + __ldg(d.tcn + n)) = v;
+                        mx = fmaxf(mx, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+                    }
+                }
+            } else {
+                int32_t cn[TN];
+#pragma unroll
+                for (int j = 0; j < TN; ++j) {
+                    const int n = n0 + col(j);
+                    cn[j] = n < d.N ? __ldg(d.tcn + n) : -1;
+                }
+#pragma unroll
+                for (int i = 0; i < TM; ++i) {
+                    const int m = m0 + row(i);
+                    const int32_t cm = m < d.M ? __ldg(d.tcm + m) : -1;
+#pragma unroll
+                    for (int j = 0; j < TN; ++j)
+                        if (cm >= 0 && cn[j] >= 0) {
+                            const float v = value(i, j) * sc;
+                            Cb[cm + cn[j]] = v;
+                            mx = fmaxf(mx, v);
+                        }
                 }
             }
-            continue;
-        }
-        const T sca = d.mxa ? pow2neg<T>(exp_of_bits(d.mxa[tp.beta * d.mxa_bs])) : T(1);
-        const T scb = d.mxb ? pow2neg<T>(exp_of_bits(d.mxb[tp.beta * d.mxb_bs])) : T(1);
-        const T sc = sca * scb;
-        T *Cb = (T *)d.C + tp.beta * d.bsc + __ldg(d.tcg + tp.g);
-        T mx = 0;
-        int32_t cn[TN];
-#pragma unroll
-        for (int j = 0; j < TN; ++j) {
-            const int n = n0 + in + j * NT;
-            cn[j] = n < d.N ? __ldg(d.tcn + n) : -1;
+            record_max(d.mxc, tp.beta, true, (double)mx);
         }
 #pragma unroll
-        for (int i = 0; i < TM; ++i) {
-            const int m = m0 + im + i * MT;
-            const int32_t cm = m < d.M ? __ldg(d.tcm + m) : -1;
+        for (int i = 0; i < TM / 2; ++i)
 #pragma unroll
-            for (int j = 0; j < TN; ++j) {
-                if (cm >= 0 && cn[j] >= 0) {
-                    const T v = acc[i][j] * sc;
-                    Cb[cm + cn[j]] = v;
-                    mx = mx > v ? mx : v;
-                }
-                acc[i][j] = T(0);
-            }
-        }
-        record_max(d.mxc, tp.beta, true, (double)mx);
+            for (int j = 0; j < TN; ++j) acc[i][j] = 0ull;
     }
     cp_async_wait<0>();
 }
@@ -379,32 +520,22 @@ __global__ void __launch_bounds__(kThreads) k_bgemm_fin(const __grid_constant__ 
     record_max(d.mxc, beta, active, (double)v);
 }
 
-// Tile shapes (BM x BN, thread tiles TM x TN): 0 for n > 48, 1 for
-// 16 < n <= 48, 2 for 8 < n <= 16, 3 for n <= 8 (128 x 8: the 256 x 16 tile
-// would leave half of every row and, for short rows, half of every column
-// idle).
-template <typename T>
-struct Tiles;
-template <>
-struct Tiles<float> {
-    static constexpr int BM[4] = {128, 256, 256, 128}, BN[4] = {64, 32, 16, 8};
-    static constexpr int TM[4] = {8, 8, 8, 4}, TN[4] = {4, 4, 2, 1};
-};
-template <typename T, int TILE>
-constexpr size_t smem_bytes() {
-    return (size_t)kStages * kBK *
-           ((size_t)Tiles<T>::BM[TILE] + 1 + (size_t)Tiles<T>::BN[TILE] + 1) * sizeof(T);
-}
+// FP32 tile shapes (BM x BN, thread tiles TM x TN): 0 for n > 48, 1 for
+// 16 < n <= 48, 2 for 8 < n <= 16, 3 for n <= 8 and few rows (128 x 8: the wider
+// tiles would leave half of every row and, for short rows, half of every column
+// idle), 4 for n > 64 and 5 for n <= 8 where there are rows enough.
+constexpr int kBM[6] = {128, 256, 256, 128, 128, 256}, kBN[6] = {64, 32, 16, 8, 128, 8};
+constexpr int kTM[6] = {8, 8, 8, 4, 8, 4}, kTN[6] = {4, 4, 2, 1, 8, 2};
 
 // Launch one instantiation as a persistent grid: resident blocks per SM from
 // the occupancy calculator (queried once), at most one block per tile.
-template <typename T, int TILE, bool NFAST>
-void go(const BDesc &d, T *part, int64_t ntiles, cudaStream_t st) {
+template <int TILE, bool NFAST, int RQ>
+void go(const BDesc &d, float *part, int64_t ntiles, cudaStream_t st) {
     // tile counts are checked on the host to fit 31 bits
-    constexpr int BM = Tiles<T>::BM[TILE], BN = Tiles<T>::BN[TILE];
-    constexpr int TM = Tiles<T>::TM[TILE], TN = Tiles<T>::TN[TILE];
-    constexpr size_t smem = smem_bytes<T, TILE>();
-    auto kern = k_bgemm<T, BM, BN, TM, TN, NFAST>;
+    constexpr int BM = kBM[TILE], BN = kBN[TILE];
+    constexpr size_t smem =
+        (size_t)kStages * (Gather<BM>::SIZE + Gather<BN>::SIZE) * sizeof(float);
+    auto kern = k_bgemm<BM, BN, kTM[TILE], kTN[TILE], NFAST, RQ>;
     static std::once_flag once;
     static int per_sm = 1, nsm = 152;
     std::call_once(once, [&] {
@@ -422,6 +553,13 @@ void go(const BDesc &d, T *part, int64_t ntiles, cudaStream_t st) {
     });
     const int64_t grid = std::min<int64_t>(ntiles, (int64_t)nsm * per_sm);
     kern<<<(unsigned)grid, kThreads, smem, st>>>(d, part, (int)ntiles);
+}
+
+template <int TILE>
+void go_rows(const BDesc &d, float *part, int64_t ntiles, cudaStream_t st) {
+    if (d.c_nfast) go<TILE, true, 4>(d, part, ntiles, st);
+    else if (d.vc == 4) go<TILE, false, 4>(d, part, ntiles, st);
+    else go<TILE, false, 2>(d, part, ntiles, st);
 }
 
 }  // namespace
@@ -488,7 +626,13 @@ void bgemm_configure(BDesc &d, int elem_bytes) {
         if ((double)direct_tasks(d) * d.nsplit >= 1e10) d.tile = -1;
         return;
     }
-    const int bm = Tiles<float>::BM[d.tile], bn = Tiles<float>::BN[d.tile];
+    // 128 x 128 where that pads the columns no more than 128 x 64 and leaves
+    // every SM two blocks
+    if (d.N > 64 && (d.N + 127) / 128 * 128 <= (d.N + 63) / 64 * 64 * 9 / 8 &&
+        ((d.M + 127) / 128) * ((d.N + 127) / 128) * d.G * d.nbeta >= 152 * 2)
+        d.tile = 4;
+    if (d.N <= 8 && ((d.M + 255) / 256) * d.G * d.nbeta >= 152 * 2) d.tile = 5;
+    const int bm = kBM[d.tile], bn = kBN[d.tile];
     const int64_t tiles = ((d.M + bm - 1) / bm) * ((d.N + bn - 1) / bn) * d.G * d.nbeta;
     // split the summed space when the output tiles alone leave most SMs idle
     // and every split still runs several K steps; partials stay under 1 GiB
@@ -571,19 +715,17 @@ void launch_bgemm<float>(const BDesc &d, void *scratch, cudaStream_t st) {
         launch_tc_gather(d, st);
         return;
     }
-    const int bm = Tiles<float>::BM[d.tile], bn = Tiles<float>::BN[d.tile];
+    const int bm = kBM[d.tile], bn = kBN[d.tile];
     const int64_t ntiles =
         ((d.M + bm - 1) / bm) * ((d.N + bn - 1) / bn) * d.G * d.nbeta * d.nsplit;
     float *part = (float *)scratch;
-    switch (d.tile * 2 + (d.c_nfast ? 1 : 0)) {
-        case 0: go<float, 0, false>(d, part, ntiles, st); break;
-        case 1: go<float, 0, true>(d, part, ntiles, st); break;
-        case 2: go<float, 1, false>(d, part, ntiles, st); break;
-        case 3: go<float, 1, true>(d, part, ntiles, st); break;
-        case 4: go<float, 2, false>(d, part, ntiles, st); break;
-        case 5: go<float, 2, true>(d, part, ntiles, st); break;
-        case 6: go<float, 3, false>(d, part, ntiles, st); break;
-        default: go<float, 3, true>(d, part, ntiles, st); break;
+    switch (d.tile) {
+        case 0: go_rows<0>(d, part, ntiles, st); break;
+        case 1: go_rows<1>(d, part, ntiles, st); break;
+        case 2: go_rows<2>(d, part, ntiles, st); break;
+        case 3: go_rows<3>(d, part, ntiles, st); break;
+        case 4: go_rows<4>(d, part, ntiles, st); break;
+        default: go_rows<5>(d, part, ntiles, st); break;
     }
     if (d.nsplit > 1)
         k_bgemm_fin<float>

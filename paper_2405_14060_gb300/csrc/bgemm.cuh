@@ -26,6 +26,7 @@ struct BDesc {
     int a_kfast;                   // A's fastest label is summed (else it is in M or G)
     int b_kfast;                   // B's fastest label is summed (else in N or G)
     int c_nfast;                   // C's fastest label is in N (else in M or G)
+    int va, vb, vc;                // floats per copy of A and B and per store of C (1, 2, 4)
     int c_gfast;                   // a G label lies inside C's 32-byte sectors: tiles
                                    // enumerate G fastest, so that the tiles writing
                                    // the same sectors run together (their partial

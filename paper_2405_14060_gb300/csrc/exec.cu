@@ -1005,6 +1005,44 @@ static bool make_bgemm(const std::vector<int> &card, const Labels &lx, bool bx, 
     if (perx >= (1LL << 31) || pery >= (1LL << 31) || pero >= (1LL << 31)) return false;
     const int64_t ntab = 3 * d.G + 2 * d.M + 2 * d.N + 2 * d.K;
     if (ntab > (1LL << 26)) return false;
+    // the group holding each tensor's fastest label (of size > 1)
+    auto in = [](const Labels &l, int v) { return std::find(l.begin(), l.end(), v) != l.end(); };
+    d.a_kfast = in(K, fastest_of(lx)) ? 1 : 0;
+    d.b_kfast = in(K, fastest_of(ly)) ? 1 : 0;
+    d.c_nfast = in(N, fo) ? 1 : 0;
+    if (esz == 4 && !d.a_kfast && d.b_kfast) {
+        // only B's contiguous labels are summed: they enumerate fastest
+        Labels k;
+        for (int v : ly)
+            if (in(K, v)) k.push_back(v);
+        K = k;
+    }
+    // floats per copy: the run of `grp` that is contiguous in a tensor when it
+    // holds whole, aligned groups of 4 or 2 and every other stride is one too
+    auto width = [&](const Labels &grp, const Labels &lt, int64_t item, const void *ptr) {
+        std::set<int> run;
+        int64_t len = 1;
+        for (int i = (int)grp.size() - 1; i >= 0; --i) {
+            const int v = grp[i];
+            if (card[v] == 1) continue;
+            if (stride_in(card, lt, v) != len) break;
+            len *= card[v];
+            run.insert(v);
+        }
+        for (int w : {4, 2}) {
+            bool ok = len % w == 0 && item % w == 0 && ((uintptr_t)ptr % (4 * w)) == 0;
+            for (int v : lt) ok = ok && (card[v] == 1 || run.count(v) || stride_in(card, lt, v) % w == 0);
+            if (ok) return w;
+        }
+        return 1;
+    };
+    d.va = d.vb = d.vc = 1;
+    if (esz == 4) {
+        // (stages hold rows side by side: wider copies only along those)
+        if (!d.a_kfast) d.va = width(M, lx, bo && bx ? perx : 0, X);
+        if (!d.b_kfast) d.vb = width(N, ly, bo && by ? pery : 0, Y);
+        d.vc = width(d.c_nfast ? N : M, lo, bo ? pero : 0, O);
+    }
     // tables as dimensions for the device to fill, where they fit its records
     if (dims) {
         GroupTabs &g = *dims;
@@ -1080,16 +1118,6 @@ static bool make_bgemm(const std::vector<int> &card, const Labels &lx, bool bx, 
     d.tcn = (const int32_t *)(intptr_t)o_cn;
     d.tak = (const int32_t *)(intptr_t)o_ak;
     d.tbk = (const int32_t *)(intptr_t)o_bk;
-    // the group holding each tensor's fastest label (of size > 1)
-    auto fastest = [&](const Labels &lt) {
-        for (int k = (int)lt.size() - 1; k >= 0; --k)
-            if (card[lt[k]] > 1) return lt[k];
-        return -1;
-    };
-    auto in = [](const Labels &l, int v) { return std::find(l.begin(), l.end(), v) != l.end(); };
-    d.a_kfast = in(K, fastest(lx)) ? 1 : 0;
-    d.b_kfast = in(K, fastest(ly)) ? 1 : 0;
-    d.c_nfast = in(N, fastest(lo)) ? 1 : 0;
     // a group label inside C's 32-byte sectors: tiles enumerate G fastest,
     // so the tiles sharing a sector write it at about the same time
     d.c_gfast = 0;

@@ -120,6 +120,30 @@ def test_direct_fp64(m, n, k, spec):
     np.testing.assert_allclose(C.cpu().numpy(), ref, rtol=k * 2.3e-16 + 1e-15, atol=0)
 
 
+# FP32 batched GEMM: rows and columns around every tile (8, 16, 32, 64, 128
+# columns), last K steps of at most half (8, 24, 37) and more (13, 16), copies of
+# 4, 2 and 1 floats, summed fastest in one, both or no operand, quads / pairs /
+# single floats of C side by side, a group label inside C's sectors
+@pytest.mark.parametrize("m,n,k", [(1, 1, 3), (100, 8, 24), (300, 7, 37), (2048, 8, 13), (257, 16, 8),
+                                   (640, 33, 16), (130, 66, 100), (3000, 130, 7), (16384, 128, 20)])
+@pytest.mark.parametrize("spec", ["mk,kn->mn", "km,kn->nm", "mk,nk->nm", "gkm,kgn->gnm",
+                                  "mgk,kgn->nmg", "kmg,gnk->mng", "mhk,kn->nmh"])
+def test_bgemm_fp32_tiles(m, n, k, spec):
+    (a, b), c = spec.split("->")[0].split(","), spec.split("->")[1]
+    letters = "ghkmn"
+    size = dict(g=2, h=2, k=k, m=m, n=n)
+    rng = np.random.default_rng(m + n * k)
+    A = rng.random([size[l] for l in a]).astype(np.float32)
+    B = rng.random([size[l] for l in b]).astype(np.float32)
+    ref = np.einsum(spec, A.astype(np.float64), B.astype(np.float64))
+    C = torch.full([size[l] for l in c], float("nan"), dtype=torch.float32, device="cuda")
+    tn.contract_dev([size[l] for l in letters], [letters.index(l) for l in a], torch.tensor(A).cuda(),
+                    [letters.index(l) for l in b], torch.tensor(B).cuda(),
+                    [letters.index(l) for l in c], C, prec="fp32")
+    # positive terms: every order of summation is within k + 1 roundings
+    np.testing.assert_allclose(C.cpu().numpy(), ref, rtol=(k + 1) * 6e-8, atol=0)
+
+
 # FP32 GEMM: one tile of every shape and several, ragged rows, columns and
 # summed space, operands already in GEMM form, split long summed spaces
 @pytest.mark.parametrize("m,n,k", [(64, 64, 64), (65, 70, 77), (193, 129, 96), (1000, 900, 130),
