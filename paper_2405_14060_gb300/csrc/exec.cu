@@ -298,11 +298,22 @@ struct Program {
 
 // The programs of the last MMAP call (its query / evidence pattern and
 // precision): a call with the same pattern replays them with new values.
+// Their graphs are branches of one graph, the top program's behind all of them,
+// and they read one evidence buffer, so a call is one copy and one launch (with
+// a launch, a copy and a wait per group, 1.3 of a 300-variable call's 2.5 ms
+// passed between the kernels).
 struct MmapCache {
     std::vector<int8_t> key;   // per variable: 0 summed, 1 queried, 2 observed; then dtype
     std::vector<std::unique_ptr<Program>> groups;
     std::unique_ptr<Program> top;
     double lconst = 0;
+    DevMem mem;
+    int32_t *d_evid = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    int64_t launches = 0;
+    ~MmapCache() {
+        if (exec) cudaGraphExecDestroy(exec);
+    }
 };
 
 struct tn_model {
@@ -1566,7 +1577,7 @@ static void trace_program(const Program &P) {
 tn_status build_program(tn_model *m, const Net &net, const Tree &tree, int kind, int dtype,
                         int nbeta, bool grads, const tn_options *opts, Program &P,
                         const std::vector<LeafRec> *spec = nullptr,
-                        const Tune *tune = nullptr) {
+                        const Tune *tune = nullptr, int32_t *shared_evid = nullptr) {
     if (tune) P.tune = *tune;
     P.kind = kind;
     P.dtype = dtype;
@@ -1845,14 +1856,16 @@ tn_status build_program(tn_model *m, const Net &net, const Tree &tree, int kind,
     CK(P.mem.alloc(&P.arena, (size_t)P.arena_elems * P.esz));
     CK(P.mem.alloc(&P.mx, (size_t)nmx * 8));
     if (am_total) CK(P.mem.alloc(&P.am, (size_t)am_total * 4));
-    CK(P.mem.alloc(&P.d_evid, (size_t)nbeta * std::max(1, m->md.nvars) * 4));
+    P.d_evid = shared_evid;
+    if (!shared_evid) CK(P.mem.alloc(&P.d_evid, (size_t)nbeta * std::max(1, m->md.nvars) * 4));
     CK(P.mem.alloc(&P.d_slice_val, 4 * std::max<size_t>(1, m->slice_vars.size())));
     CK(cudaMemset(P.d_slice_val, 0, 4 * std::max<size_t>(1, m->slice_vars.size())));
     CK(P.mem.alloc(&P.d_logz, (size_t)nbeta * 8));
     CK(P.mem.alloc(&P.d_sigma, (size_t)nbeta * 8));
     CK(P.mem.alloc(&P.d_card, net.card.size() * 4 + 4));
     CK(cudaMemcpy(P.d_card, net.card.data(), net.card.size() * 4, cudaMemcpyHostToDevice));
-    CK(cudaMemset(P.d_evid, 0xff, (size_t)nbeta * std::max(1, m->md.nvars) * 4));
+    if (!shared_evid)
+        CK(cudaMemset(P.d_evid, 0xff, (size_t)nbeta * std::max(1, m->md.nvars) * 4));
     // ---- leaf records
     for (int id = 0; id < n; ++id) {
         LeafRec r;
@@ -2752,7 +2765,10 @@ void enqueue_program(tn_model *m, Program &P, cudaStream_t st, Prof *pr = nullpt
     cudaMemsetAsync(P.mx, 0, (size_t)P.nmx * 8, st);
     if (P.nrcnt) cudaMemsetAsync(P.rcnt, 0, (size_t)P.nrcnt * P.nlanes * 4, st);
     ++nl;
-    launch_leaves<T>(P.d_leaf, P.nleafrec, m->d_tables, P.d_card, m->md.nvars, P.d_evid, P.nbeta,
+    int64_t largest = 1;   // entries of the largest table leaf
+    for (const LeafRec &r : P.leafrec)
+        if (r.kind != LEAF_UNITY) largest = std::max(largest, r.size);
+    launch_leaves<T>(P.d_leaf, P.nleafrec, largest, m->d_tables, P.d_card, m->md.nvars, P.d_evid, P.nbeta,
                      maxplus ? 1 : 0, (T *)P.arena, P.mx, m->d_flags, P.d_slice_val, st);
     ++nl;
     const bool par = lanes && P.nlanes > 1 && (int)P.ev.size() >= 2 * NN + 1 + P.nlanes;
@@ -3011,9 +3027,38 @@ tn_status check_device_error(tn_model *m) {
     return TN_OK;
 }
 
-// Run a captured program: copy the evidence in, replay the graph, time it.
+// A copy of results behind a program's kernels.
+struct OutCopy {
+    void *dst;
+    const void *src;
+    size_t bytes;
+};
+
+// Run a captured graph between the model's timing events, then copy its results
+// and the flag of device-side waits behind it, all before the one wait.
+tn_status run_graph(tn_model *m, cudaGraphExec_t exec, cudaStream_t st,
+                    std::initializer_list<OutCopy> outs, cudaMemcpyKind kind) {
+    CK(cudaEventRecord(m->ev0, st));
+    CK(cudaGraphLaunch(exec, st));
+    CK(cudaEventRecord(m->ev1, st));
+    for (const OutCopy &o : outs)
+        if (o.bytes) CK(cudaMemcpyAsync(o.dst, o.src, o.bytes, kind, st));
+    int err = 0;
+    CK(cudaMemcpyAsync(&err, m->d_err, 4, cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    float ms = 0;
+    CK(cudaEventElapsedTime(&ms, m->ev0, m->ev1));
+    m->last_ms = ms;
+    CK(cudaGetLastError());
+    return err ? check_device_error(m) : TN_OK;
+}
+
+// Run a captured program: copy the evidence in, replay the graph, time it and
+// copy its results out (sync), or only enqueue the replay.
 tn_status run_program(tn_model *m, Program &P, const int32_t *evid, bool evid_on_device,
-                      cudaStream_t st, bool sync = true, int nrows = -1) {
+                      cudaStream_t st, bool sync = true, int nrows = -1,
+                      std::initializer_list<OutCopy> outs = {},
+                      cudaMemcpyKind kind = cudaMemcpyDeviceToHost) {
     if (nrows < 0) nrows = P.nbeta;
     size_t row = (size_t)m->md.nvars * 4, eb = (size_t)P.nbeta * row;
     if (eb) {
@@ -3024,21 +3069,10 @@ tn_status run_program(tn_model *m, Program &P, const int32_t *evid, bool evid_on
             CK(cudaMemsetAsync((char *)P.d_evid + (evid ? (size_t)nrows * row : 0), 0xff,
                                eb - (evid ? (size_t)nrows * row : 0), st));
     }
-    if (!sync) {
-        CK(cudaGraphLaunch(P.gexec, st));
-        m->last_launches = P.launches;
-        return TN_OK;
-    }
-    CK(cudaEventRecord(m->ev0, st));
-    CK(cudaGraphLaunch(P.gexec, st));
-    CK(cudaEventRecord(m->ev1, st));
-    CK(cudaStreamSynchronize(st));
-    float ms = 0;
-    CK(cudaEventElapsedTime(&ms, m->ev0, m->ev1));
-    m->last_ms = ms;
     m->last_launches = P.launches;
-    CK(cudaGetLastError());
-    return check_device_error(m);
+    if (sync) return run_graph(m, P.gexec, st, outs, kind);
+    CK(cudaGraphLaunch(P.gexec, st));
+    return TN_OK;
 }
 
 // Number of slice assignments and (lazily) the device table of all of them,
@@ -3465,17 +3499,21 @@ static tn_status pr_common(tn_model *m, int batch, const int32_t *evid, bool evi
     for (int i = 0; i < batch; i += sub) {
         int nr = std::min(sub, batch - i);
         const int32_t *ev = evid ? evid + (size_t)i * m->md.nvars : nullptr;
-        s = m->slice_vars.empty() ? run_program(m, *P, ev, evid_dev, st, !async, nr)
-                                  : run_sliced(m, *P, ev, evid_dev, false, st, nr);
-        if (s) return s;
+        const cudaMemcpyKind k = logz_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+        const OutCopy out{logz + i, P->d_logz, (size_t)nr * 8};
+        if (m->slice_vars.empty() && !async) {
+            s = run_program(m, *P, ev, evid_dev, st, true, nr, {out}, k);
+            if (s) return s;
+        } else {
+            s = async ? run_program(m, *P, ev, evid_dev, st, false, nr)
+                      : run_sliced(m, *P, ev, evid_dev, false, st, nr);
+            if (s) return s;
+            CK(cudaMemcpyAsync(out.dst, out.src, out.bytes, k, st));
+            if (!async) CK(cudaStreamSynchronize(st));
+        }
         ms += m->last_ms;
-        CK(cudaMemcpyAsync(logz + i, P->d_logz, (size_t)nr * 8,
-                           logz_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st));
     }
-    if (!async) {
-        CK(cudaStreamSynchronize(st));
-        m->last_ms = ms;
-    }
+    if (!async) m->last_ms = ms;
     return TN_OK;
 }
 
@@ -3509,19 +3547,24 @@ static tn_status mar_common(tn_model *m, int batch, const int32_t *evid, bool de
     for (int i = 0; i < batch; i += sub) {
         int nr = std::min(sub, batch - i);
         const int32_t *ev = evid ? evid + (size_t)i * m->md.nvars : nullptr;
-        s = m->slice_vars.empty() ? run_program(m, *P, ev, dev, st, !async, nr)
-                                  : run_sliced(m, *P, ev, dev, true, st, nr);
-        if (s) return s;
+        const OutCopy oz{logz + i, P->d_logz, (size_t)nr * 8},
+            om{marg + (size_t)i * P->marg_stride, P->d_marg, (size_t)nr * P->marg_stride * 8},
+            og{grad ? grad + (size_t)i * P->grad_stride : nullptr, P->d_grad,
+               grad ? (size_t)nr * P->grad_stride * 8 : 0};
+        if (m->slice_vars.empty() && !async) {
+            s = run_program(m, *P, ev, dev, st, true, nr, {oz, om, og}, k);
+            if (s) return s;
+        } else {
+            s = async ? run_program(m, *P, ev, dev, st, false, nr)
+                      : run_sliced(m, *P, ev, dev, true, st, nr);
+            if (s) return s;
+            for (const OutCopy &o : {oz, om, og})
+                if (o.bytes) CK(cudaMemcpyAsync(o.dst, o.src, o.bytes, k, st));
+            if (!async) CK(cudaStreamSynchronize(st));
+        }
         ms += m->last_ms;
-        CK(cudaMemcpyAsync(logz + i, P->d_logz, (size_t)nr * 8, k, st));
-        CK(cudaMemcpyAsync(marg + (size_t)i * P->marg_stride, P->d_marg,
-                           (size_t)nr * P->marg_stride * 8, k, st));
-        if (grad)
-            CK(cudaMemcpyAsync(grad + (size_t)i * P->grad_stride, P->d_grad,
-                               (size_t)nr * P->grad_stride * 8, k, st));
     }
     if (async) return TN_OK;
-    CK(cudaStreamSynchronize(st));
     m->last_ms = ms;
     if (!dev) {
         for (int b = 0; b < batch; ++b)
@@ -3702,11 +3745,9 @@ tn_status tn_map(tn_model *m, const int32_t *evid, const tn_options *opts, int32
     cudaStream_t st = stream_of(m, opts);
     s = override_tables(m, nullptr, 0, st);
     if (s) return s;
-    s = run_program(m, *P, evid, false, st);
+    s = run_program(m, *P, evid, false, st, true, -1,
+                    {{logp, P->d_logz, 8}, {assign, P->d_assign, (size_t)m->md.nvars * 4}});
     if (s) return s;
-    CK(cudaMemcpyAsync(logp, P->d_logz, 8, cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(assign, P->d_assign, (size_t)m->md.nvars * 4, cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
     if (!(*logp > -INFINITY)) return fail(TN_E_ARG, "p(e) = 0");
     return TN_OK;
 }
@@ -3756,10 +3797,9 @@ tn_status tn_sample(tn_model *m, const int32_t *evid, uint64_t seed, int64_t n,
     if (s) return s;
     const int nv = m->md.nvars;
     if (m->slice_vars.empty()) {
-        s = run_program(m, *P, evid, false, st);
-        if (s) return s;
         double lz;
-        CK(cudaMemcpy(&lz, P->d_logz, 8, cudaMemcpyDeviceToHost));
+        s = run_program(m, *P, evid, false, st, true, -1, {{&lz, P->d_logz, 8}});
+        if (s) return s;
         if (!(lz > -INFINITY)) return fail(TN_E_ARG, "p(e) = 0");
         if (n == 0) return TN_OK;
         CallMem out(st);
@@ -3789,6 +3829,7 @@ tn_status tn_sample(tn_model *m, const int32_t *evid, uint64_t seed, int64_t n,
     std::vector<int32_t> ev(nv, -1);
     if (evid) std::copy(evid, evid + nv, ev.begin());
     double tms = 0;
+    double lz_a = 0;   // log Z of the last assignment run
     // forward pass of assignment a; `possible` false when the evidence rules it out
     auto run_assignment = [&](int64_t a, bool &possible) -> tn_status {
         std::vector<int32_t> ea = ev;
@@ -3804,7 +3845,7 @@ tn_status tn_sample(tn_model *m, const int32_t *evid, uint64_t seed, int64_t n,
         if (!possible) return TN_OK;
         CK(cudaMemcpyAsync(P->d_slice_val, m->d_sl_tab + a * nsl, (size_t)nsl * 4,
                            cudaMemcpyDeviceToDevice, st));
-        tn_status e = run_program(m, *P, ea.data(), false, st);
+        tn_status e = run_program(m, *P, ea.data(), false, st, true, -1, {{&lz_a, P->d_logz, 8}});
         tms += m->last_ms;
         return e;
     };
@@ -3814,8 +3855,7 @@ tn_status tn_sample(tn_model *m, const int32_t *evid, uint64_t seed, int64_t n,
         s = run_assignment(a, ok);
         if (s) return s;
         if (!ok) continue;
-        CK(cudaMemcpy(&lz[a], P->d_logz, 8, cudaMemcpyDeviceToHost));
-        if (!(lz[a] > -INFINITY)) lz[a] = -INFINITY;
+        lz[a] = lz_a > -INFINITY ? lz_a : -INFINITY;
     }
     double mx = -INFINITY;
     for (double v : lz) mx = std::max(mx, v);
@@ -3907,37 +3947,26 @@ tn_status tn_mmap(tn_model *m, const int32_t *evid, int nq, const int32_t *query
     std::vector<int8_t> key(md.nvars + 1);
     for (int v = 0; v < md.nvars; ++v) key[v] = isq[v] ? 1 : ise[v] ? 2 : 0;
     key[md.nvars] = (int8_t)(dtype * 4 + (int)prec);
-    // results of the top-level MPE program: log p and the assignment
-    auto finish = [&](Program &P2, double lconst, double ms, int64_t launches) -> tn_status {
+    // one launch of every program; results of the top-level MPE program
+    auto solve = [&](MmapCache &c) -> tn_status {
         double lp;
         std::vector<int32_t> x(md.nvars);
-        CK(cudaMemcpyAsync(&lp, P2.d_logz, 8, cudaMemcpyDeviceToHost, st));
-        CK(cudaMemcpyAsync(x.data(), P2.d_assign, (size_t)md.nvars * 4, cudaMemcpyDeviceToHost,
-                           st));
-        CK(cudaStreamSynchronize(st));
-        *logp = lp + lconst;
+        const size_t eb = (size_t)md.nvars * 4;
+        if (evid) CK(cudaMemcpyAsync(c.d_evid, evid, eb, cudaMemcpyHostToDevice, st));
+        else CK(cudaMemsetAsync(c.d_evid, 0xff, eb, st));
+        tn_status r = run_graph(m, c.exec, st, {{&lp, c.top->d_logz, 8}, {x.data(), c.top->d_assign, eb}},
+                                cudaMemcpyDeviceToHost);
+        if (r) return r;
+        *logp = lp + c.lconst;
         for (int i = 0; i < nq; ++i) assign[i] = x[query[i]];
-        m->last_launches = launches;
-        m->last_ms = ms;
+        m->last_launches = c.launches;
         if (!(lp > -INFINITY)) return fail(TN_E_ARG, "p(e) = 0");
         return TN_OK;
     };
-    if (m->mmap && m->mmap->key == key) {
-        double ms = 0;
-        int64_t launches = 0;
-        for (auto &P : m->mmap->groups) {
-            s = run_program(m, *P, evid, false, st);
-            if (s) return s;
-            ms += m->last_ms;
-            launches += P->launches;
-        }
-        s = run_program(m, *m->mmap->top, evid, false, st);
-        if (s) return s;
-        return finish(*m->mmap->top, m->mmap->lconst, ms + m->last_ms,
-                      launches + m->mmap->top->launches);
-    }
+    if (m->mmap && m->mmap->key == key) return solve(*m->mmap);
     m->mmap.reset();
-    double build_ms = 0;
+    auto c = std::make_unique<MmapCache>();
+    CK(c->mem.alloc(&c->d_evid, (size_t)std::max(1, md.nvars) * 4));
     // union-find over factors sharing a summed variable
     std::vector<int> par(md.nfactors);
     std::iota(par.begin(), par.end(), 0);
@@ -3968,11 +3997,9 @@ tn_status tn_mmap(tn_model *m, const int32_t *evid, int nq, const int32_t *query
         for (int v = 0; v < md.nvars; ++v)
             if (!seen[v] && !isq[v] && !ise[v]) lconst += std::log((double)md.card[v]);
     }
-    std::vector<std::unique_ptr<Program>> progs;
     Net net2;
     net2.card = md.card;
     std::vector<LeafRec> spec2;
-    int64_t launches = 0;
     for (auto &g : groups) {
         Net net;
         net.card = md.card;
@@ -4003,14 +4030,11 @@ tn_status tn_mmap(tn_model *m, const int32_t *evid, int nq, const int32_t *query
         }
         Tree t = optimize_tree(net, 1, 4, 12345);
         auto P = std::make_unique<Program>();
-        s = build_program(m, net, t, K_SUMNET, dtype, 1, false, opts, *P, &spec);
+        s = build_program(m, net, t, K_SUMNET, dtype, 1, false, opts, *P, &spec, nullptr, c->d_evid);
         if (s) return s;
         s = capture_program(m, *P);
         if (s) return s;
-        s = run_program(m, *P, evid, false, st);
-        if (s) return s;
-        build_ms += m->last_ms;
-        launches += P->launches;
+        c->launches += P->launches;
         const Node &root = P->plan.node[P->plan.root];
         net2.leaf.push_back(root.labels);
         net2.leaf_beta.push_back(0);
@@ -4021,7 +4045,7 @@ tn_status tn_mmap(tn_model *m, const int32_t *evid, int nq, const int32_t *query
         r.sigma = P->d_sigma;
         r.size = root.size;
         spec2.push_back(r);
-        progs.push_back(std::move(P));
+        c->groups.push_back(std::move(P));
     }
     std::set<int> evars2;
     for (int f : ungrouped) {
@@ -4057,22 +4081,28 @@ tn_status tn_mmap(tn_model *m, const int32_t *evid, int nq, const int32_t *query
         return fail(TN_E_UNSUPPORTED, "MMAP network with a single tensor");
     }
     Tree t2 = optimize_tree(net2, 1, 4, 54321);
-    auto P2 = std::make_unique<Program>();
-    s = build_program(m, net2, t2, K_MAP, dtype, 1, false, opts, *P2, &spec2);
+    c->top = std::make_unique<Program>();
+    s = build_program(m, net2, t2, K_MAP, dtype, 1, false, opts, *c->top, &spec2, nullptr, c->d_evid);
     if (s) return s;
-    s = capture_program(m, *P2);
+    s = capture_program(m, *c->top);
     if (s) return s;
-    s = run_program(m, *P2, evid, false, st);
-    if (s) return s;
-    build_ms += m->last_ms;
-    launches += P2->launches;
-    auto c = std::make_unique<MmapCache>();
+    c->launches += c->top->launches;
     c->key = key;
-    c->groups = std::move(progs);
-    c->top = std::move(P2);
     c->lconst = lconst;
+    cudaGraph_t all = nullptr;
+    CK(cudaGraphCreate(&all, 0));
+    std::vector<cudaGraphNode_t> nodes(c->groups.size());
+    cudaError_t e = cudaSuccess;
+    for (size_t i = 0; i < nodes.size() && e == cudaSuccess; ++i)
+        e = cudaGraphAddChildGraphNode(&nodes[i], all, nullptr, 0, c->groups[i]->graph);
+    cudaGraphNode_t top;
+    if (e == cudaSuccess)
+        e = cudaGraphAddChildGraphNode(&top, all, nodes.data(), nodes.size(), c->top->graph);
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&c->exec, all, 0);
+    cudaGraphDestroy(all);
+    if (e != cudaSuccess) return fail(TN_E_CUDA, std::string("MMAP graph: ") + cudaGetErrorString(e));
     m->mmap = std::move(c);
-    return finish(*m->mmap->top, lconst, build_ms, launches);
+    return solve(*m->mmap);
 }
 
 // Scratch memory of the calls that keep no program (single contractions, the

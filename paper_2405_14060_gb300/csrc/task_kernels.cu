@@ -2,6 +2,7 @@
 // unity / evidence vectors), log Z from the root and the rescaling exponents,
 // marginals from the adjoints of the unity vectors, factor marginals, MPE
 // backtracking and backward sampling.
+#include <algorithm>
 #include <cfloat>
 #include <cmath>
 #include <mutex>
@@ -22,17 +23,21 @@ __device__ __forceinline__ int exp_bits(unsigned long long b) {
 // Unity leaf of variable v (Sec. MAR step 1; Sec. MPE step 1): all ones for a
 // free variable; for an observed variable the indicator of its value, which
 // multiplies in the slicing T_{V|E=e} of Eq. pr.  In the log domain ones are
-// 0 and zeros are -inf.  Each leaf records its maximum for rescaling.
+// 0 and zeros are -inf.  Each leaf records its maximum for rescaling.  One block
+// per 256 entries of a table (a logarithm is some 50 FP64 operations, at two a
+// clock and SM: a 2^14-entry external leaf took 190 us in one block, LEAF_NOW).
 template <typename T>
 __global__ void k_leaves(const LeafRec *recs, const double *tables, const int *card, int nvars,
                          const int32_t *evid, int nbeta, int log_mode, T *base,
                          unsigned long long *mx, const int *flags, const int32_t *slice_val) {
-    const LeafRec r = recs[blockIdx.x];
+    const LeafRec &r = recs[blockIdx.x];
     T *dst = base + r.dst;
     __shared__ double smax[32];
     if (r.kind == LEAF_FACTOR || r.kind == LEAF_EXTERNAL) {
+        if ((int64_t)blockIdx.y * blockDim.x >= r.size) return;
         double m = log_mode ? -INFINITY : 0.0;
-        for (int64_t i = threadIdx.x; i < r.size; i += blockDim.x) {
+        for (int64_t i = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; i < r.size;
+             i += (int64_t)gridDim.y * blockDim.x) {
             double x;
             if (r.kind == LEAF_FACTOR) {
                 int64_t off = r.src + i;
@@ -68,10 +73,13 @@ __global__ void k_leaves(const LeafRec *recs, const double *tables, const int *c
         if (threadIdx.x == 0) {
             double t = log_mode ? -INFINITY : 0.0;
             for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t = fmax(t, smax[w]);
-            mx[r.mx] = log_mode ? (isfinite(t) ? okey(t) : 0ull)
-                                : (unsigned long long)__double_as_longlong(t);
+            const unsigned long long k = log_mode ? (isfinite(t) ? okey(t) : 0ull)
+                                                  : (unsigned long long)__double_as_longlong(t);
+            if (r.size <= blockDim.x) mx[r.mx] = k;
+            else if (k) atomicMax(mx + r.mx, k);   // zeroed at the start of every run
         }
     } else {
+        if (blockIdx.y) return;
         int v = r.var, c = card[v];
         int nb = r.beta ? nbeta : 1;
         if (r.slice_of_var >= 0) {
@@ -97,12 +105,13 @@ __global__ void k_leaves(const LeafRec *recs, const double *tables, const int *c
 }
 
 template <typename T>
-void launch_leaves(const LeafRec *recs, int nrec, const double *tables, const int *card,
-                   int nvars, const int32_t *evid, int nbeta, int log_mode, T *base,
+void launch_leaves(const LeafRec *recs, int nrec, int64_t largest, const double *tables,
+                   const int *card, int nvars, const int32_t *evid, int nbeta, int log_mode, T *base,
                    unsigned long long *mx, const int *flags, const int32_t *slice_val,
                    cudaStream_t st) {
     if (nrec <= 0) return;
-    k_leaves<T><<<nrec, 256, 0, st>>>(recs, tables, card, nvars, evid, nbeta, log_mode, base, mx,
+    const int64_t parts = std::min<int64_t>((largest + 255) / 256, 256);
+    k_leaves<T><<<dim3((unsigned)nrec, (unsigned)std::max<int64_t>(1, parts)), 256, 0, st>>>(recs, tables, card, nvars, evid, nbeta, log_mode, base, mx,
                                       flags, slice_val);
 }
 
@@ -745,7 +754,8 @@ void launch_cdf_blocks(const CDesc &d, int64_t rows, int bs, double *cdf, cudaSt
 }
 
 #define INST(T)                                                                                  \
-    template void launch_leaves<T>(const LeafRec *, int, const double *, const int *, int,      \
+    template void launch_leaves<T>(const LeafRec *, int, int64_t, const double *, const int *,  \
+                                   int,                                                         \
                                    const int32_t *, int, int, T *, unsigned long long *,        \
                                    const int *, const int32_t *, cudaStream_t);                 \
     template void launch_logz<T>(int, const T *, int, const unsigned long long *,              \

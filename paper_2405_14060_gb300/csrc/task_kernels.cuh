@@ -71,8 +71,8 @@ struct alignas(16) SampLab {
 };
 
 template <typename T>
-void launch_leaves(const LeafRec *recs, int nrec, const double *tables, const int *card,
-                   int nvars, const int32_t *evid, int nbeta, int log_mode, T *base,
+void launch_leaves(const LeafRec *recs, int nrec, int64_t largest, const double *tables,
+                   const int *card, int nvars, const int32_t *evid, int nbeta, int log_mode, T *base,
                    unsigned long long *mx, const int *flags, const int32_t *slice_val,
                    cudaStream_t st);
 // Slice combination (sum over slice assignments, Sec. "Tensor networks":
