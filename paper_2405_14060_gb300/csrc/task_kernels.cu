@@ -457,35 +457,38 @@ __device__ __forceinline__ double uniform01(uint64_t sample, uint32_t node, uint
 // k_cdf_blocks where the executor planned them.  16 x 16 grid, FP64, 100000
 // samples (166 drawing nodes of 991, one with 4096 entries): 26.2 ms with
 // values in global memory, every node visited and two full scans; a whole call
-// (forward pass and copy to the host included) went from 27.7 to 3.0 ms.
+// (forward pass and copy to the host included) went from 27.7 to 3.0 ms; with the
+// draws of up to eight entries on integer comparisons the kernel went from 870 to
+// 715 us.
 
 // Draw among N or fewer summed assignments held in registers.
 template <typename T, int N>
 __device__ __forceinline__ int64_t samp_small(const T *A, const T *B,
                                               const longlong2 *__restrict__ kt, int K, double u) {
-    double w[N], tot = 0, c = 0;
+    // running sums: the last is the total, and the draw compares with each.
+    // Sums of non-negative values order like their bits, and integer comparisons
+    // leave the FP64 pipe (two operations a clock and SM, what bounds the kernel)
+    // to the products and sums
+    double c[N];
+    unsigned long long w[N];
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-        w[k] = 0;
+        double v = 0;
         if (k < K) {
             const longlong2 o = __ldg(kt + k);
-            w[k] = (double)A[o.x] * (double)B[o.y];
+            v = (double)A[o.x] * (double)B[o.y];
         }
+        w[k] = dbits(v);
+        c[k] = k == 0 ? v : c[k - 1] + v;
     }
-#pragma unroll
-    for (int k = 0; k < N; ++k)
-        if (k < K) tot += w[k];
-    const double r0 = u * tot;
+    const unsigned long long r0 = dbits(u * c[N - 1]);
     int pick = K - 1;
     bool done = false;
 #pragma unroll
     for (int k = 0; k < N; ++k)
-        if (k < K) {
-            c += w[k];
-            if (!done && r0 < c && w[k] > 0) {
-                pick = k;
-                done = true;
-            }
+        if (!done && r0 < dbits(c[k]) && w[k] != 0ull) {
+            pick = k;
+            done = true;
         }
     return pick;
 }
