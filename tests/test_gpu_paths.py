@@ -163,3 +163,26 @@ def test_gemm_fp32_tiles(m, n, k, spec):
                     [letters.index(l) for l in c], C, prec="fp32")
     err = ((C.double() - ref).abs() / ref).max().item()
     assert err <= (k + 1) * 6e-8
+
+
+# tensor-core GEMM: rows and columns around its 128 x 256 (long summed space:
+# 256 x 256) tiles and the 32-column chunks of the epilogue, row lengths that
+# allow 16-byte stores or not, short (persistent) and long summed spaces
+@pytest.mark.parametrize("m,n,k", [(64, 64, 64), (127, 257, 100), (129, 290, 64), (300, 770, 96),
+                                   (1000, 260, 72), (200, 300, 2300), (520, 515, 4500)])
+@pytest.mark.parametrize("prec", ["tf32", "bf16"])
+@pytest.mark.parametrize("spec", ["mk,nk->mn", "gmk,gkn->gmn"])
+def test_tc_gemm_edges(m, n, k, prec, spec):
+    (a, b), c = spec.split("->")[0].split(","), spec.split("->")[1]
+    letters = "gkmn"
+    size = dict(g=2, k=k, m=m, n=n)
+    rng = np.random.default_rng(m + n * k)
+    A = torch.tensor(rng.random([size[l] for l in a]), dtype=torch.float32, device="cuda")
+    B = torch.tensor(rng.random([size[l] for l in b]), dtype=torch.float32, device="cuda")
+    ref = torch.einsum(spec, A.double(), B.double())
+    C = torch.full([size[l] for l in c], float("nan"), dtype=torch.float32, device="cuda")
+    tn.contract_dev([size[l] for l in letters], [letters.index(l) for l in a], A,
+                    [letters.index(l) for l in b], B, [letters.index(l) for l in c], C, prec=prec)
+    # two roundings of each product's inputs (2^-11 TF32 truncated to 2^-10, 2^-9 BF16)
+    err = ((C.double() - ref).abs() / ref).max().item()
+    assert err <= (2 * 2.0 ** -10 if prec == "tf32" else 2 * 2.0 ** -8)
