@@ -511,12 +511,16 @@ void launch_permute(const PDesc &p, cudaStream_t st) {
 
 // ------------------------------------------------------------ tcgen05 GEMM
 
-constexpr int TC_BM = 128, TC_BN = 256, TC_STAGES = 4;
+constexpr int TC_BM = 128, TC_BN = 256;
 constexpr int TC_XBYTES = TC_BM * 128, TC_YBYTES = TC_BN * 128;    // one 128-byte K slab
 // epilogue staging: per warp, 32 rows of 32 columns (rows of 36 floats, so that
 // 16-byte accesses along and across rows meet no bank conflict)
 constexpr int TC_EROW = 36, TC_EPI = 4 * 32 * TC_EROW * 4;
-constexpr int TC_SMEM = TC_STAGES * (TC_XBYTES + TC_YBYTES) + TC_EPI + 1024 + 256;
+// MT blocks of 128 rows a tile: K slabs in the ring, shared memory
+constexpr int tc_stages(int mt) { return mt == 2 ? 3 : 4; }
+constexpr int tc_smem(int mt) {
+    return tc_stages(mt) * (mt * TC_XBYTES + TC_YBYTES) + TC_EPI + 1024 + 256;
+}
 constexpr int TC_THREADS = 192;   // warps 0-3 epilogue, warp 4 MMA issuer, warp 5 TMA producer
 
 struct TCParams {
@@ -537,6 +541,7 @@ struct TCParams {
 // so that the tiles processed together read a few row panels of X and a few
 // column panels of Y (which then stay in L2) rather than all of Y.
 constexpr int TC_GROUP = 8;
+template <int MT>
 __device__ __forceinline__ void tc_tile(const TCParams &p, int64_t t, int &bz, int64_t &m0,
                                         int64_t &n0) {
     const int64_t per_b = p.ntn * p.ntm;
@@ -545,39 +550,41 @@ __device__ __forceinline__ void tc_tile(const TCParams &p, int64_t t, int &bz, i
     const int64_t per_g = (int64_t)TC_GROUP * p.ntn;
     const int64_t grp = rem / per_g, loc = rem - grp * per_g;
     const int64_t rows = min((int64_t)TC_GROUP, p.ntm - grp * TC_GROUP);
-    m0 = (grp * TC_GROUP + loc % rows) * TC_BM;
+    m0 = (grp * TC_GROUP + loc % rows) * (TC_BM * MT);
     n0 = (loc / rows) * TC_BN;
 }
 
 // Persistent: CTA b takes tiles b, b + grid, ...  The TMA warp fills a ring
-// of TC_STAGES K slabs (X and Y tiles, 128-byte swizzle) across tile
+// of three or four K slabs (X and Y tiles, 128-byte swizzle) across tile
 // boundaries; the MMA warp accumulates tile i into one of two 256-column TMEM
 // buffers (i & 1) while the four epilogue warps drain the other one, so a
 // tile's TMEM -> global epilogue overlaps the next tile's MMAs.  Every wait
 // is bounded: on a timeout the error flag is set, the producer waits for the
 // copies it issued, the MMA warp for the MMAs it issued, and TMEM is freed.
-template <int BF16>
+template <int BF16, int MT>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_tc_gemm(const __grid_constant__ CUtensorMap tx, const __grid_constant__ CUtensorMap ty,
               const __grid_constant__ TCParams p) {
+    constexpr int S = tc_stages(MT), XB = MT * TC_XBYTES;
+    constexpr int NB = MT == 2 ? 1 : 2;   // accumulators of a tile that TMEM holds
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t *sX = smem;
-    uint8_t *sY = smem + TC_STAGES * TC_XBYTES;
+    uint8_t *sY = smem + S * XB;
     // barriers: full[S], empty[S], tfull[2], tempty[2], fin; then the TMEM slot
-    float *sE = (float *)(sY + TC_STAGES * TC_YBYTES);
+    float *sE = (float *)(sY + S * TC_YBYTES);
     uint64_t *bars = (uint64_t *)((uint8_t *)sE + TC_EPI);
-    uint32_t *tslot = (uint32_t *)(bars + 2 * TC_STAGES + 5);
+    uint32_t *tslot = (uint32_t *)(bars + 2 * S + 5);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + TC_STAGES),
-                   tfull0 = smem_u32(bars + 2 * TC_STAGES),
-                   tempty0 = smem_u32(bars + 2 * TC_STAGES + 2),
-                   fin = smem_u32(bars + 2 * TC_STAGES + 4);
+    const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + S),
+                   tfull0 = smem_u32(bars + 2 * S),
+                   tempty0 = smem_u32(bars + 2 * S + 2),
+                   fin = smem_u32(bars + 2 * S + 4);
     const int mine = p.ntiles > (int64_t)blockIdx.x
                          ? (int)((p.ntiles - 1 - (int64_t)blockIdx.x) / gridDim.x) + 1
                          : 0;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < TC_STAGES; ++s) {
+        for (int s = 0; s < S; ++s) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full0 + 8 * s));
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(empty0 + 8 * s));
         }
@@ -610,24 +617,27 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             for (int li = 0; li < mine && ok; ++li) {
                 int bz;
                 int64_t m0, n0;
-                tc_tile(p, (int64_t)blockIdx.x + (int64_t)li * gridDim.x, bz, m0, n0);
+                tc_tile<MT>(p, (int64_t)blockIdx.x + (int64_t)li * gridDim.x, bz, m0, n0);
                 for (int kt = 0; kt < KT; ++kt, ++q) {
-                    const int s = q % TC_STAGES;
-                    if (q >= TC_STAGES &&
-                        !mbar_wait(empty0 + 8 * s, ((q / TC_STAGES) - 1) & 1, p.err, p.wait_ns)) {
+                    const int s = q % S;
+                    if (q >= S &&
+                        !mbar_wait(empty0 + 8 * s, ((q / S) - 1) & 1, p.err, p.wait_ns)) {
                         ok = false;
                         break;
                     }
                     const uint32_t fb = full0 + 8 * s;
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb),
-                                 "r"(TC_XBYTES + TC_YBYTES)
+                                 "r"(XB + TC_YBYTES)
                                  : "memory");
                     const int kx = kt * (BF16 ? 64 : 32);
-                    asm volatile(
-                        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
-                        " [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(smem_u32(sX + s * TC_XBYTES)),
-                        "l"(&tx), "r"(fb), "r"(kx), "r"((int)m0), "r"(bz)
-                        : "memory");
+#pragma unroll
+                    for (int h = 0; h < MT; ++h)   // rows past the end are filled with zeros
+                        asm volatile(
+                            "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
+                            " [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(
+                                smem_u32(sX + s * XB + h * TC_XBYTES)),
+                            "l"(&tx), "r"(fb), "r"(kx), "r"((int)m0 + h * TC_BM), "r"(bz)
+                            : "memory");
                     asm volatile(
                         "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
                         " [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(smem_u32(sY + s * TC_YBYTES)),
@@ -637,8 +647,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             }
             // the last transfers issued land before the CTA exits (already
             // the case when the MMA warp consumed them; it may have given up)
-            for (int r = q > TC_STAGES ? q - TC_STAGES : 0; r < q; ++r)
-                mbar_drain(full0 + 8 * (r % TC_STAGES), (r / TC_STAGES) & 1, p.err);
+            for (int r = q > S ? q - S : 0; r < q; ++r)
+                mbar_drain(full0 + 8 * (r % S), (r / S) & 1, p.err);
         }
         __syncwarp();
     } else if (warp == 4) {
@@ -653,25 +663,27 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             int q = 0;
             bool ok = true;
             for (int li = 0; li < mine && ok; ++li) {
-                const int a = li & 1;
-                // the epilogue has drained this TMEM buffer (tile li - 2)
-                if (li >= 2 && !mbar_wait(tempty0 + 8 * a, ((li >> 1) - 1) & 1, p.err, p.wait_ns)) {
+                const int a = li % NB;
+                // the epilogue has drained this TMEM buffer (tile li - NB)
+                if (li >= NB && !mbar_wait(tempty0 + 8 * a, (li / NB - 1) & 1, p.err, p.wait_ns)) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
-                const uint32_t acc_t = tmem + (uint32_t)(a * TC_BN);
+                const uint32_t acc_0 = tmem + (uint32_t)(a * TC_BN);
                 for (int kt = 0; kt < KT; ++kt, ++q) {
-                    const int s = q % TC_STAGES;
-                    if (!mbar_wait(full0 + 8 * s, (q / TC_STAGES) & 1, p.err, p.wait_ns)) {
+                    const int s = q % S;
+                    if (!mbar_wait(full0 + 8 * s, (q / S) & 1, p.err, p.wait_ns)) {
                         ok = false;
                         break;
                     }
                     tc_fence_after();
-                    const uint64_t ad = sdesc_sw128(smem_u32(sX + s * TC_XBYTES));
                     const uint64_t bd = sdesc_sw128(smem_u32(sY + s * TC_YBYTES));
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk) {
+                    for (int hk = 0; hk < 4 * MT; ++hk) {
+                        const int kk = hk & 3, h = hk >> 2;   // K step, block of rows
+                        const uint64_t ad = sdesc_sw128(smem_u32(sX + s * XB + h * TC_XBYTES));
+                        const uint32_t acc_t = acc_0 + (uint32_t)(h * TC_BN);
                         const uint32_t accum = (kt | kk) ? 1u : 0u;
                         if (BF16)
                             asm volatile(
@@ -711,78 +723,84 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         // warp w drains TMEM lanes 32w..32w+31 (rows of the tile)
         const float sxs = p.mxsx ? pow2neg<float>(exp_of_bits(*p.mxsx)) : 1.f;
         for (int li = 0; li < mine; ++li) {
-            const int a = li & 1;
-            bool have = mbar_wait(tfull0 + 8 * a, (li >> 1) & 1, p.err, p.wait_ns);
+            const int a = li % NB;
+            bool have = mbar_wait(tfull0 + 8 * a, (li / NB) & 1, p.err, p.wait_ns);
             have = __all_sync(0xffffffffu, have);
             if (!have) break;
             tc_fence_after();
             int bz;
             int64_t m0, n0;
-            tc_tile(p, (int64_t)blockIdx.x + (int64_t)li * gridDim.x, bz, m0, n0);
-            const int64_t row = m0 + warp * 32 + lane;
-            float mx = 0;
-            float *D = p.D + (int64_t)bz * p.bsd;
-            float *we = sE + warp * 32 * TC_EROW;
-            const bool dvec = (p.ldd & 3) == 0 && (p.bsd & 3) == 0 && ((uintptr_t)p.D & 15) == 0;
-            for (int ch = 0; ch < TC_BN / 32; ++ch) {
-                if (n0 + ch * 32 >= p.C) break;   // warp-uniform: no columns left
-                uint32_t r[32];
-                const uint32_t ta =
-                    tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(a * TC_BN + ch * 32);
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, "
-                    "%10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, "
-                    "%26, %27, %28, %29, %30, %31}, [%32];"
-                    : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
-                      "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]),
-                      "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]),
-                      "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-                      "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]),
-                      "=r"(r[30]), "=r"(r[31])
-                    : "r"(ta));
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                // lanes hold rows: through shared memory, so that a warp stores
-                // 128 contiguous bytes of a row at a time (a lane writing its own
-                // row touched 32 half-used sectors per instruction: rows 3000, 777
-                // columns, TF32 38 us, 24 us now; 4.3 GB of results of the batched
-                // workload 2.06 ms, 1.60 ms now)
-                const int64_t c0 = n0 + ch * 32;
-                const bool in = row < p.R;
-                __syncwarp();   // the previous chunk has been read
+            tc_tile<MT>(p, (int64_t)blockIdx.x + (int64_t)li * gridDim.x, bz, m0, n0);
+#pragma unroll 1
+            for (int h = 0; h < MT; ++h) {
+                const int64_t row = m0 + h * TC_BM + warp * 32 + lane;
+                float mx = 0;
+                float *D = p.D + (int64_t)bz * p.bsd;
+                float *we = sE + warp * 32 * TC_EROW;
+                const bool dvec = (p.ldd & 3) == 0 && (p.bsd & 3) == 0 && ((uintptr_t)p.D & 15) == 0;
+                for (int ch = 0; ch < TC_BN / 32; ++ch) {
+                    if (n0 + ch * 32 >= p.C) break;   // warp-uniform: no columns left
+                    uint32_t r[32];
+                    const uint32_t ta =
+                        tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((a + h) * TC_BN + ch * 32);
+                    asm volatile(
+                        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, "
+                        "%10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, "
+                        "%26, %27, %28, %29, %30, %31}, [%32];"
+                        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+                          "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]),
+                          "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]),
+                          "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+                          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]),
+                          "=r"(r[30]), "=r"(r[31])
+                        : "r"(ta));
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    // lanes hold rows: through shared memory, so that a warp stores
+                    // 128 contiguous bytes of a row at a time (a lane writing its own
+                    // row touched 32 half-used sectors per instruction: rows 3000, 777
+                    // columns, TF32 38 us, 24 us now; 4.3 GB of results of the batched
+                    // workload 2.06 ms, 1.60 ms now)
+                    const int64_t c0 = n0 + ch * 32;
+                    const bool in = row < p.R;
+                    __syncwarp();   // the previous chunk has been read
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    float4 v;
-                    v.x = __uint_as_float(r[4 * j + 0]) * sxs;
-                    v.y = __uint_as_float(r[4 * j + 1]) * sxs;
-                    v.z = __uint_as_float(r[4 * j + 2]) * sxs;
-                    v.w = __uint_as_float(r[4 * j + 3]) * sxs;
-                    *(float4 *)(we + lane * TC_EROW + 4 * j) = v;
-                    // columns past C are products of zero-filled rows of Y
-                    if (in) mx = fmaxf(mx, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
-                }
-                __syncwarp();
-                const int64_t rw = m0 + warp * 32;   // the warp's first row
-                if (dvec && c0 + 32 <= p.C) {
-                    const int rl = lane >> 3, cq = (lane & 7) * 4;
-                    float *d = D + (rw + rl) * p.ldd + c0 + cq;
+                    for (int j = 0; j < 8; ++j) {
+                        float4 v;
+                        v.x = __uint_as_float(r[4 * j + 0]) * sxs;
+                        v.y = __uint_as_float(r[4 * j + 1]) * sxs;
+                        v.z = __uint_as_float(r[4 * j + 2]) * sxs;
+                        v.w = __uint_as_float(r[4 * j + 3]) * sxs;
+                        *(float4 *)(we + lane * TC_EROW + 4 * j) = v;
+                        // columns past C are products of zero-filled rows of Y
+                        if (in) mx = fmaxf(mx, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+                    }
+                    __syncwarp();
+                    const int64_t rw = m0 + h * TC_BM + warp * 32;   // the warp's first row
+                    if (dvec && c0 + 32 <= p.C) {
+                        const int rl = lane >> 3, cq = (lane & 7) * 4;
+                        float *d = D + (rw + rl) * p.ldd + c0 + cq;
 #pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        if (rw + 4 * q + rl < p.R)
-                            *(float4 *)(d + (int64_t)(4 * q) * p.ldd) =
-                                *(const float4 *)(we + (4 * q + rl) * TC_EROW + cq);
-                } else if (c0 + lane < p.C) {
-                    const int nr = (int)min((int64_t)32, p.R - rw);
-                    for (int q = 0; q < nr; ++q)
-                        D[(rw + q) * p.ldd + c0 + lane] = we[q * TC_EROW + lane];
+                        for (int q = 0; q < 8; ++q)
+                            if (rw + 4 * q + rl < p.R)
+                                *(float4 *)(d + (int64_t)(4 * q) * p.ldd) =
+                                    *(const float4 *)(we + (4 * q + rl) * TC_EROW + cq);
+                    } else if (c0 + lane < p.C) {
+                        const int nr = (int)min((int64_t)32, p.R - rw);
+                        for (int q = 0; q < nr; ++q)
+                            D[(rw + q) * p.ldd + c0 + lane] = we[q * TC_EROW + lane];
+                    }
                 }
+                if (h == MT - 1) {
+                    // this TMEM buffer may take the MMAs of tile li + NB
+                    tc_fence_before();
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty0 + 8 * a)
+                                 : "memory");
+                }
+                const int64_t beta = p.beta_div_batch > 0 ? (int64_t)bz / p.beta_div_batch
+                                     : p.beta_div_row > 0 ? (row < p.R ? row : p.R - 1) / p.beta_div_row
+                                                          : 0;
+                record_max(p.mxd, beta, row < p.R, (double)mx);
             }
-            // this TMEM buffer may take the MMAs of tile li + 2
-            tc_fence_before();
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty0 + 8 * a) : "memory");
-            const int64_t beta = p.beta_div_batch > 0 ? (int64_t)bz / p.beta_div_batch
-                                 : p.beta_div_row > 0 ? (row < p.R ? row : p.R - 1) / p.beta_div_row
-                                                      : 0;
-            record_max(p.mxd, beta, row < p.R, (double)mx);
         }
     }
     tc_fence_before();
@@ -834,8 +852,10 @@ static bool make_map(CUtensorMap *m, const void *base, int64_t K, int64_t rows, 
 cudaError_t launch_tc_gemm(const GDesc &g, int *err_flag, cudaStream_t st) {
     static std::once_flag once;
     std::call_once(once, [] {
-        cudaFuncSetAttribute(k_tc_gemm<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
-        cudaFuncSetAttribute(k_tc_gemm<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
+        cudaFuncSetAttribute(k_tc_gemm<0, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem(1));
+        cudaFuncSetAttribute(k_tc_gemm<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem(1));
+        cudaFuncSetAttribute(k_tc_gemm<0, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem(2));
+        cudaFuncSetAttribute(k_tc_gemm<1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem(2));
     });
     bool bf16 = g.xtype == E_BF16;
     int es = bf16 ? 2 : 4;
@@ -878,9 +898,27 @@ cudaError_t launch_tc_gemm(const GDesc &g, int *err_flag, cudaStream_t st) {
                   ? n
                   : 152;
     }
+    // long K: 256 x 256 tiles, whose accumulators fill TMEM, when that costs no
+    // extra round of tiles.  128 x 256 tiles need 43 (TF32) or 85 (BF16)
+    // multiply-adds a byte from L2, 23 to 26 TB/s at the tensor peak; these need
+    // three quarters of that.  16384-long BF16 nodes of the batched workload 2.70 ->
+    // 2.29 ms (1.92 PFLOP/s), 4096^3 TF32 nodes of the 24 x 24 grid 219 -> 175 us.
+    // At 64 slabs and fewer the epilogue, which then overlaps nothing, costs as
+    // much as it gains (4096^3 BF16 97 us either way) or more (K = 1024: 1.61 ms
+    // against 2.26).
+    const int64_t ntm2 = (g.R + 2 * TC_BM - 1) / (2 * TC_BM), t2 = p.ntn * ntm2 * g.batch;
+    const bool wide = p.kt > 64 && g.R < (1LL << 30) &&
+                      20 * ((t2 + nsm - 1) / nsm) <= 11 * ((p.ntiles + nsm - 1) / nsm);
+    if (wide) {
+        p.ntm = ntm2;
+        p.ntiles = t2;
+        if (bf16) k_tc_gemm<1, 2><<<(unsigned)t2, TC_THREADS, tc_smem(2), st>>>(mx, my, p);
+        else k_tc_gemm<0, 2><<<(unsigned)t2, TC_THREADS, tc_smem(2), st>>>(mx, my, p);
+        return cudaGetLastError();
+    }
     dim3 grid((unsigned)(p.kt <= 64 ? std::min<int64_t>(p.ntiles, nsm) : p.ntiles), 1, 1);
-    if (bf16) k_tc_gemm<1><<<grid, TC_THREADS, TC_SMEM, st>>>(mx, my, p);
-    else k_tc_gemm<0><<<grid, TC_THREADS, TC_SMEM, st>>>(mx, my, p);
+    if (bf16) k_tc_gemm<1, 1><<<grid, TC_THREADS, tc_smem(1), st>>>(mx, my, p);
+    else k_tc_gemm<0, 1><<<grid, TC_THREADS, tc_smem(1), st>>>(mx, my, p);
     return cudaGetLastError();
 }
 

@@ -25,7 +25,7 @@ __device__ __forceinline__ int exp_bits(unsigned long long b) {
 // multiplies in the slicing T_{V|E=e} of Eq. pr.  In the log domain ones are
 // 0 and zeros are -inf.  Each leaf records its maximum for rescaling.  One block
 // per 256 entries of a table (a logarithm is some 50 FP64 operations, at two a
-// clock and SM: a 2^14-entry external leaf took 190 us in one block, LEAF_NOW).
+// clock and SM: an 18432-entry external leaf took 190 us in one block, 19 us now).
 template <typename T>
 __global__ void k_leaves(const LeafRec *recs, const double *tables, const int *card, int nvars,
                          const int32_t *evid, int nbeta, int log_mode, T *base,
