@@ -435,13 +435,36 @@ __global__ void __launch_bounds__(kThreads) k_bgemm_direct(const __grid_constant
 #pragma unroll
         for (int j = 0; j < TN; ++j)
             bo[j] = __ldg(d.tbn + (tp.n0 + j < d.N ? tp.n0 + j : d.N - 1));
+        // what the stores need is on its way beside the operands
+        int32_t cn[TN];
+#pragma unroll
+        for (int j = 0; j < TN; ++j) cn[j] = __ldg(d.tcn + (tp.n0 + j < d.N ? tp.n0 + j : d.N - 1));
+        T *Cb = (T *)d.C + tp.beta * d.bsc + __ldg(d.tcg + tp.g) + __ldg(d.tcm + (om ? m : 0));
+        const unsigned long long ma = d.mxa ? d.mxa[tp.beta * d.mxa_bs] : 0ull;
+        const unsigned long long mb = d.mxb ? d.mxb[tp.beta * d.mxb_bs] : 0ull;
         T acc[TN];
 #pragma unroll
         for (int j = 0; j < TN; ++j) acc[j] = T(0);
         const int k0 = (int)(tp.split * d.kchunk);
         const int k1 = (int)min(d.K, (int64_t)k0 + d.kchunk);
-#pragma unroll 4
-        for (int k = k0 + ks; k < k1; k += KL) {
+        constexpr int U = TN == 1 ? 8 : TN == 2 ? 6 : 4;   // summed indices loaded together
+        int k = k0 + ks;
+        for (; k + (U - 1) * KL < k1; k += U * KL) {
+            T a[U], b[U][TN];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int32_t ka = __ldg(d.tak + k + u * KL), kb = __ldg(d.tbk + k + u * KL);
+                a[u] = __ldg(A + ka);
+#pragma unroll
+                for (int j = 0; j < TN; ++j) b[u][j] = __ldg(B + (bo[j] + kb));
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int j = 0; j < TN; ++j) acc[j] += a[u] * b[u][j];
+        }
+#pragma unroll 2
+        for (; k < k1; k += KL) {
             const int32_t ka = __ldg(d.tak + k), kb = __ldg(d.tbk + k);
             const T a = __ldg(A + ka);
 #pragma unroll
@@ -458,15 +481,14 @@ __global__ void __launch_bounds__(kThreads) k_bgemm_direct(const __grid_constant
             for (int j = 0; j < TN; ++j)
                 if (st && tp.n0 + j < d.N) P[(tp.n0 + j) * d.M + m] = acc[j];
         } else {
-            const T sca = d.mxa ? pow2neg<T>(exp_of_bits(d.mxa[tp.beta * d.mxa_bs])) : T(1);
-            const T scb = d.mxb ? pow2neg<T>(exp_of_bits(d.mxb[tp.beta * d.mxb_bs])) : T(1);
+            const T sca = d.mxa ? pow2neg<T>(exp_of_bits(ma)) : T(1);
+            const T scb = d.mxb ? pow2neg<T>(exp_of_bits(mb)) : T(1);
             const T sc = sca * scb;
-            T *Cb = (T *)d.C + tp.beta * d.bsc + __ldg(d.tcg + tp.g) + __ldg(d.tcm + (om ? m : 0));
 #pragma unroll
             for (int j = 0; j < TN; ++j)
                 if (st && tp.n0 + j < d.N) {
                     const T v = acc[j] * sc;
-                    Cb[__ldg(d.tcn + tp.n0 + j)] = v;
+                    Cb[cn[j]] = v;
                     mx = mx > v ? mx : v;
                 }
         }
