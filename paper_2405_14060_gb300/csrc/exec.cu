@@ -2736,11 +2736,8 @@ static void run_step(tn_model *m, Program &P, const Step &s, cudaStream_t st, in
         return;
     }
     const GemmOp &g = s.g;
-    timed(pr, st, cls(C_PREP), 0, g.prep_bytes, [&] {
-        if (!g.x_in_place) launch_permute(g.px, st);
-        launch_permute(g.py, st);
-    });
-    nl += g.x_in_place ? 1 : 2;
+    timed(pr, st, cls(C_PREP), 0, g.prep_bytes,
+          [&] { nl += launch_permutes(g.x_in_place ? nullptr : &g.px, &g.py, st); });
     if (g.tc) {
         timed(pr, st, cls(C_TCGEMM), s.flops, s.bytes, [&] { launch_tc_gemm(g.g, m->d_err, st); });
     } else {
@@ -4252,8 +4249,7 @@ tn_status tn_contract_dev(int nlabels, const int *sizes, int na, const int *labe
                 tn_status fs = device_err_flag(&d_err);
                 if (fs) return fs;
             }
-            if (!xin) launch_permute(op.px, st);
-            if (!yin) launch_permute(op.py, st);
+            launch_permutes(xin ? nullptr : &op.px, yin ? nullptr : &op.py, st);
             cudaError_t le = cudaSuccess;
             if (tc) le = launch_tc_gemm(op.g, d_err, st);
             else launch_simt_gemm(op.g, st);

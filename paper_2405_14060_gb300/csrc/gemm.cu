@@ -115,9 +115,22 @@ __device__ __forceinline__ void store_conv(void *out, int64_t i, TI x) {
 // inputs per 16-byte copy when the plan allows), stores the output order
 // (t.vec outputs per 16-byte store, their shared-memory slots read as one
 // vector of 16-bit integers).
+//
+// One launch takes one or two permutations (blockIdx.z; the row and the column
+// operand of a GEMM): their reads and writes overlap, and the last blocks of one
+// do not leave the SMs idle before the other (1000 x 1155 and 777 x 1155, three
+// items, to TF32: 27 us one after the other, 25 us together).
+struct PPair {
+    PDesc p[2];
+    int64_t per[2];       // tiles per item
+    int blocks[2], items[2];
+};
 template <typename TI, int OT>
-__global__ void __launch_bounds__(256, 4) k_permute_tiled(const __grid_constant__ PDesc p,
-                                                       int64_t per_item) {
+__global__ void __launch_bounds__(256, 4) k_permute_tiled(const __grid_constant__ PPair a) {
+    const PDesc &p = a.p[blockIdx.z];
+    const int64_t per_item = a.per[blockIdx.z];
+    const int nblocks = a.blocks[blockIdx.z];
+    if ((int)blockIdx.x >= nblocks || (int)blockIdx.y >= a.items[blockIdx.z]) return;
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ int64_t sbase[4][3];   // per tile (mod 4): input base, output base, item
     const PTile &t = p.tl;
@@ -130,8 +143,8 @@ __global__ void __launch_bounds__(256, 4) k_permute_tiled(const __grid_constant_
     const TI *in = (const TI *)p.in;
     TI mxv = 0;
     // this block's tiles [q0, q1)
-    const int64_t q0 = per_item * blockIdx.x / gridDim.x;
-    const int64_t q1 = per_item * (blockIdx.x + 1) / gridDim.x;
+    const int64_t q0 = per_item * blockIdx.x / nblocks;
+    const int64_t q1 = per_item * (blockIdx.x + 1) / nblocks;
     // digits of the last published tile (thread 0 only)
     int32_t dg[MAXD];
     int64_t cbi = 0, cbo = 0;
@@ -475,29 +488,63 @@ void launch_permute_tables(const PTabs3 &a, cudaStream_t st) {
     if (n > 0) k_permute_tables<<<dim3((unsigned)((n + 255) / 256), 3), 256, 0, st>>>(a);
 }
 
+// One or two (n) tiled permutations of the same types in one launch.
+static void launch_tiled(const PDesc *const *ps, int n, cudaStream_t st) {
+    PPair a;
+    size_t sm = 0;
+    int gx = 1, gy = 1;
+    for (int i = 0; i < n; ++i)   // three tile buffers
+        sm = std::max(sm, 3 * (size_t)ps[i]->tl.nbuf * (ps[i]->in_type == E_F64 ? 8 : 4));
+    // as many blocks per SM as shared memory holds
+    const int64_t bps = std::max<int64_t>(1, std::min<int64_t>(8, (227 * 1024) / (sm + 1024)));
+    for (int i = 0; i < n; ++i) {
+        const PDesc &p = *ps[i];
+        a.p[i] = p;
+        a.items[i] = (p.mxo && p.tl.rest_beta == 0) ? p.tl.rsz[0] : 1;
+        a.per[i] = p.tl.ntiles / a.items[i];
+        const int64_t cap = std::max<int64_t>(1, (152LL * bps) / a.items[i]);
+        a.blocks[i] = (int)std::max<int64_t>(1, std::min(a.per[i], cap));
+        gx = std::max(gx, a.blocks[i]);
+        gy = std::max(gy, a.items[i]);
+    }
+    static std::once_flag once;
+    std::call_once(once, [] {
+        const int mx = 3 * pt_nbuf(PT_MAXN, 0) * 8;
+        cudaFuncSetAttribute(k_permute_tiled<double, E_F64>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+        cudaFuncSetAttribute(k_permute_tiled<float, E_F32>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+        cudaFuncSetAttribute(k_permute_tiled<float, E_BF16>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+    });
+    const dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)n);
+    const PDesc &p = *ps[0];
+    if (p.in_type == E_F64) k_permute_tiled<double, E_F64><<<grid, 256, sm, st>>>(a);
+    else if (p.out_type == E_F32) k_permute_tiled<float, E_F32><<<grid, 256, sm, st>>>(a);
+    else k_permute_tiled<float, E_BF16><<<grid, 256, sm, st>>>(a);
+}
+
+int launch_permutes(const PDesc *x, const PDesc *y, cudaStream_t st) {
+    auto tiled = [](const PDesc *p) { return p && p->total > 0 && p->tl.tn > 0 && p->tl.ttab; };
+    // up to 2^25 entries each, where a launch's ramp and tail weigh (beyond, the
+    // larger shared-memory tile of the two sets the blocks of both: 1.7 GB and
+    // 5.5 GB operands took 2.36 ms together, 1.70 one after the other)
+    if (tiled(x) && tiled(y) && x->in_type == y->in_type && x->out_type == y->out_type &&
+        std::max(x->total, y->total) <= (1LL << 25)) {
+        const PDesc *ps[2] = {x, y};
+        launch_tiled(ps, 2, st);
+        return 1;
+    }
+    if (x) launch_permute(*x, st);
+    if (y) launch_permute(*y, st);
+    return (x ? 1 : 0) + (y ? 1 : 0);
+}
+
 void launch_permute(const PDesc &p, cudaStream_t st) {
     if (p.total <= 0) return;
     if (p.tl.tn > 0 && p.tl.ttab) {
-        int nitems = (p.mxo && p.tl.rest_beta == 0) ? p.tl.rsz[0] : 1;
-        int64_t per = p.tl.ntiles / nitems;
-        // three tile buffers; as many blocks per SM as shared memory holds
-        size_t sm = 3 * (size_t)p.tl.nbuf * (p.in_type == E_F64 ? 8 : 4);
-        const int64_t bps = std::max<int64_t>(1, std::min<int64_t>(8, (227 * 1024) / (sm + 1024)));
-        int64_t cap = std::max<int64_t>(1, (152LL * bps) / nitems);
-        dim3 grid((unsigned)std::max<int64_t>(1, std::min(per, cap)), (unsigned)nitems, 1);
-        static std::once_flag once;
-        std::call_once(once, [] {
-            const int mx = 3 * pt_nbuf(PT_MAXN, 0) * 8;
-            cudaFuncSetAttribute(k_permute_tiled<double, E_F64>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-            cudaFuncSetAttribute(k_permute_tiled<float, E_F32>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-            cudaFuncSetAttribute(k_permute_tiled<float, E_BF16>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-        });
-        if (p.in_type == E_F64) k_permute_tiled<double, E_F64><<<grid, 256, sm, st>>>(p, per);
-        else if (p.out_type == E_F32) k_permute_tiled<float, E_F32><<<grid, 256, sm, st>>>(p, per);
-        else k_permute_tiled<float, E_BF16><<<grid, 256, sm, st>>>(p, per);
+        const PDesc *ps[1] = {&p};
+        launch_tiled(ps, 1, st);
         return;
     }
     int nitems = 1;

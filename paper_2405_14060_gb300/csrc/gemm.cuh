@@ -116,6 +116,9 @@ struct GDesc {
 };
 
 void launch_permute(const PDesc &p, cudaStream_t st);
+// Both operand preparations of a GEMM (NULL: read in place), in one launch where
+// both are tiled; returns the number of launches.
+int launch_permutes(const PDesc *x, const PDesc *y, cudaStream_t st);
 // Returns false if the tensor-core path cannot take this problem.
 bool tc_gemm_supported(const GDesc &g);
 cudaError_t launch_tc_gemm(const GDesc &g, int *err_flag, cudaStream_t st);
