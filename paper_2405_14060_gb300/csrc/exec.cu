@@ -959,6 +959,13 @@ static bool make_reduce(const std::vector<int> &card, const Labels &lx, bool bx,
     return true;
 }
 
+// Entries of its offset tables, and the most it takes: past that a contraction
+// in GEMM form stays on the tiled GEMM, any other on the strided kernels.
+static int64_t group_entries(int64_t G, int64_t M, int64_t N, int64_t K) {
+    return 3 * G + 2 * M + 2 * N + 2 * K;
+}
+constexpr int64_t kGroupEntries = 1LL << 26;
+
 // Batched strided GEMM: O[g, m, n] = sum_k X[g, m, k] Y[g, k, n] with the
 // label groups G (in X, Y and O), M (X and O), N (Y and O) and K (X and Y),
 // each label of O, X and Y in exactly one group (no label summed inside one
@@ -1014,8 +1021,7 @@ static bool make_bgemm(const std::vector<int> &card, const Labels &lx, bool bx, 
         return make_bgemm(card, ly, by, pery, Y, mxy, lx, bx, perx, X, mxx, lo, bo, pero, O, mxo,
                           nbeta, esz, d, tab, tc_orient, dims, true);
     if (perx >= (1LL << 31) || pery >= (1LL << 31) || pero >= (1LL << 31)) return false;
-    const int64_t ntab = 3 * d.G + 2 * d.M + 2 * d.N + 2 * d.K;
-    if (ntab > (1LL << 26)) return false;
+    if (group_entries(d.G, d.M, d.N, d.K) > kGroupEntries) return false;
     // the group holding each tensor's fastest label (of size > 1)
     auto in = [](const Labels &l, int v) { return std::find(l.begin(), l.end(), v) != l.end(); };
     d.a_kfast = in(K, fastest_of(lx)) ? 1 : 0;
@@ -1085,7 +1091,7 @@ static bool make_bgemm(const std::vector<int> &card, const Labels &lx, bool bx, 
         if (!ok) g.total = 0;   // filled here instead
     }
     const bool host = !dims || dims->total == 0;
-    tab.assign(host ? (size_t)ntab : 0, 0);
+    tab.assign(host ? (size_t)group_entries(d.G, d.M, d.N, d.K) : 0, 0);
     // offsets of every index of a group (labels in the given order, last
     // fastest) in one tensor
     auto fill = [&](const Labels &grp, const Labels &lt, const std::set<int> &st, int32_t *out) {
@@ -4199,9 +4205,10 @@ tn_status tn_contract_dev(int nlabels, const int *sizes, int na, const int *labe
         // the batched GEMM splits over blocks (100 x 130 x 4000: 6 tiles, 286 us
         // a call on the tiled GEMM, 73 there)
         const bool tcp = prec == TN_TF32 || prec == TN_BF16;
-        const bool direct = (dtype == 0 || (!tcp && few_gemm_tiles(prod(bt), prod(gm), prod(gn),
-                                                                   prod(gk)))) && prod(la) < (1LL << 31) && prod(lb) < (1LL << 31) &&
-                            prod(lc) < (1LL << 31);
+        const int64_t G = prod(bt), M = prod(gm), N = prod(gn), K = prod(gk);
+        const bool direct = (dtype == 0 || (!tcp && few_gemm_tiles(G, M, N, K))) &&
+                            prod(la) < (1LL << 31) && prod(lb) < (1LL << 31) &&
+                            prod(lc) < (1LL << 31) && group_entries(G, M, N, K) <= kGroupEntries;
         if (!direct && !onesided && prod(gm) >= 64 && prod(gn) >= 64 && prod(gk) >= 64) {
             int store_t = dtype == 0 ? E_F64 : E_F32;
             int gemm_t = dtype == 0 ? E_F64 : prec == TN_BF16 ? E_BF16 : E_F32;
