@@ -53,6 +53,13 @@ static tn_status fail(tn_status s, const std::string &msg) {
 
 namespace {
 
+// Scratch memory of the calls that keep no program (single contractions, the
+// samples of tn_sample) comes from a pool of the library's own on each device:
+// stream-ordered as before, safe from any thread and stream, but up to
+// kPoolKeep bytes stay with it between calls (the default pool hands every
+// byte back at each synchronisation: 100 to 250 us a call to map it again).
+// What it holds is given back before a program measures the free memory, and
+// whenever an allocation of the library fails.
 constexpr uint64_t kPoolKeep = 512ull << 20;
 std::mutex g_pool_mu;
 std::map<int, cudaMemPool_t> g_pools;
@@ -1211,8 +1218,11 @@ struct MicroList {
     }
     // false when the records exceed MICRO_BLOB bytes
     bool close(int esz) {
-        std::stable_sort(open.begin(), open.end(),
-                         [](const Item &x, const Item &y) { return x.level < y.level; });
+        // nodes by level (indices: the records stay where they are)
+        std::vector<int> order(open.size());
+        std::iota(order.begin(), order.end(), 0);
+        std::stable_sort(order.begin(), order.end(),
+                         [&](int x, int y) { return open[x].level < open[y].level; });
         std::vector<int32_t> lev;
         std::vector<uint32_t> at, tasks;   // head positions relative to the first head
         // offset tables of the outputs of an item and of the summed indices
@@ -1249,7 +1259,7 @@ struct MicroList {
             units += (uint32_t)(sizeof(MicroHead) / 16 + it.dims.size());
         }
         int last = -1;
-        for (size_t i = 0; i < open.size(); ++i) {
+        for (int i : order) {
             if (open[i].level != last) lev.push_back((int32_t)tasks.size());
             last = open[i].level;
             const int per = 32 >> open[i].h.klog, nt = (open[i].h.elems + per - 1) / per;
@@ -1271,7 +1281,8 @@ struct MicroList {
         // maxima: staged together, or all left in global memory
         std::vector<uint32_t> mslot;
         {
-            std::map<int64_t, int32_t> pos;
+            std::unordered_map<int64_t, int32_t> pos;
+            pos.reserve(2 * open.size());
             bool ok = true;
             auto want = [&](int64_t slot, int n, bool own) {
                 if (slot < 0 || !ok) return;
@@ -1299,39 +1310,46 @@ struct MicroList {
         std::vector<uint32_t> src;
         size_t vals = 0;
         {
-            struct Tn { int64_t n; bool own; int32_t pos; };
-            std::map<int64_t, Tn> ten;   // by arena offset
-            for (auto &it : open) ten[it.h.offC] = {it.h.elems, true, -1};
+            struct Tn { int64_t off, n; bool own; int32_t pos; };
+            std::vector<Tn> tens;
+            std::unordered_map<int64_t, int> ten;   // arena offset -> tensor
+            ten.reserve(3 * open.size());
+            auto want = [&](int64_t off, int64_t n, bool own) {
+                if (ten.emplace(off, (int)tens.size()).second) tens.push_back({off, n, own, -1});
+            };
+            for (auto &it : open) want(it.h.offC, it.h.elems, true);
             for (auto &it : open) {
-                ten.insert({it.h.offA, {it.nA, false, -1}});
-                ten.insert({it.h.offB, {it.nB, false, -1}});
+                want(it.h.offA, it.nA, false);
+                want(it.h.offB, it.nB, false);
             }
-            std::vector<std::pair<int64_t, int64_t>> order;   // entries, offset
-            for (auto &t : ten) order.push_back({t.second.n, t.first});
-            std::sort(order.begin(), order.end());
+            std::vector<int> by(tens.size());
+            std::iota(by.begin(), by.end(), 0);
+            std::sort(by.begin(), by.end(), [&](int x, int y) {
+                return tens[x].n != tens[y].n ? tens[x].n < tens[y].n : tens[x].off < tens[y].off;
+            });
             const size_t room =
                 ((size_t)MICRO_SMEM - bytes - ((mslot.size() + 1) & ~(size_t)1) * 8) / esz;
-            for (auto &o : order) {
-                Tn &t = ten[o.second];
+            for (int i : by) {
+                Tn &t = tens[i];
                 if (vals + (size_t)t.n > room) break;
-                if (!t.own && o.second + t.n > 0xffffffffLL) continue;
+                if (!t.own && t.off + t.n > 0xffffffffLL) continue;
                 vals += (size_t)t.n;
                 t.pos = 0;   // taken
             }
             int32_t next = 0;
             for (bool own : {false, true})   // inputs first: one gather fills them
-                for (auto &kv : ten) {
-                    Tn &t = kv.second;
+                for (Tn &t : tens) {
                     if (t.pos < 0 || t.own != own) continue;
                     t.pos = next;
                     next += (int32_t)t.n;
                     if (!own)
-                        for (int64_t j = 0; j < t.n; ++j) src.push_back((uint32_t)(kv.first + j));
+                        for (int64_t j = 0; j < t.n; ++j) src.push_back((uint32_t)(t.off + j));
                 }
+            auto place = [&](int64_t off) { return tens[ten[off]].pos; };
             for (auto &it : open) {
-                it.h.sA = ten[it.h.offA].pos;
-                it.h.sB = ten[it.h.offB].pos;
-                it.h.sC = ten[it.h.offC].pos;
+                it.h.sA = place(it.h.offA);
+                it.h.sB = place(it.h.offB);
+                it.h.sC = place(it.h.offC);
             }
         }
         const size_t off = blob.size();
@@ -4108,13 +4126,6 @@ tn_status tn_mmap(tn_model *m, const int32_t *evid, int nq, const int32_t *query
     return solve(*m->mmap);
 }
 
-// Scratch memory of the calls that keep no program (single contractions, the
-// samples of tn_sample) comes from a pool of the library's own on each device:
-// stream-ordered as before, safe from any thread and stream, but up to
-// kPoolKeep bytes stay with it between calls (the default pool hands every
-// byte back at each synchronisation: 100 to 250 us a call to map it again).
-// What it holds is given back before a program measures the free memory, and
-// whenever an allocation of the library fails.
 // One wait-timeout flag per device for the single-contraction entry points,
 // created on first use.
 static tn_status device_err_flag(int **out) {
