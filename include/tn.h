@@ -359,14 +359,15 @@ const char *tn_last_error(void);
  * dtype: 0 = double, 1 = float.  A sum-product contraction whose row, column
  * and summed label groups each hold at least 64 entries (and with no label
  * summed inside one operand alone) runs as a batched GEMM: TN_TF32 / TN_BF16
- * on tcgen05 tensor cores (float data only), TN_FP32 / TN_FP64 on a CUDA-core
- * tiled GEMM; other sum-product contractions with no label summed inside one
- * operand run on a batched strided GEMM over the label groups (CUDA cores,
- * operands read in place through per-group offset tables); everything else
- * runs on the strided contraction kernels.  No
- * rescaling is applied.  The call allocates its scratch memory (operand
- * workspaces, split-K partial sums) stream-ordered from the CUDA memory pool
- * and synchronises `cuda_stream` before returning.
+ * on tcgen05 tensor cores (float data only), TN_FP32 on a CUDA-core tiled GEMM
+ * where its output tiles fill the device; other sum-product contractions with
+ * no label summed inside one operand (and double data below 2^31 entries) run on a
+ * batched strided GEMM over the label groups (CUDA cores, operands read in
+ * place through per-group offset tables); everything else runs on the strided
+ * contraction kernels.  No rescaling is applied.  The call takes its scratch
+ * memory (operand workspaces, tables, split-K partial sums) stream-ordered
+ * from a memory pool of the library, which keeps at most 512 MiB between
+ * calls, and synchronises `cuda_stream` before returning.
  */
 tn_status tn_contract_dev(int nlabels, const int *sizes,
                           int na, const int *labels_a, const void *A,

@@ -526,7 +526,8 @@ static void launch_tiled(const PDesc *const *ps, int n, cudaStream_t st) {
 
 int launch_permutes(const PDesc *x, const PDesc *y, cudaStream_t st) {
     auto tiled = [](const PDesc *p) { return p && p->total > 0 && p->tl.tn > 0 && p->tl.ttab; };
-    // up to 2^25 entries each, where a launch's ramp and tail weigh (beyond, the
+    // up to 2^25 entries each, where a launch's ramp and tail weigh: three
+    // 1000 x 777 x 1155 products in TF32 133.5 -> 130.6 us a call, 4096^3 BF16 284 -> 276 (beyond, the
     // larger shared-memory tile of the two sets the blocks of both: 1.7 GB and
     // 5.5 GB operands took 2.36 ms together, 1.70 one after the other)
     if (tiled(x) && tiled(y) && x->in_type == y->in_type && x->out_type == y->out_type &&
