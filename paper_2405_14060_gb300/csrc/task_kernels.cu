@@ -356,10 +356,11 @@ __global__ void __launch_bounds__(256) k_backtrack(const BackHead h, const uint4
     if (SM) {
         for (int i = threadIdx.x; i < h.bytes / 16; i += 256) ((uint4 *)bsm)[i] = __ldg(blob + i);
         x = (int32_t *)(bsm + h.bytes);
-        for (int v = threadIdx.x; v < nvars; v += 256) x[v] = row[v];
         rec = bsm;
-        __syncthreads();
     }
+    // a variable of one value is maximised by no record: free, it takes that value
+    for (int v = threadIdx.x; v < nvars; v += 256) x[v] = max(row[v], 0);
+    __syncthreads();
     const BackNode *nodes = (const BackNode *)rec;
     const BackLab *labs = (const BackLab *)(rec + h.labs);
     const int2 *digs = (const int2 *)(rec + h.digs);

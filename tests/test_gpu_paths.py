@@ -186,3 +186,58 @@ def test_tc_gemm_edges(m, n, k, prec, spec):
     # two roundings of each product's inputs (2^-11 TF32 truncated to 2^-10, 2^-9 BF16)
     err = ((C.double() - ref).abs() / ref).max().item()
     assert err <= (2 * 2.0 ** -10 if prec == "tf32" else 2 * 2.0 ** -8)
+
+
+# domains of one value in the backtrack (no record maximises them): inside larger
+# factors, alone, eliminated before and after their neighbours, observed and
+# queried; the last model's records do not fit shared memory
+def _size1_model(card, scopes, seed):
+    rng = np.random.default_rng(seed)
+    card = np.array(card, np.int32)
+    return synth.Model(card, [np.array(s, np.int32) for s in scopes],
+                       [rng.random(int(np.prod(card[s]))) + 0.1 for s in scopes])
+
+
+SIZE1 = [([1, 2], [[0, 1], [1]]),
+         ([1, 2, 1, 3], [[0, 1], [1, 2, 3], [3, 0], [2]]),
+         ([2, 1, 1, 4, 1], [[1, 0, 2, 3], [3, 1], [0, 2], [2, 1], [4]]),
+         ([1, 1], [[0, 1]])]
+
+
+@pytest.mark.parametrize("card,scopes", SIZE1)
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_backtrack_size1_domains(card, scopes, prec):
+    m = _size1_model(card, scopes, len(card))
+    M = tn.Model.from_synth(m)
+    tol = 1e-9 if prec == "fp64" else 1e-4
+    ev = np.full(m.nvars, -1, np.int32)
+    for observed in ([], [card.index(1)]):
+        ev[observed] = 0
+        xb, lb = oracle.brute_map(m, ev)
+        for method in range(4):
+            M.set_order(*M.optimize_order(method, 2, 1))
+            x, lp = M.map(ev, prec=prec)
+            np.testing.assert_array_equal(x, xb)
+            assert abs(lp - lb) < tol
+    if m.nvars < 3:
+        return
+    for query in ([0, 3], [1, 2], [0, 1, 2], [3, 2]):
+        xb, lb = oracle.brute_mmap(m, query)
+        x, lp = M.mmap(query, prec=prec)
+        np.testing.assert_array_equal(x, xb)
+        assert abs(lp - lb) < tol
+
+
+def test_backtrack_size1_domains_large():
+    m = synth.chain_model(5000, [2, 1, 3, 2] * 1250, 7)
+    x, lp = tn.Model.from_synth(m).map()
+    best, back = np.log(m.tables[0]), []     # Viterbi along the chain
+    for one, s, t in zip(m.tables[1:], m.scopes[m.nvars:], m.tables[m.nvars:]):
+        w = best[:, None] + np.log(t.reshape(m.card[s])) + np.log(one)
+        back.append(w.argmax(0))
+        best = w.max(0)
+    xo = [int(best.argmax())]
+    for b in reversed(back):
+        xo.append(int(b[xo[-1]]))
+    np.testing.assert_array_equal(x, xo[::-1])
+    assert abs(lp - best.max()) < 1e-9 * abs(best.max())
