@@ -50,7 +50,7 @@ __global__ void k_leaves(const LeafRec *recs, const double *tables, const int *c
                     }
                     for (int j = 0; j < r.nsd; ++j) off += (int64_t)slice_val[r.sidx[j]] * r.sst[j];
                 }
-                x = tables[off];
+                x = tables[off] + 0.0;   // -0.0 (a valid entry) to 0.0: tensors order like their bits
                 bool in_log = flags && flags[0];
                 if (log_mode && !in_log) x = log(x);
                 else if (!log_mode && in_log) x = exp(x);
@@ -467,9 +467,9 @@ template <typename T, int N>
 __device__ __forceinline__ int64_t samp_small(const T *A, const T *B,
                                               const longlong2 *__restrict__ kt, int K, double u) {
     // running sums: the last is the total, and the draw compares with each.
-    // Sums of non-negative values order like their bits, and integer comparisons
-    // leave the FP64 pipe (two operations a clock and SM, what bounds the kernel)
-    // to the products and sums
+    // Sums of values without a sign order like their bits (the leaves turn -0.0
+    // into 0.0), and integer comparisons leave the FP64 pipe (two operations a
+    // clock and SM, what bounds the kernel) to the products and sums
     double c[N];
     unsigned long long w[N];
 #pragma unroll

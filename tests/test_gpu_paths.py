@@ -241,3 +241,18 @@ def test_backtrack_size1_domains_large():
         xo.append(int(b[xo[-1]]))
     np.testing.assert_array_equal(x, xo[::-1])
     assert abs(lp - best.max()) < 1e-9 * abs(best.max())
+
+
+# tables with negative zeros are those with zeros: draws of up to 2, up to 8 and
+# more entries
+@pytest.mark.parametrize("card", [2, 3, 8, 9, 120])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_negative_zero_sampling(card, prec):
+    t = np.linspace(1.0, 2.0, card)
+    t[0] = t[card // 2 + 1:] = -0.0
+    M = tn.Model.from_arrays([card], [[0]], [t])
+    s = M.sample(20000, seed=5, prec=prec)[:, 0].astype(np.int64)
+    pos = tn.Model.from_arrays([card], [[0]], [np.abs(t)])
+    np.testing.assert_array_equal(s, pos.sample(20000, seed=5, prec=prec)[:, 0])
+    emp = np.bincount(s, minlength=card) / 20000
+    assert np.all(np.abs(emp - np.abs(t) / t.sum()) < 5 * np.sqrt(0.25 / 20000))
