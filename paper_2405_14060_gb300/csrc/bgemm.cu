@@ -28,7 +28,6 @@
 // kernel records the maximum of C.
 #include <algorithm>
 #include <cmath>
-#include <mutex>
 #include <utility>
 
 #include "bgemm.cuh"
@@ -558,22 +557,18 @@ void go(const BDesc &d, float *part, int64_t ntiles, cudaStream_t st) {
     constexpr size_t smem =
         (size_t)kStages * (Gather<BM>::SIZE + Gather<BN>::SIZE) * sizeof(float);
     auto kern = k_bgemm<BM, BN, kTM[TILE], kTN[TILE], NFAST, RQ>;
-    static std::once_flag once;
-    static int per_sm = 1, nsm = 152;
-    std::call_once(once, [&] {
+    static PerDevice once;
+    static std::atomic<int> per_sm{1};   // the same on every sm_103a device
+    const int dev = current_device();
+    once.once(dev, [&] {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         int b = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, kThreads, smem) ==
                 cudaSuccess &&
             b > 0)
             per_sm = b;
-        int dev = 0, n = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-            n > 0)
-            nsm = n;
     });
-    const int64_t grid = std::min<int64_t>(ntiles, (int64_t)nsm * per_sm);
+    const int64_t grid = std::min<int64_t>(ntiles, (int64_t)sm_count(dev) * per_sm);
     kern<<<(unsigned)grid, kThreads, smem, st>>>(d, part, (int)ntiles);
 }
 

@@ -21,7 +21,6 @@
 #pragma once
 #include <algorithm>
 #include <cstdint>
-#include <mutex>
 
 #include "devutil.cuh"
 #include "stream.cuh"

@@ -4,7 +4,25 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "per_device.h"
+
 namespace tn {
+
+inline int current_device() {
+    int dev = 0;
+    return cudaGetDevice(&dev) == cudaSuccess ? dev : 0;
+}
+// SMs of a device, read from it once.
+inline int sm_count(int dev) {
+    static std::atomic<int> sms[64];
+    const bool kept = dev >= 0 && dev < 64;
+    int n = kept ? sms[dev].load(std::memory_order_relaxed) : 0;
+    if (n > 0) return n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
+        return 152;
+    if (kept) sms[dev].store(n, std::memory_order_relaxed);
+    return n;
+}
 
 __device__ __forceinline__ int exp_of_bits(unsigned long long b) {
     if (b == 0ull) return 0;

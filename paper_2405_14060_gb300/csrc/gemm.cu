@@ -507,8 +507,8 @@ static void launch_tiled(const PDesc *const *ps, int n, cudaStream_t st) {
         gx = std::max(gx, a.blocks[i]);
         gy = std::max(gy, a.items[i]);
     }
-    static std::once_flag once;
-    std::call_once(once, [] {
+    static PerDevice once;
+    once.once(current_device(), [] {
         const int mx = 3 * pt_nbuf(PT_MAXN, 0) * 8;
         cudaFuncSetAttribute(k_permute_tiled<double, E_F64>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
@@ -898,8 +898,9 @@ static bool make_map(CUtensorMap *m, const void *base, int64_t K, int64_t rows, 
 }
 
 cudaError_t launch_tc_gemm(const GDesc &g, int *err_flag, cudaStream_t st) {
-    static std::once_flag once;
-    std::call_once(once, [] {
+    static PerDevice once;
+    const int dev = current_device();
+    once.once(dev, [] {
         cudaFuncSetAttribute(k_tc_gemm<0, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem(1));
         cudaFuncSetAttribute(k_tc_gemm<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem(1));
         cudaFuncSetAttribute(k_tc_gemm<0, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem(2));
@@ -938,14 +939,7 @@ cudaError_t launch_tc_gemm(const GDesc &g, int *err_flag, cudaStream_t st) {
     // the tile, and CTAs started in tile order keep the concurrently read
     // operand panels close together in L2, where persistent CTAs drift apart
     // over hundreds of K slabs; measured on the batched workload's nodes)
-    static int nsm = 0;
-    if (nsm == 0) {
-        int dev = 0, n = 0;
-        nsm = (cudaGetDevice(&dev) == cudaSuccess &&
-               cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0)
-                  ? n
-                  : 152;
-    }
+    const int nsm = sm_count(dev);
     // long K: 256 x 256 tiles, whose accumulators fill TMEM, when that costs no
     // extra round of tiles.  128 x 256 tiles need 43 (TF32) or 85 (BF16)
     // multiply-adds a byte from L2, 23 to 26 TB/s at the tensor peak; these need

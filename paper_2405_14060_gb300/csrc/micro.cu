@@ -18,7 +18,6 @@
 // when the whole tree of 599 nodes is one subtree.
 #include <algorithm>
 #include <cmath>
-#include <mutex>
 
 #include "devutil.cuh"
 #include "kernels.cuh"
@@ -270,8 +269,8 @@ template <typename T>
 void launch_micro(const unsigned char *blob, const MicroSub *subs, int nsub, int smem, int semiring,
                   int threads, T *arena, unsigned long long *mx, int32_t *am, cudaStream_t st) {
     if (nsub <= 0) return;
-    static std::once_flag once;
-    std::call_once(once, [] {
+    static PerDevice once;
+    once.once(current_device(), [] {
         cudaFuncSetAttribute(k_micro<T, SUM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              MICRO_SMEM);
         cudaFuncSetAttribute(k_micro<T, MAXPLUS>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -14,7 +14,6 @@
 #pragma once
 #include <algorithm>
 #include <cstdint>
-#include <mutex>
 #include <vector>
 
 #include "dense_impl.cuh"
@@ -463,8 +462,8 @@ static void reduce_dense_go(const RDesc &d, void *scratch, cudaStream_t st) {
     reduce_dense_shape(d, chunk, nchunks);
     const int modes = reduce_dense_modes(d);
     const size_t smem = reduce_dense_smem<T>(((modes & 3) == 3) + (((modes >> 2) & 3) == 3));
-    static std::once_flag once;
-    std::call_once(once, [] {
+    static PerDevice once;
+    once.once(current_device(), [] {
         cudaFuncSetAttribute(k_reduce_dense<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)reduce_dense_smem<T>(2));
     });
@@ -507,8 +506,8 @@ static void reduce_go(const RDesc &d, const RedPiece &p, void *scratch, cudaStre
         }
     }
     constexpr size_t smem = (size_t)red_stages<T>() * (NS + NT) * 256 * sizeof(T);
-    static std::once_flag once;
-    std::call_once(once, [] {
+    static PerDevice once;
+    once.once(current_device(), [] {
         cudaFuncSetAttribute(k_reduce_part<T, NS, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
     });

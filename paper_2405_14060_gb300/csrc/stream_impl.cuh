@@ -17,7 +17,6 @@
 
 #pragma once
 #include <algorithm>
-#include <mutex>
 #include <vector>
 
 #include "dense_impl.cuh"
@@ -501,8 +500,8 @@ static DenseModes absorb_dense_modes(const ADesc &d) {
 template <typename T, int XM>
 static void absorb_dense_go(const ADesc &d, int ym, cudaStream_t st) {
     constexpr size_t smem = absorb_dense_smem<T, XM>();
-    static std::once_flag once;
-    std::call_once(once, [] {
+    static PerDevice once;
+    once.once(current_device(), [] {
         cudaFuncSetAttribute(k_absorb_dense<T, XM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
     });

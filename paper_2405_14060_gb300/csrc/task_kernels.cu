@@ -5,7 +5,6 @@
 #include <algorithm>
 #include <cfloat>
 #include <cmath>
-#include <mutex>
 
 #include "devutil.cuh"
 #include "task_kernels.cuh"
@@ -395,8 +394,8 @@ void launch_backtrack(const BackHead &h, const uint4 *blob, const int32_t *argma
         k_backtrack<false><<<nbeta, 256, 0, st>>>(h, blob, argmax, nvars, assign);
         return;
     }
-    static std::once_flag once;
-    std::call_once(once, [] {
+    static PerDevice once;
+    once.once(current_device(), [] {
         cudaFuncSetAttribute(k_backtrack<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kCap);
     });
@@ -666,8 +665,8 @@ void launch_sample(const SampNode *nodes, int nnodes, const SampLab *labs, const
             nodes, nnodes, labs, digs, ktab, base, cdf, evid, nvars, nsamp, seed, out);
         return;
     }
-    static std::once_flag once;
-    std::call_once(once, [] {
+    static PerDevice once;
+    once.once(current_device(), [] {
         cudaFuncSetAttribute(k_sample<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kCap);
     });

@@ -26,7 +26,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
-#include <mutex>
 
 #include "bgemm.cuh"
 #include "devutil.cuh"
@@ -313,18 +312,13 @@ template <int BN>
 void go_tc(const GParams &gp, cudaStream_t st) {
     constexpr int S = stages<BN>();
     constexpr size_t smem = (size_t)S * (kAB + BN * 128) + 1024 + 256;
-    static std::once_flag once;
-    static int nsm = 152;
-    std::call_once(once, [] {
+    static PerDevice once;
+    const int dev = current_device();
+    once.once(dev, [] {
         cudaFuncSetAttribute(k_tc_gather<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
-        int dev = 0, n = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-            n > 0)
-            nsm = n;
     });
-    const int grid = std::min(gp.ntiles, nsm);
+    const int grid = std::min(gp.ntiles, sm_count(dev));
     k_tc_gather<BN><<<grid, kThr, smem, st>>>(gp);
 }
 
