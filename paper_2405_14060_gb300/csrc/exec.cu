@@ -57,10 +57,12 @@ namespace {
 // samples of tn_sample) comes from a pool of the library's own on each device:
 // stream-ordered as before, safe from any thread and stream, but up to
 // kPoolKeep bytes stay with it between calls (the default pool hands every
-// byte back at each synchronisation: 100 to 250 us a call to map it again).
-// What it holds is given back before a program measures the free memory, and
-// whenever an allocation of the library fails.
-constexpr uint64_t kPoolKeep = 512ull << 20;
+// byte back at each synchronisation: 100 to 250 us a call to map it again, and
+// more for larger scratch: 4 x 4096^3 in TF32, 512 MiB, 923 us a call against
+// 1129).  A call with more scratch than that gives all of it back.  What the pool
+// holds is given back before a program measures the free memory, and whenever
+// an allocation of a program fails.
+constexpr uint64_t kPoolKeep = 1ull << 30;
 std::mutex g_pool_mu;
 std::map<int, cudaMemPool_t> g_pools;
 
@@ -98,14 +100,18 @@ void trim_scratch_pool() {
     if (it != g_pools.end() && it->second) cudaMemPoolTrimTo(it->second, 0);
 }
 
-// Stream-ordered scratch of one call; freed on its stream with the object.
+// Stream-ordered scratch of one call, freed on its stream: by free() before the
+// call's wait, so that the wait sees the memory unused and the pool's bound
+// holds when the call returns, else with the object.
 struct CallMem {
     cudaStream_t st;
     void *p = nullptr;
     explicit CallMem(cudaStream_t s) : st(s) {}
     CallMem(const CallMem &) = delete;
-    ~CallMem() {
+    ~CallMem() { free(); }
+    void free() {
         if (p) cudaFreeAsync(p, st);
+        p = nullptr;
     }
     cudaError_t alloc(size_t bytes) {
         cudaMemPool_t pool;
@@ -3831,6 +3837,7 @@ tn_status tn_sample(tn_model *m, const int32_t *evid, uint64_t seed, int64_t n,
         if (s) return s;
         CK(cudaEventRecord(m->ev1, st));
         CK(cudaMemcpyAsync(samples, d_out, (size_t)n * nv, cudaMemcpyDeviceToHost, st));
+        out.free();
         CK(cudaStreamSynchronize(st));
         float ms = 0;
         CK(cudaEventElapsedTime(&ms, m->ev0, m->ev1));
@@ -3917,6 +3924,7 @@ tn_status tn_sample(tn_model *m, const int32_t *evid, uint64_t seed, int64_t n,
     }
     std::vector<int8_t> h((size_t)n * nv);
     CK(cudaMemcpyAsync(h.data(), d_out, h.size(), cudaMemcpyDeviceToHost, st));
+    out.free();
     CK(cudaStreamSynchronize(st));
     // rows grouped by assignment -> a uniformly random order (Fisher-Yates)
     std::vector<int64_t> perm(n);
@@ -4149,10 +4157,12 @@ static bool few_gemm_tiles(int64_t batch, int64_t rows, int64_t cols, int64_t k)
     return k >= 256 && (double)((rows + 63) / 64) * (double)((cols + 63) / 64) * (double)batch < 76;
 }
 
-// End of a single contraction: wait for its stream; `err` (tensor-core
-// kernels): the flag of a wait that gave up, read behind the kernels.
-static tn_status finish_call(cudaStream_t st, int *err) {
+// End of a single contraction: free its scratch and wait for its stream; `err`
+// (tensor-core kernels): the flag of a wait that gave up, read behind the kernels.
+static tn_status finish_call(CallMem &ws, int *err) {
+    const cudaStream_t st = ws.st;
     int herr = 0;
+    ws.free();
     if (err) CK(cudaMemcpyAsync(&herr, err, 4, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     if (herr) {
@@ -4276,7 +4286,7 @@ tn_status tn_contract_dev(int nlabels, const int *sizes, int na, const int *labe
             if (le != cudaSuccess || e2 != cudaSuccess)
                 return fail(TN_E_CUDA, std::string("GEMM launch: ") +
                                            cudaGetErrorString(le != cudaSuccess ? le : e2));
-            return finish_call(st, tc ? d_err : nullptr);
+            return finish_call(ws, tc ? d_err : nullptr);
         }
     }
     int es = dtype == 0 ? 8 : 4;
@@ -4311,7 +4321,7 @@ tn_status tn_contract_dev(int nlabels, const int *sizes, int na, const int *labe
                 return fail(TN_E_CUDA,
                             std::string("batched GEMM launch: ") + cudaGetErrorString(e));
             }
-            return finish_call(st, bd.tc ? bd.err : nullptr);
+            return finish_call(ws, bd.tc ? bd.err : nullptr);
         }
     }
     CDesc d;
@@ -4326,8 +4336,7 @@ tn_status tn_contract_dev(int nlabels, const int *sizes, int na, const int *labe
     else launch_contract<float>(d, semiring, ws.p, sb, st, nullptr);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(TN_E_CUDA, std::string("contract launch: ") + cudaGetErrorString(e));
-    CK(cudaStreamSynchronize(st));
-    return TN_OK;
+    return finish_call(ws, nullptr);
 }
 
 // Time every kernel of a PR (task 0) or PR + MAR (task 1) pass one launch at a

@@ -256,3 +256,14 @@ def test_negative_zero_sampling(card, prec):
     np.testing.assert_array_equal(s, pos.sample(20000, seed=5, prec=prec)[:, 0])
     emp = np.bincount(s, minlength=card) / 20000
     assert np.all(np.abs(emp - np.abs(t) / t.sum()) < 5 * np.sqrt(0.25 / 20000))
+
+
+# scratch kept between single contractions stays within the stated bound (1.3 GiB
+# of operand workspaces here)
+def test_scratch_kept_is_bounded():
+    for n in (128, 13312):       # (the first loads the kernels)
+        A, B, C = (torch.zeros(n, n, device="cuda") for _ in range(3))
+        torch.cuda.empty_cache()
+        free = torch.cuda.mem_get_info()[0]
+        tn.contract_dev([n, n, n], [2, 0], A, [2, 1], B, [0, 1], C, prec="tf32")
+    assert free - torch.cuda.mem_get_info()[0] <= 1 << 30
