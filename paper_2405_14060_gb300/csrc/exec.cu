@@ -60,8 +60,9 @@ namespace {
 // byte back at each synchronisation: 100 to 250 us a call to map it again, and
 // more for larger scratch: 4 x 4096^3 in TF32, 512 MiB, 923 us a call against
 // 1129).  A call with more scratch than that gives all of it back.  What the pool
-// holds is given back before a program measures the free memory, and whenever
-// an allocation of a program fails.
+// holds unused is given back before a program measures the free memory and when
+// one of its allocations fails, and the driver takes it back for any other
+// allocation of the process that would fail.
 constexpr uint64_t kPoolKeep = 1ull << 30;
 std::mutex g_pool_mu;
 std::map<int, cudaMemPool_t> g_pools;
