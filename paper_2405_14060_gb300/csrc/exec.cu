@@ -19,7 +19,6 @@
 #include <set>
 #include <string>
 #include <tuple>
-#include <unordered_map>
 #include <vector>
 
 #include "bgemm.cuh"
@@ -422,23 +421,23 @@ std::string make_desc(const std::vector<int> &card, const Labels &la, bool ba, i
                       const Labels *korder, int nbeta, int32_t *argmax, CDesc &d) {
     std::memset(&d, 0, sizeof(d));
     if ((ba || bb) && !bc) return "batch label cannot be summed";
-    std::set<int> sc(lc.begin(), lc.end()), sa(la.begin(), la.end()), sb(lb.begin(), lb.end());
+    // (labels are few: a scan costs less than a set)
+    auto in = [](const Labels &l, int v) { return std::find(l.begin(), l.end(), v) != l.end(); };
     Labels ks;
     if (korder) ks = *korder;
     else {
         for (int v : la)
-            if (!sc.count(v)) ks.push_back(v);
+            if (!in(lc, v)) ks.push_back(v);
         for (int v : lb)
-            if (!sc.count(v) && !sa.count(v)) ks.push_back(v);
+            if (!in(lc, v) && !in(la, v)) ks.push_back(v);
     }
     struct Dim { int64_t sz, sa, sb; };
     auto build = [&](const Labels &L, std::vector<Dim> &out) {
         std::vector<Dim> raw;
         for (int v : L) {
             if (card[v] == 1) continue;
-            int64_t a = sa.count(v) ? stride_in(card, la, v) : 0;
-            int64_t b = sb.count(v) ? stride_in(card, lb, v) : 0;
-            raw.push_back({card[v], a, b});
+            const int64_t a = stride_in(card, la, v), b = stride_in(card, lb, v);
+            raw.push_back({card[v], std::max<int64_t>(a, 0), std::max<int64_t>(b, 0)});
         }
         out.clear();
         for (auto &x : raw) {
@@ -1171,26 +1170,34 @@ static bool make_bgemm(const std::vector<int> &card, const Labels &lx, bool bx, 
 }
 
 // Records of one pass over the micro subtrees (micro.cuh), built subtree by
-// subtree: nodes are added with their level, then the subtree is closed.
+// subtree: nodes are added with their level and the numbers of their tensors
+// (what is staged is looked up by number), then the subtree is closed.
 struct MicroList {
     std::vector<unsigned char> blob;
     std::vector<MicroSub> subs;
     int smem = 0;      // largest subtree (bytes)
     int width = 1;     // largest level (tasks)
     struct Item {
-        int level;
+        int level, dim0;          // dims[dim0 ..): output, then summed dimensions
+        int tA, tB, tC;           // tensor numbers
+        int64_t nA, nB;           // entries of the operands
         MicroHead h;
-        std::vector<int4> dims;
-        int64_t nA, nB;   // entries of the operands
     };
     std::vector<Item> open;
+    std::vector<int4> dims;
+    explicit MicroList(int ntensors) : mpos(ntensors, -1), tpos(ntensors, -1) {}
 
-    bool add(const CDesc &d, int level, int64_t na, int64_t nb, const char *arena, int esz,
-             const unsigned long long *mxb, const int32_t *amb) {
+    bool add(const CDesc &d, int level, int tA, int64_t na, int tB, int64_t nb, int tC,
+             const char *arena, int esz, const unsigned long long *mxb, const int32_t *amb) {
         if (d.nbeta > MICRO_BETA || d.nout_total * d.nbeta > MICRO_MAX || d.ktotal > (1LL << 30))
             return false;
-        Item it;
+        open.emplace_back();
+        Item &it = open.back();
         it.level = level;
+        it.dim0 = (int)dims.size();
+        it.tA = tA;
+        it.tB = tB;
+        it.tC = tC;
         it.nA = na;
         it.nB = nb;
         MicroHead &m = it.h;
@@ -1210,9 +1217,9 @@ struct MicroList {
         m.bsa = (int16_t)d.bsa;   // at most MICRO_MAX, as every tensor
         m.bsb = (int16_t)d.bsb;
         for (int i = 0; i < d.nout; ++i)
-            it.dims.push_back(int4{d.osz[i], d.osh[i], (int)d.osa[i], (int)d.osb[i]});
+            dims.push_back(int4{d.osz[i], d.osh[i], (int)d.osa[i], (int)d.osb[i]});
         for (int i = 0; i < d.nk; ++i)
-            it.dims.push_back(int4{d.ksz[i], d.ksh[i], (int)d.ksa[i], (int)d.ksb[i]});
+            dims.push_back(int4{d.ksz[i], d.ksh[i], (int)d.ksa[i], (int)d.ksb[i]});
         m.mxa = d.mxa ? d.mxa - mxb : -1;
         m.mxb = d.mxb ? d.mxb - mxb : -1;
         m.mxc = d.mxc ? d.mxc - mxb : -1;
@@ -1220,51 +1227,33 @@ struct MicroList {
         m.mxb_bs = d.mxb_bs;
         m.amoff = d.argmax ? d.argmax - amb : -1;
         m.sA = m.sB = m.sC = m.smxa = m.smxb = m.smxc = -1;
-        open.push_back(std::move(it));
         return true;
     }
     // false when the records exceed MICRO_BLOB bytes
     bool close(int esz) {
         // nodes by level (indices: the records stay where they are)
-        std::vector<int> order(open.size());
+        order.resize(open.size());
         std::iota(order.begin(), order.end(), 0);
-        std::stable_sort(order.begin(), order.end(),
-                         [&](int x, int y) { return open[x].level < open[y].level; });
-        std::vector<int32_t> lev;
-        std::vector<uint32_t> at, tasks;   // head positions relative to the first head
+        std::sort(order.begin(), order.end(), [&](int x, int y) {
+            return open[x].level != open[y].level ? open[x].level < open[y].level : x < y;
+        });
         // offset tables of the outputs of an item and of the summed indices
         // (equal ones stored once); dimensions only where there is no table
-        std::vector<uint32_t> tabs;
-        std::unordered_map<std::string, int32_t> seen;   // by sizes and strides
-        auto table = [&](const int4 *dim, int nd, int total) {
-            auto r = seen.emplace(std::string((const char *)dim, (size_t)nd * sizeof(int4)),
-                                  (int32_t)(tabs.size() * 4));
-            if (!r.second) return r.first->second;
-            int dig[MAXD] = {0};
-            uint32_t a = 0, b = 0;
-            for (int i = 0; i < total; ++i) {
-                tabs.push_back(a | (b << 16));
-                for (int q = nd - 1; q >= 0; --q) {
-                    a += (uint32_t)dim[q].z;
-                    b += (uint32_t)dim[q].w;
-                    if (++dig[q] < dim[q].x) break;
-                    a -= (uint32_t)(dim[q].z * dim[q].x);
-                    b -= (uint32_t)(dim[q].w * dim[q].x);
-                    dig[q] = 0;
-                }
-            }
-            return r.first->second;
-        };
+        tabs.clear();
+        size_t cap = 64;
+        while (cap < 4 * open.size()) cap *= 2;   // two tables a node: at most half full
+        seen.assign(cap, Tab{0, -1, 0});
+        at.clear();   // head positions relative to the first head
         uint32_t units = 0;
         for (auto &it : open) {
             MicroHead &m = it.h;
-            m.otab = m.nout_total <= MICRO_OTAB ? table(it.dims.data(), m.nout, m.nout_total) : -1;
-            m.ktab = m.ktotal <= MICRO_KTAB
-                         ? table(it.dims.data() + m.nout, m.nk, m.ktotal) : -1;
-            if (m.otab >= 0 && m.ktab >= 0) it.dims.clear();
+            m.otab = m.nout_total <= MICRO_OTAB ? table(it.dim0, m.nout, m.nout_total) : -1;
+            m.ktab = m.ktotal <= MICRO_KTAB ? table(it.dim0 + m.nout, m.nk, m.ktotal) : -1;
             at.push_back(units);
-            units += (uint32_t)(sizeof(MicroHead) / 16 + it.dims.size());
+            units += (uint32_t)(sizeof(MicroHead) / 16 + ndims(it));
         }
+        lev.clear();
+        tasks.clear();
         int last = -1;
         for (int i : order) {
             if (open[i].level != last) lev.push_back((int32_t)tasks.size());
@@ -1286,62 +1275,74 @@ struct MicroList {
         if (bytes > (size_t)MICRO_BLOB) return false;
         for (auto &t : tasks) t += (uint32_t)(h0 / 16) << 16;
         // maxima: staged together, or all left in global memory
-        std::vector<uint32_t> mslot;
+        mslot.clear();
         {
-            std::unordered_map<int64_t, int32_t> pos;
-            pos.reserve(2 * open.size());
             bool ok = true;
-            auto want = [&](int64_t slot, int n, bool own) {
+            used.clear();
+            auto want = [&](int t, int64_t slot, int n, bool own) {
                 if (slot < 0 || !ok) return;
-                auto r = pos.emplace(slot, (int32_t)mslot.size());
                 if (slot + n > 0x7fffffffLL) ok = false;
-                else if (r.second)
+                else if (mpos[t] < 0) {
+                    mpos[t] = (int32_t)mslot.size();
+                    used.push_back(t);
                     for (int j = 0; j < n; ++j)
                         mslot.push_back((uint32_t)(slot + j) | (own ? 0x80000000u : 0u));
+                }
                 if ((int)mslot.size() > MICRO_MAXIMA) ok = false;
             };
-            for (auto &it : open) want(it.h.mxc, it.h.nbeta, true);
+            for (auto &it : open) want(it.tC, it.h.mxc, it.h.nbeta, true);
             for (auto &it : open) {
-                want(it.h.mxa, it.h.mxa_bs ? it.h.nbeta : 1, false);
-                want(it.h.mxb, it.h.mxb_bs ? it.h.nbeta : 1, false);
+                want(it.tA, it.h.mxa, it.h.mxa_bs ? it.h.nbeta : 1, false);
+                want(it.tB, it.h.mxb, it.h.mxb_bs ? it.h.nbeta : 1, false);
             }
             if (!ok) mslot.clear();
             else
                 for (auto &it : open) {
-                    if (it.h.mxa >= 0) it.h.smxa = pos[it.h.mxa];
-                    if (it.h.mxb >= 0) it.h.smxb = pos[it.h.mxb];
-                    if (it.h.mxc >= 0) it.h.smxc = pos[it.h.mxc];
+                    if (it.h.mxa >= 0) it.h.smxa = mpos[it.tA];
+                    if (it.h.mxb >= 0) it.h.smxb = mpos[it.tB];
+                    if (it.h.mxc >= 0) it.h.smxc = mpos[it.tC];
                 }
+            for (int t : used) mpos[t] = -1;
         }
         // values: the smallest tensors first, while they fit
-        std::vector<uint32_t> src;
+        src.clear();
         size_t vals = 0;
         {
-            struct Tn { int64_t off, n; bool own; int32_t pos; };
-            std::vector<Tn> tens;
-            std::unordered_map<int64_t, int> ten;   // arena offset -> tensor
-            ten.reserve(3 * open.size());
-            auto want = [&](int64_t off, int64_t n, bool own) {
-                if (ten.emplace(off, (int)tens.size()).second) tens.push_back({off, n, own, -1});
+            tens.clear();
+            auto want = [&](int t, int64_t off, int64_t n, bool own) {
+                if (tpos[t] >= 0) return;
+                tpos[t] = (int)tens.size();
+                tens.push_back({off, n, t, own, -1});
             };
-            for (auto &it : open) want(it.h.offC, it.h.elems, true);
+            for (auto &it : open) want(it.tC, it.h.offC, it.h.elems, true);
             for (auto &it : open) {
-                want(it.h.offA, it.nA, false);
-                want(it.h.offB, it.nB, false);
+                want(it.tA, it.h.offA, it.nA, false);
+                want(it.tB, it.h.offB, it.nB, false);
             }
-            std::vector<int> by(tens.size());
-            std::iota(by.begin(), by.end(), 0);
-            std::sort(by.begin(), by.end(), [&](int x, int y) {
-                return tens[x].n != tens[y].n ? tens[x].n < tens[y].n : tens[x].off < tens[y].off;
-            });
             const size_t room =
                 ((size_t)MICRO_SMEM - bytes - ((mslot.size() + 1) & ~(size_t)1) * 8) / esz;
-            for (int i : by) {
-                Tn &t = tens[i];
-                if (vals + (size_t)t.n > room) break;
-                if (!t.own && t.off + t.n > 0xffffffffLL) continue;
-                vals += (size_t)t.n;
-                t.pos = 0;   // taken
+            size_t all = 0;
+            for (Tn &t : tens) all += (size_t)t.n;
+            if (all <= room) {
+                for (Tn &t : tens)
+                    if (t.own || t.off + t.n <= 0xffffffffLL) {
+                        vals += (size_t)t.n;
+                        t.pos = 0;   // taken
+                    }
+            } else {
+                by.resize(tens.size());
+                std::iota(by.begin(), by.end(), 0);
+                std::sort(by.begin(), by.end(), [&](int x, int y) {
+                    return tens[x].n != tens[y].n ? tens[x].n < tens[y].n
+                                                  : tens[x].off < tens[y].off;
+                });
+                for (int i : by) {
+                    Tn &t = tens[i];
+                    if (vals + (size_t)t.n > room) break;
+                    if (!t.own && t.off + t.n > 0xffffffffLL) continue;
+                    vals += (size_t)t.n;
+                    t.pos = 0;
+                }
             }
             int32_t next = 0;
             for (bool own : {false, true})   // inputs first: one gather fills them
@@ -1352,12 +1353,12 @@ struct MicroList {
                     if (!own)
                         for (int64_t j = 0; j < t.n; ++j) src.push_back((uint32_t)(t.off + j));
                 }
-            auto place = [&](int64_t off) { return tens[ten[off]].pos; };
             for (auto &it : open) {
-                it.h.sA = place(it.h.offA);
-                it.h.sB = place(it.h.offB);
-                it.h.sC = place(it.h.offC);
+                it.h.sA = tens[tpos[it.tA]].pos;
+                it.h.sB = tens[tpos[it.tB]].pos;
+                it.h.sC = tens[tpos[it.tC]].pos;
             }
+            for (Tn &t : tens) tpos[t.t] = -1;
         }
         const size_t off = blob.size();
         blob.resize(off + r16(bytes + (src.size() + mslot.size()) * 4), 0);
@@ -1366,8 +1367,8 @@ struct MicroList {
         for (size_t i = 0; i < open.size(); ++i) {
             unsigned char *p = &blob[off + h0 + (size_t)at[i] * 16];
             std::memcpy(p, &open[i].h, sizeof(MicroHead));
-            if (!open[i].dims.empty())
-                std::memcpy(p + sizeof(MicroHead), open[i].dims.data(), open[i].dims.size() * 16);
+            if (const int nd = ndims(open[i]))
+                std::memcpy(p + sizeof(MicroHead), &dims[open[i].dim0], (size_t)nd * 16);
         }
         if (!tabs.empty()) std::memcpy(&blob[off + tab0], tabs.data(), tabs.size() * 4);
         if (!src.empty()) std::memcpy(&blob[off + bytes], src.data(), src.size() * 4);
@@ -1384,7 +1385,57 @@ struct MicroList {
         subs.push_back(sub);
         smem = std::max(smem, (int)(bytes + ((mslot.size() + 1) & ~(size_t)1) * 8 + vals * esz));
         open.clear();
+        dims.clear();
         return true;
+    }
+
+  private:
+    // Working storage of close(), kept between subtrees.
+    struct Tn { int64_t off, n; int t; bool own; int32_t pos; };
+    struct Tab { int dim0, nd; int32_t pos; };
+    std::vector<int> order, by, used;
+    std::vector<uint32_t> at, tasks, tabs, mslot, src;
+    std::vector<int32_t> lev, mpos, tpos;   // mpos, tpos: by tensor number, -1: none
+    std::vector<Tn> tens;
+    std::vector<Tab> seen;   // open addressing by a hash of sizes and strides; nd < 0: free
+
+    // Dimensions that follow a head: none where both offset tables stand for them.
+    static int ndims(const Item &it) {
+        return it.h.otab >= 0 && it.h.ktab >= 0 ? 0 : it.h.nout + it.h.nk;
+    }
+    // Position (bytes from the first table) of the {A, B} offsets of all `total`
+    // indices over dims[dim0 .. dim0 + nd).
+    int32_t table(int dim0, int nd, int total) {
+        const int4 *dim = dims.data() + dim0;
+        uint64_t h = 1469598103934665603ull ^ (uint64_t)nd;
+        for (int i = 0; i < nd; ++i)
+            for (int v : {dim[i].x, dim[i].z, dim[i].w}) h = (h ^ (uint32_t)v) * 1099511628211ull;
+        size_t q0 = (size_t)(h >> 20) & (seen.size() - 1);
+        for (; seen[q0].nd >= 0; q0 = (q0 + 1) & (seen.size() - 1)) {
+            const Tab &t = seen[q0];
+            bool same = t.nd == nd;
+            for (int i = 0; i < nd && same; ++i) {
+                const int4 &o = dims[t.dim0 + i];
+                same = o.x == dim[i].x && o.z == dim[i].z && o.w == dim[i].w;
+            }
+            if (same) return t.pos;
+        }
+        const int32_t pos = (int32_t)(tabs.size() * 4);
+        seen[q0] = Tab{dim0, nd, pos};
+        int dig[MAXD] = {0};
+        uint32_t a = 0, b = 0;
+        for (int i = 0; i < total; ++i) {
+            tabs.push_back(a | (b << 16));
+            for (int q = nd - 1; q >= 0; --q) {
+                a += (uint32_t)dim[q].z;
+                b += (uint32_t)dim[q].w;
+                if (++dig[q] < dim[q].x) break;
+                a -= (uint32_t)(dim[q].z * dim[q].x);
+                b -= (uint32_t)(dim[q].w * dim[q].x);
+                dig[q] = 0;
+            }
+        }
+        return pos;
     }
 };
 
@@ -2283,20 +2334,21 @@ tn_status build_program(tn_model *m, const Net &net, const Tree &tree, int kind,
     P.mlane_beg.assign(P.nlanes + 1, 0);
     for (auto &lo : morder) P.mlane_beg[lo.first + 1]++;
     for (int l = 0; l < P.nlanes; ++l) P.mlane_beg[l + 1] += P.mlane_beg[l];
-    MicroList mf, mb;
+    // tensor numbers: forward v, adjoint NN + v
+    MicroList mf(NN), mb(2 * NN);
     std::vector<int> mlev(NN, 0);   // height inside the subtree (forward level)
+    std::vector<int> depth(NN, 0);   // backward level: distance from the subtree's root
     for (auto &lo : morder) {
         auto &kv = *msub.find(lo.second);
         for (int id : kv.second) {
             const Node &nd = pl.node[id];
             mlev[id] = 1 + std::max(mlev[nd.a], mlev[nd.b]);
-            if (!mf.add(P.fdesc[id - n], mlev[id], P.fwd[nd.a].elems, P.fwd[nd.b].elems, P.arena,
-                        P.esz, P.mx, P.am))
+            if (!mf.add(P.fdesc[id - n], mlev[id], nd.a, P.fwd[nd.a].elems, nd.b,
+                        P.fwd[nd.b].elems, id, P.arena, P.esz, P.mx, P.am))
                 return fail(TN_E_UNSUPPORTED, "micro node conversion");
         }
         if (!mf.close(P.esz)) return fail(TN_E_UNSUPPORTED, "micro subtree records");
         if (!backward) continue;
-        std::vector<int> depth(NN, 0);   // backward level: distance from the subtree's root
         for (auto it = kv.second.rbegin(); it != kv.second.rend(); ++it) {
             int id = *it;
             const Node &nd = pl.node[id];
@@ -2309,8 +2361,9 @@ tn_status build_program(tn_model *m, const Net &net, const Tree &tree, int kind,
                                 P.mx + P.adj[id].mx, nb.labels, nb.beta, P.fwd[nd.b].per,
                                 fptr(nd.b), P.mx + P.fwd[nd.b].mx, alab(nd.a), P.adj_beta[nd.a],
                                 aptr(nd.a), P.mx + P.adj[nd.a].mx, nullptr, nbeta, nullptr, d);
-                if (!err.empty() || !mb.add(d, depth[id], P.adj[id].elems, P.fwd[nd.b].elems,
-                                            P.arena, P.esz, P.mx, P.am))
+                if (!err.empty() ||
+                    !mb.add(d, depth[id], NN + id, P.adj[id].elems, nd.b, P.fwd[nd.b].elems,
+                            NN + nd.a, P.arena, P.esz, P.mx, P.am))
                     return fail(TN_E_UNSUPPORTED, "micro adjoint conversion");
             }
             if (P.need_adj[nd.b]) {
@@ -2318,8 +2371,9 @@ tn_status build_program(tn_model *m, const Net &net, const Tree &tree, int kind,
                                 P.mx + P.fwd[nd.a].mx, alab(id), P.adj_beta[id], P.adj[id].per,
                                 cbar, P.mx + P.adj[id].mx, alab(nd.b), P.adj_beta[nd.b],
                                 aptr(nd.b), P.mx + P.adj[nd.b].mx, nullptr, nbeta, nullptr, d);
-                if (!err.empty() || !mb.add(d, depth[id], P.fwd[nd.a].elems, P.adj[id].elems,
-                                            P.arena, P.esz, P.mx, P.am))
+                if (!err.empty() ||
+                    !mb.add(d, depth[id], nd.a, P.fwd[nd.a].elems, NN + id, P.adj[id].elems,
+                            NN + nd.b, P.arena, P.esz, P.mx, P.am))
                     return fail(TN_E_UNSUPPORTED, "micro adjoint conversion");
             }
         }
