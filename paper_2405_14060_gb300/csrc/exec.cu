@@ -2935,7 +2935,9 @@ void enqueue_program(tn_model *m, Program &P, cudaStream_t st, Prof *pr = nullpt
     P.launches = nl;
 }
 
-tn_status capture_program(tn_model *m, Program &P) {
+// `own`: the program is launched by itself (else only as a child of another graph,
+// and has no executable of its own).
+tn_status capture_program(tn_model *m, Program &P, bool own = true) {
     cudaGraph_t g = nullptr;
     if (P.nlanes > 1) {
         while ((int)m->lanes.size() < P.nlanes - 1) {
@@ -2955,8 +2957,8 @@ tn_status capture_program(tn_model *m, Program &P) {
     else enqueue_program<float>(m, P, m->stream, nullptr, &m->lanes);
     cudaError_t e = cudaStreamEndCapture(m->stream, &g);
     if (e != cudaSuccess) return fail(TN_E_CUDA, std::string("graph capture: ") + cudaGetErrorString(e));
-    e = cudaGraphInstantiate(&P.gexec, g, 0);
     P.graph = g;
+    if (own) e = cudaGraphInstantiate(&P.gexec, g, 0);
     if (e != cudaSuccess) return fail(TN_E_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
     return TN_OK;
 }
@@ -4116,7 +4118,7 @@ tn_status tn_mmap(tn_model *m, const int32_t *evid, int nq, const int32_t *query
         auto P = std::make_unique<Program>();
         s = build_program(m, net, t, K_SUMNET, dtype, 1, false, opts, *P, &spec, nullptr, c->d_evid);
         if (s) return s;
-        s = capture_program(m, *P);
+        s = capture_program(m, *P, false);
         if (s) return s;
         c->launches += P->launches;
         const Node &root = P->plan.node[P->plan.root];
@@ -4168,7 +4170,7 @@ tn_status tn_mmap(tn_model *m, const int32_t *evid, int nq, const int32_t *query
     c->top = std::make_unique<Program>();
     s = build_program(m, net2, t2, K_MAP, dtype, 1, false, opts, *c->top, &spec2, nullptr, c->d_evid);
     if (s) return s;
-    s = capture_program(m, *c->top);
+    s = capture_program(m, *c->top, false);
     if (s) return s;
     c->launches += c->top->launches;
     c->key = key;
