@@ -4348,14 +4348,20 @@ tn_status tn_contract_dev(int nlabels, const int *sizes, int na, const int *labe
     }
     int es = dtype == 0 ? 8 : 4;
     // other sum-product contractions without a label summed inside one
-    // operand: the batched strided GEMM
+    // operand: the batched strided GEMM (it refuses tensors of 2^31 entries and
+    // more, which its 32-bit offsets don't reach)
     if (semiring == 0) {
+        auto entries = [&](const Labels &l) {
+            int64_t q = 1;
+            for (int v : l) q *= card[v];
+            return q;
+        };
         BDesc bd;
         GroupTabs gt;
         std::vector<int32_t> tab;
         const bool tc_in = prec == TN_TF32 || prec == TN_BF16;
-        if (make_bgemm(card, la, false, 0, A, nullptr, lb, false, 0, B, nullptr, lc, false, 0, C,
-                       nullptr, 1, es, bd, tab, tc_in, &gt)) {
+        if (make_bgemm(card, la, false, entries(la), A, nullptr, lb, false, entries(lb), B, nullptr,
+                       lc, false, entries(lc), C, nullptr, 1, es, bd, tab, tc_in, &gt)) {
             if (!tc_in) bd.tc = 0;   // TF32 inputs only when asked
             const size_t ntab = gt.total ? (size_t)gt.total : tab.size();
             const size_t tb = (ntab * 4 + 255) & ~(size_t)255;

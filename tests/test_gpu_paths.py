@@ -293,3 +293,25 @@ def test_scratch_kept_is_given_back_to_models():
         torch.cuda.empty_cache()
     want = np.log(m.tables[0].sum())
     assert abs(lz - want) <= 1e-4 * abs(want)
+
+
+# operands of more than 2^31 entries with groups too small for a GEMM: rows at both
+# ends, summed fastest and not
+@pytest.mark.parametrize("spec", ["mk,kn->mn", "km,kn->nm"])
+def test_skinny_beyond_32bit_offsets(spec):
+    size = dict(k=136, m=(1 << 24) + 3, n=3)
+    (a, b), c = spec.split("->")[0].split(","), spec.split("->")[1]
+    letters = "kmn"
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    A, B = (torch.rand([size[l] for l in s], generator=gen, device="cuda") for s in (a, b))
+    C = torch.full([size[l] for l in c], float("nan"), device="cuda")
+    tn.contract_dev([size[l] for l in letters], [letters.index(l) for l in a], A,
+                    [letters.index(l) for l in b], B, [letters.index(l) for l in c], C, prec="fp32")
+    assert A.numel() > 1 << 31
+    for first in (0, size["m"] // 2, size["m"] - 5000):
+        x, y = A.narrow(a.index("m"), first, 5000), C.narrow(c.index("m"), first, 5000)
+        ref = torch.einsum(spec, x.double(), B.double())
+        # positive terms: every order of summation is within k + 1 roundings
+        assert ((y.double() - ref).abs() / ref).max().item() <= (size["k"] + 1) * 6e-8
+    del A, B, C, x, y
+    torch.cuda.empty_cache()
