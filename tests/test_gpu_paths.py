@@ -315,3 +315,72 @@ def test_skinny_beyond_32bit_offsets(spec):
         assert ((y.double() - ref).abs() / ref).max().item() <= (size["k"] + 1) * 6e-8
     del A, B, C, x, y
     torch.cuda.empty_cache()
+
+
+def _contract(spec, size, A, B, C, prec):
+    (a, b), c = spec.split("->")[0].split(","), spec.split("->")[1]
+    letters = sorted(size)
+    tn.contract_dev([size[l] for l in letters], [letters.index(l) for l in a], A,
+                    [letters.index(l) for l in b], B, [letters.index(l) for l in c], C, prec=prec)
+
+
+# 256 x 256 tiles (more than 64 summed slabs, and half the rounds of 128 x 256
+# tiles): a last row tile with rows in its first half only and in both, a ragged
+# last 32-column chunk, row lengths with and without 16-byte stores, a K tail.
+# Whole numbers up to 3: products, and sums below 2^24, are exact
+@pytest.mark.parametrize("prec,k", [("tf32", 2100), ("bf16", 4150)])
+@pytest.mark.parametrize("m,n,g", [(3172, 2317, 1), (3272, 2348, 1), (3172, 1101, 2)])
+def test_tc_gemm_wide_tiles(prec, k, m, n, g):
+    spec = "mk,nk->mn" if g == 1 else "gmk,gkn->gmn"
+    (a, b), c = spec.split("->")[0].split(","), spec.split("->")[1]
+    size = dict(k=k, m=m, n=n) if g == 1 else dict(g=g, k=k, m=m, n=n)
+    gen = torch.Generator(device="cuda").manual_seed(m + n)
+    A, B = (torch.randint(0, 4, [size[l] for l in s], generator=gen, device="cuda").float()
+            for s in (a, b))
+    C = torch.full([size[l] for l in c], float("nan"), device="cuda")
+    _contract(spec, size, A, B, C, prec)
+    assert torch.equal(C.double(), torch.einsum(spec, A.double(), B.double()))
+
+
+# operands and results that start off 16-byte boundaries (views into a buffer):
+# copies and stores fall back to the widest their addresses allow
+@pytest.mark.parametrize("oa,ob,oc", [(1, 0, 0), (0, 1, 0), (0, 0, 1), (2, 2, 2), (3, 1, 2)])
+@pytest.mark.parametrize("spec,size", [
+    ("mk,nk->mn", dict(k=96, m=400, n=260)),            # GEMM form, in place when aligned
+    ("km,kn->nm", dict(k=96, m=400, n=260)),            # both operands and the result reordered
+    ("gmk,gkn->gmn", dict(g=2, k=72, m=130, n=1100)),
+    ("km,kn->nm", dict(k=24, m=2048, n=40)),            # batched GEMM: copies and stores of quads
+    ("mgk,kgn->ngm", dict(g=4, k=20, m=1000, n=64)),
+    ("mk,kn->mn", dict(k=12, m=3000, n=72))])
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "tf32", "bf16"])
+def test_contract_unaligned_pointers(spec, size, oa, ob, oc, prec):
+    (a, b), c = spec.split("->")[0].split(","), spec.split("->")[1]
+    dt = torch.float64 if prec == "fp64" else torch.float32
+    gen = torch.Generator(device="cuda").manual_seed(7)
+
+    def view(s, off):
+        shape = [size[l] for l in s]
+        n = int(np.prod(shape))
+        return torch.randint(0, 4, [n + off], generator=gen, device="cuda").to(dt)[off:].view(shape)
+    A, B, C = view(a, oa), view(b, ob), view(c, oc)
+    _contract(spec, size, A, B, C, prec)
+    # whole numbers: exact in every precision and order
+    assert torch.equal(C.double(), torch.einsum(spec, A.double(), B.double()))
+
+
+# FP64 GEMM form past the direct kernel's limits: 2^26 table entries (operands in
+# place) and 2^31 entries (prepared)
+@pytest.mark.parametrize("m", [(1 << 25) - 64, (1 << 25) + 3])
+def test_fp64_gemm_past_direct_limits(m):
+    k = n = 64
+    gen = torch.Generator(device="cuda").manual_seed(2)
+    A, B = (torch.rand(s, generator=gen, device="cuda", dtype=torch.float64)
+            for s in ((m, k), (n, k)))
+    C = torch.full((m, n), float("nan"), dtype=torch.float64, device="cuda")
+    _contract("mk,nk->mn", dict(k=k, m=m, n=n), A, B, C, "fp64")
+    for first in (0, m // 2, m - 5000):
+        ref = A[first:first + 5000] @ B.T
+        err = ((C[first:first + 5000] - ref).abs() / ref).max().item()
+        assert err <= k * 2.3e-16 + 1e-15      # positive terms, as above
+    del A, B, C, ref
+    torch.cuda.empty_cache()
