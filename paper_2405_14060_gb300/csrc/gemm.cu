@@ -9,13 +9,16 @@
 //                layout while recording its per-item maximum.
 //   k_tc_gemm    tcgen05 tensor-core GEMM: D = X Y^T per batch, X and Y
 //                K-major, TF32 (kind::tf32) or BF16 (kind::f16) inputs staged
-//                by TMA (128-byte swizzle) through a 4-stage mbarrier
-//                pipeline, FP32 accumulators in TMEM (two 128 x 256 buffers
-//                per CTA), epilogue through tcgen05.ld.  One thread issues
-//                TMA, one issues MMAs, four warps drain TMEM; persistent over
-//                tiles for short K, so that a tile's epilogue overlaps the
-//                next tile's MMAs.
-//   k_simt_gemm  CUDA-core tiled GEMM for FP32 and FP64.
+//                by TMA (128-byte swizzle) through an mbarrier ring, FP32
+//                accumulators in TMEM, epilogue through tcgen05.ld and shared
+//                memory.  One thread issues TMA, one issues MMAs, four warps
+//                drain TMEM.  128 x 256 tiles (ring of four slabs, two TMEM
+//                buffers), persistent for short K, so that a tile's epilogue
+//                overlaps the next tile's MMAs; 256 x 256 tiles (ring of
+//                three, one buffer of two accumulators) for long K.
+//   k_sgemm      FP32 GEMM on CUDA cores: four tile shapes, packed pairs.
+//   k_simt_gemm  FP64 GEMM on CUDA cores, for contractions past the index
+//                ranges of the direct kernel (bgemm.cu).
 //
 // Every mbarrier wait is bounded in time: a wait that exceeds ~2 s sets the
 // error flag and the CTA skips the rest of its work.  Before it frees its
@@ -964,10 +967,10 @@ cudaError_t launch_tc_gemm(const GDesc &g, int *err_flag, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// ------------------------------------------------------------- SIMT GEMM
+// ------------------------------------------------------- CUDA-core GEMMs
 
-template <typename T>
 __global__ void __launch_bounds__(256) k_simt_gemm(const __grid_constant__ GDesc g) {
+    using T = double;
     constexpr int BM = 64, BN = 64, BK = 16;
     __shared__ T sx[BK][BM + 1];
     __shared__ T sy[BK][BN + 1];
@@ -1204,7 +1207,7 @@ static int64_t sgemm_tiles(const GDesc &g) {
 void launch_simt_gemm(const GDesc &g, cudaStream_t st) {
     if (g.xtype == E_F64) {
         dim3 grid((unsigned)(((g.C + 63) / 64) * ((g.R + 63) / 64) * g.batch), 1, 1);
-        k_simt_gemm<double><<<grid, 256, 0, st>>>(g);
+        k_simt_gemm<<<grid, 256, 0, st>>>(g);
         return;
     }
     // the tile whose busiest SM has the least work: tiles per SM, rounded up,

@@ -105,13 +105,13 @@ __global__ void k_leaves(const LeafRec *recs, const double *tables, const int *c
 
 template <typename T>
 void launch_leaves(const LeafRec *recs, int nrec, int64_t largest, const double *tables,
-                   const int *card, int nvars, const int32_t *evid, int nbeta, int log_mode, T *base,
-                   unsigned long long *mx, const int *flags, const int32_t *slice_val,
+                   const int *card, int nvars, const int32_t *evid, int nbeta, int log_mode,
+                   T *base, unsigned long long *mx, const int *flags, const int32_t *slice_val,
                    cudaStream_t st) {
     if (nrec <= 0) return;
-    const int64_t parts = std::min<int64_t>((largest + 255) / 256, 256);
-    k_leaves<T><<<dim3((unsigned)nrec, (unsigned)std::max<int64_t>(1, parts)), 256, 0, st>>>(recs, tables, card, nvars, evid, nbeta, log_mode, base, mx,
-                                      flags, slice_val);
+    const int64_t parts = std::max<int64_t>(1, std::min<int64_t>((largest + 255) / 256, 256));
+    k_leaves<T><<<dim3((unsigned)nrec, (unsigned)parts), 256, 0, st>>>(
+        recs, tables, card, nvars, evid, nbeta, log_mode, base, mx, flags, slice_val);
 }
 
 // ------------------------------------------------------------ slicing
