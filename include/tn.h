@@ -367,7 +367,7 @@ const char *tn_last_error(void);
  * contraction kernels.  No rescaling is applied.  The call takes its scratch
  * memory (operand workspaces, tables, split-K partial sums) stream-ordered
  * from a memory pool of the library, which keeps at most 1 GiB a device
- * between calls, and synchronises `cuda_stream` before returning.
+ * between calls (and up to 64 MiB of a stream's last call), and synchronises `cuda_stream` before returning.
  */
 tn_status tn_contract_dev(int nlabels, const int *sizes,
                           int na, const int *labels_a, const void *A,
