@@ -361,19 +361,27 @@ struct tn_model {
     std::unique_ptr<MmapCache> mmap;
     double last_ms = 0;
     int64_t last_launches = 0;
-    ~tn_model() {
+    ~tn_model() { release_device(); }
+    // Give up everything that lives on the model's device.
+    void release_device() {
         progs.clear();
         mmap.reset();
         for (void *p : {(void *)d_sM, (void *)d_sS, (void *)d_sA, (void *)d_sl_var,
-                        (void *)d_sl_card, (void *)d_sl_tab, (void *)d_sl_moff})
+                        (void *)d_sl_card, (void *)d_sl_tab, (void *)d_sl_moff, (void *)d_tables,
+                        (void *)d_flags, (void *)d_err})
             if (p) cudaFree(p);
-        if (d_tables) cudaFree(d_tables);
-        if (d_flags) cudaFree(d_flags);
-        if (d_err) cudaFree(d_err);
+        d_sM = d_sS = d_sA = d_tables = nullptr;
+        s_cap_b = s_cap_m = 0;
+        d_sl_var = d_sl_card = d_sl_tab = nullptr;
+        d_sl_moff = nullptr;
+        d_flags = d_err = nullptr;
         if (ev0) cudaEventDestroy(ev0);
         if (ev1) cudaEventDestroy(ev1);
+        ev0 = ev1 = nullptr;
         for (auto l : lanes) cudaStreamDestroy(l);
+        lanes.clear();
         if (stream) cudaStreamDestroy(stream);
+        stream = nullptr;
     }
 };
 
@@ -2977,15 +2985,7 @@ tn_status ensure_device(tn_model *m) {
     CK(cudaGetDevice(&dev));
     if (m->device == dev && m->d_tables && !m->tables_overridden) return TN_OK;
     if (m->device != dev) {
-        m->progs.clear();
-        m->mmap.reset();
-        if (m->d_tables) cudaFree(m->d_tables);
-        m->d_tables = nullptr;
-        if (m->stream) cudaStreamDestroy(m->stream);
-        for (auto l : m->lanes) cudaStreamDestroy(l);
-        m->lanes.clear();
-        if (m->ev0) cudaEventDestroy(m->ev0);
-        if (m->ev1) cudaEventDestroy(m->ev1);
+        m->release_device();
         CK(cudaStreamCreateWithFlags(&m->stream, cudaStreamNonBlocking));
         CK(cudaEventCreate(&m->ev0));
         CK(cudaEventCreate(&m->ev1));
